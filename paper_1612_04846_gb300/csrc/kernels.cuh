@@ -78,6 +78,7 @@ struct OuterCfg {
     double c[KMAXP], d[KMAXP];  // weights and shifts
     double lambda_lo;           // lower bound on lambda_min(A); 0: relative residual thresholds
     double inner_rtol;          // largest residual reduction asked of one FP32 inner solve
+    double rtol_slack;          // inner_rtol^1e-9 (the margin of the refinement plan's step count)
     long long wait_cycles;      // TMA ring wait budget of the inner solves (0: default)
     int K, max_outer, max_iters;
 };
@@ -265,6 +266,51 @@ template <class T>
 cudaError_t fdiag_prepare(int nx, int ny, int nsys, int* G, size_t* smem);
 template <class T>
 cudaError_t fdiag_launch(const FdiagArgs& a, int G, size_t smem, int nsys, cudaStream_t s);
+
+// A whole mixed-precision solve of a small 2-D constant-coefficient plan in one launch (resident.cu): a
+// thread-block cluster per system runs the refinement and CG loops on vectors kept in shared memory.
+constexpr int kResMaxLevels = 8;
+constexpr int kResMaxOuter = 64;                 // refinement steps whose iteration counts a record holds
+constexpr size_t kResSmemMax = 230912;           // dynamic shared memory of a CTA (227 KB less the static arrays)
+constexpr size_t kResSmemHalf = 114176;          // ... of one of two CTAs that share an SM
+struct ResOut {                                  // a system's outcome
+    double rr, fnorm2;
+    int outer, siters, status;
+    int its[kResMaxOuter];                       // CG iterations of each refinement step
+};
+struct ResLevel {
+    int nx, ny;
+    float wx, wy;
+    const float *c1, *c2;                        // Chebyshev tables of the level, [step][Kp]
+    int oR, oX, oY, oD;                          // shared-memory offsets (floats)
+};
+struct ResArgs {
+    int le, ne;                                  // the exact level (the last one) and its rows
+    int re, ce;                                  // rows and columns of it per CTA
+    int G, threads;                              // CTAs per system, threads per CTA
+    int Kp;
+    size_t N;
+    double wx, wy;                               // level-0 weights in FP64
+    ResLevel lev[kResMaxLevels];
+    int o_sx, o_sy, o_lam, o_zero, o_p, o_r64, o_r64_end, o_d, o_vs, o_vh, o_bt, o_br, o_cc, o_cd, o_x, floats;
+    unsigned img_bytes;
+    const float* img;                            // sine bases and eigenvalues of the exact level (res_image)
+    const float* dsh;                            // shifts
+    const OuterCfg* cfg;
+    float* x;                                    // [system][row][nx rounded up to even] inner solutions, when shared memory has
+                                                 // no room for them (o_x < 0)
+    double* v;                                   // [system][N] solutions
+    ResOut* out;                                 // [system]
+};
+size_t res_image_floats(int nx, int ny);
+void res_image(int nx, int ny, const double* sx, const double* sy, const float* lx, const float* ly, float* img);
+// Chooses the cluster size and lays out the shared memory of a plan whose levels are filled in; false if the
+// plan does not fit.  Called at plan setup, outside any capture.
+bool resident_plan(ResArgs& a);
+cudaError_t launch_resident(const ResArgs& a, int K, const double* f, double tol, cudaStream_t s);
+// u = sum_j c_j v_j (or V: the systems) and the outcome into st (page-locked host memory)
+cudaError_t launch_resident_out(const ResArgs& a, int K, const double* c, double* u, double* V, int accumulate,
+                                OuterState* st, cudaStream_t s);
 
 // ------------------------------------------------------------------ host launchers
 template <class T>

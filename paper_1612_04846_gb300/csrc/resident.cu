@@ -1,0 +1,972 @@
+// A whole mixed-precision solve of a small 2-D constant-coefficient plan in one launch, with every vector of
+// the inner solver resident in shared memory.
+//
+// The shifted systems never exchange values, so each system gets a thread-block cluster of G CTAs of its own
+// that runs the refinement loop, the multigrid-preconditioned CG inside it and all their decisions: the
+// formulas are those of the grid kernels (kernels_tma.cu, fdiag.cu), of the reductions (kernels_impl.cuh) and
+// of the controller (outer.cu), point by point; only the grouping of the dot products' sums differs.
+//
+// Why: on grids of up to about 10^5 points the graph of grid kernels is bound by its own launches.  A 383 x 255,
+// k = 8 solve is 108 launches in 812 us, 7.5 us each, for about 1 us of work each.  Here a vector is read from
+// and written to shared memory, and a phase ends in an exchange of its edge rows.
+//
+// Layout: CTA g owns a slab of grid rows on every level: rows [a, b) of the exact level le and, on a level s
+// levels above it, rows [a 2^s, b 2^s) (the last slab also the rows above (ny_le) 2^s), so that a coarse row and
+// the fine rows 2J, 2J + 1 it sits on have one owner.  A vector is rows of ld floats (zero columns on either
+// side, column 0 on an 8-byte boundary: a thread takes pairs of columns, with packed FP32 arithmetic) with halo
+// rows: R (right-hand side, 3), X (pre-smoothed iterate, 2), Y (scratch, 1), D (direction and result, 2), and on
+// level 0 the CG direction P (1).  With these halos the way down a level (both pre-smoothing steps, residual,
+// restriction) and the way up (prolongation, both post-smoothing steps) need no other slab's values: halo rows
+// are recomputed.
+//
+// Exchanges: what a phase produces is also stored into the halo rows of the slabs around it with st.async, which
+// counts its bytes on an mbarrier of the receiver; a phase waits for the bytes of its own halo rows only (about
+// 500 SM clocks less per exchange than a cluster barrier behind ordinary remote stores: 690 against 1196 measured
+// with 16 CTAs of 512 threads).  Every (buffer, level) has an mbarrier of its own, used once per CG iteration;
+// the reductions alternate between two.  A sender is never two uses ahead of a receiver: between two uses of a
+// barrier lies a reduction, which needs every CTA's contribution.  For the same reason a halo row is only
+// written when its last readers are done.  Every wait is bounded.
+//
+// The exact solve of level le is fdiag.cu's fast diagonalization, every sum in the same order.
+//
+// Measured (GB300, one solve, tol 1e-6, graph of kernels -> here): 63^2, k = 5: 168 -> 45 us; 127^2, k = 6: 372 -> 100;
+// 255^2, k = 7: 550 -> 201; 383 x 255, k = 8: 812 -> 280.  What is left is latency: a 127^2 iteration is 9.5 us, of
+// which the exact solve's four products and three exchanges take 3.6.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+#include "kernels_impl.cuh"
+#include "tma.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace bura {
+
+namespace {
+
+constexpr int kResMostWarps = 16;
+constexpr int kHR = 3, kHX = 2, kHY = 1, kHD = 2, kHP = 1;  // halo rows of R, X, Y, D, P
+constexpr int kSP = 64;                                     // leading dimension of the sine bases
+constexpr int kStrip = 4;                                   // most rows a thread takes at a time
+
+// An unevaluated sum h + l of two FP32 values (about 48 bits).  GB300's FP64 pipe takes a warp instruction in
+// 16 SM clocks, so a scalar FP64 step that all 16 warps execute costs 256: the CG's sums and scalars run on the
+// FP32 pipe in pairs instead (a reduction over 16 CTAs of 512 threads: 3700 -> 2000 clocks).
+struct Df {
+    float h, l;
+};
+__device__ __forceinline__ Df df_add(Df a, Df b) {
+    const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
+    const float e = __fadd_rn(__fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t)), __fadd_rn(a.l, b.l));
+    const float h = __fadd_rn(s, e);
+    return {h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ Df df_add(Df a, float b) { return df_add(a, Df{b, 0.f}); }
+// a / b rounded to FP32 from a pair quotient (about 45 bits)
+__device__ __forceinline__ float df_div(Df a, Df b) {
+    const float q = __fdiv_rn(a.h, b.h);
+    const float r = __fadd_rn(__fmaf_rn(-q, b.h, a.h), __fmaf_rn(-q, b.l, a.l));
+    return __fadd_rn(q, __fdiv_rn(r, b.h));
+}
+__device__ __forceinline__ Df df_shfl_xor(Df v, int o) {
+    return {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
+}
+
+__device__ __forceinline__ unsigned map_rank(const void* p, int rank) {
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+// Asynchronous stores into CTA `rank`'s copy of *p, counted on its copy of *bar.
+__device__ __forceinline__ void put(float* p, int rank, uint64_t* bar, float v) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(map_rank(p, rank)),
+                 "f"(v), "r"(map_rank(bar, rank))
+                 : "memory");
+}
+__device__ __forceinline__ void put2(void* p, int rank, uint64_t* bar, float v0, float v1) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(
+                     map_rank(p, rank)),
+                 "f"(v0), "f"(v1), "r"(map_rank(bar, rank))
+                 : "memory");
+}
+// Wait for a phase whose bytes other CTAs of the cluster store; false after the default budget.
+__device__ __forceinline__ bool wait_bytes(uint64_t* bar, unsigned parity) {
+    const long long t0 = clock64();
+    for (;;) {
+        unsigned ok;
+        asm volatile(
+            "{\n"
+            ".reg .pred p;\n"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+            "selp.u32 %0, 1, 0, p;\n"
+            "}\n"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        if (clock64() - t0 > kTmaWaitCycles) return false;
+    }
+}
+__device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ void st2(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
+
+// Rows [y0, y1) of a level with ny rows, sh levels above the exact level (ne rows, re rows per slab), that
+// slab t owns (empty for a slab past the last row).
+__device__ __forceinline__ void slab(int t, int re, int ne, int sh, int ny, int& y0, int& y1) {
+    const int a = min(t * re, ne), b = min(a + re, ne);
+    y0 = a < ne ? a << sh : ny;
+    y1 = b < ne ? b << sh : ny;
+}
+
+__host__ __device__ constexpr int even(int v) { return (v + 1) / 2 * 2; }
+// Floats per row: two in front of column 0 and at least one zero column after the last.
+__host__ __device__ constexpr int row_floats(int nx) { return 2 + even(nx + 1); }
+
+struct Slab {
+    int y0, y1;  // own rows
+    int nx, ny, ld;
+    __device__ __forceinline__ bool some() const { return y1 > y0; }
+    // bytes of the rows that fill this slab's H halo rows
+    __device__ __forceinline__ unsigned halo_bytes(int H) const {
+        return some() ? (unsigned)((min(H, y0) + min(H, ny - y1)) * even(nx) * 4) : 0u;
+    }
+};
+
+// A x at the column pair c of a row (u above, w below, l and r the values beside the pair), diag = 2 wx + 2 wy: the
+// grid kernels' order of multiply-adds.
+__device__ __forceinline__ float2 stencil2(float wx, float wy, float diag, float2 c, float l, float r, float2 u, float2 w) {
+    float2 t = __fmul2_rn(dup(diag), c);
+    t.x = fmaf(-wx, l, t.x);
+    t.y = fmaf(-wx, c.x, t.y);
+    t.x = fmaf(-wx, c.y, t.x);
+    t.y = fmaf(-wx, r, t.y);
+    t = __ffma2_rn(dup(-wy), u, t);
+    return __ffma2_rn(dup(-wy), w, t);
+}
+
+// How a level's row sweeps are split over the warps: items of h rows x 64 columns, h the number (up to kStrip) whose
+// rounds of items take the fewest row steps, for the own rows (kind 0) and with 1, 2 and 4 rows more (1, 2, 3).
+template <int kResWarps>
+struct Split {
+    int nch, q, m;  // column chunks; a warp's next item lies q rows of items and m chunks on
+    int h[4];
+    unsigned char s[kResWarps], ch[kResWarps];  // a warp's first item
+};
+
+template <int kResWarps>
+struct Ctx {
+    const ResArgs* a;
+    float* sm;
+    int g, G, warp, lane;
+    // the pair v at (y, x) of level l's buffer `ofs` with H halo rows, stored into the other slabs whose halo rows
+    // include y
+    __device__ __forceinline__ void share(int l, int ofs, int H, const Slab& s, uint64_t* bar, int y, int x, float2 v) const {
+        if (y < s.y0 + H)
+            for (int t = g - 1; t >= 0; --t) {
+                int u0, u1;
+                slab(t, a->re, a->ne, a->le - l, s.ny, u0, u1);
+                if (y >= u1 + H) break;
+                put2(sm + ofs + (y - u0 + H) * s.ld + x + 2, t, bar, v.x, v.y);
+            }
+        if (y >= s.y1 - H)
+            for (int t = g + 1; t < G; ++t) {
+                int u0, u1;
+                slab(t, a->re, a->ne, a->le - l, s.ny, u0, u1);
+                if (u0 >= s.ny || y < u0 - H) break;
+                put2(sm + ofs + (y - u0 + H) * s.ld + x + 2, t, bar, v.x, v.y);
+            }
+    }
+    // f(first row, rows, first column of a pair) over rows [r0, r1) of a level whose work is split as in sp: a warp takes
+    // 64 columns of up to h = sp.h[kind] rows at a time
+    template <class F>
+    __device__ __forceinline__ void strips(const Split<kResWarps>& sp, int kind, int r0, int r1, int nx, F&& f) const {
+        const int h = sp.h[kind], nch = sp.nch, m = sp.m;
+        int ch = sp.ch[warp];
+        for (int y = r0 + sp.s[warp] * h; y < r1;) {
+            const int x = (ch << 6) + 2 * lane;
+            if (x < nx) f(y, min(h, r1 - y), x);
+            ch += m;
+            y += sp.q * h;
+            if (ch >= nch) { ch -= nch; y += h; }
+        }
+    }
+};
+
+}  // namespace
+
+template <int kResThreads>
+__global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(const __grid_constant__ ResArgs a, const double* f, double tol) {
+    constexpr int kResWarps = kResThreads / 32;
+    extern __shared__ __align__(16) float rsm[];
+    float* const sm = rsm;
+    __shared__ double slots[2][16];      // a reduction's partial sums of every CTA (FP64, or Df pairs)
+    __shared__ double wsum[kResWarps];
+    __shared__ double bc[6];             // FP64 scalars that one warp computes for all
+    __shared__ Split<kResWarps> split[kResMaxLevels];
+    __shared__ float coef[kResMaxLevels][3];  // c2 of the first Chebyshev step, c1 and c2 of the second
+    __shared__ int late_in[16];          // each CTA's copy timed out
+    __shared__ __align__(8) uint64_t bimg, bR[kResMaxLevels], bD[kResMaxLevels], bC, bB, bV, bS[2];
+    cg::cluster_group cl = cg::this_cluster();
+    const int tid = threadIdx.x;
+    const int G = (int)cl.num_blocks(), g = (int)cl.block_rank();
+    const int sys = blockIdx.x / G;
+    Ctx<kResWarps> cx{&a, sm, g, G, tid >> 5, tid & 31};
+    const int le = a.le;
+    const float d = a.dsh[sys];
+    bool late = false;
+    if (tid == 0) {
+        mbar_init(&bimg, 1);
+        for (int l = 0; l <= le; ++l) {
+            mbar_init(&bR[l], 1);
+            mbar_init(&bD[l], 1);
+        }
+        mbar_init(&bC, 1);
+        mbar_init(&bB, 1);
+        mbar_init(&bV, 1);
+        mbar_init(&bS[0], 1);
+        mbar_init(&bS[1], 1);
+        mbar_fence_init();
+        const long long w = a.cfg->wait_cycles;
+        mbar_expect_tx(&bimg, a.img_bytes);
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(smem_u32(sm + a.o_sx)), "l"(a.img), "r"(a.img_bytes), "r"(smem_u32(&bimg))
+                     : "memory");
+        // a wait budget of the caller's starts at the copy's issue; the default one after the buffers are cleared
+        if (w > 0) late = !mbar_wait_bounded(&bimg, 0, w);
+    }
+    __syncthreads();
+    if (tid < 4 * (le + 1)) {  // thread (level, kind)
+        const int l = tid >> 2, k = tid & 3, nch = (a.lev[l].nx + 63) >> 6;
+        int y0, y1;
+        slab(g, a.re, a.ne, le - l, a.lev[l].ny, y0, y1);
+        const int rows = y1 - y0 + (k == 3 ? 4 : k);
+        int h = 1, best = 1 << 30;
+        for (int q = 1; q <= kStrip; ++q) {
+            const int cost = (((rows + q - 1) / q) * nch + kResWarps - 1) / kResWarps * (q + 1);
+            if (cost < best) { best = cost; h = q; }
+        }
+        Split<kResWarps>& sp = split[l];
+        sp.h[k] = h;
+        for (int w = k; w < kResWarps; w += 4) {
+            sp.s[w] = (unsigned char)(w / nch);
+            sp.ch[w] = (unsigned char)(w % nch);
+        }
+        if (k == 0) {
+            sp.nch = nch;
+            sp.q = kResWarps / nch;
+            sp.m = kResWarps % nch;
+        }
+        if (l < le && k < 3) coef[l][k] = k == 0 ? a.lev[l].c2[sys] : k == 1 ? a.lev[l].c1[a.Kp + sys] : a.lev[l].c2[a.Kp + sys];
+    }
+    // everything but the bases starts at zero: the zero columns and the rows outside the grid stay zero
+    for (int i = a.o_zero / 4 + tid; i < a.floats / 4; i += kResThreads)
+        reinterpret_cast<float4*>(sm)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!mbar_wait_bounded(&bimg, 0, kTmaWaitCycles)) late = true;  // (a late copy lands before the kernel goes on)
+    int faulted = __syncthreads_or(late);
+    cl.sync();  // every CTA runs and has cleared its buffers and barriers before the first remote store
+
+    unsigned uR = 0, uD = 0, uC = 0, uB = 0, uV = 0, uS = 0;  // the parity of each barrier's next phase
+    bool lost = false;  // a wait of this thread ran out
+    int gone = 0;       // ... of this CTA, as of its last reduction
+    // arm (thread 0) and await one phase; local values of the phase are published by the caller's barrier
+    auto arm = [&](uint64_t* bar, unsigned bytes) {
+        if (tid == 0) mbar_expect_tx(bar, bytes);
+    };
+    auto await = [&](uint64_t* bar, unsigned& bits, int at) {
+        if (!lost && !wait_bytes(bar, (bits >> at) & 1u)) lost = true;
+        bits ^= 1u << at;
+    };
+    auto range = [&](int l) {
+        Slab s;
+        slab(g, a.re, a.ne, le - l, a.lev[l].ny, s.y0, s.y1);
+        s.nx = a.lev[l].nx;
+        s.ny = a.lev[l].ny;
+        s.ld = row_floats(s.nx);
+        return s;
+    };
+    // (y, x) of a buffer at base + y * ld + x
+    auto at = [&](int ofs, int H, const Slab& s) { return sm + ofs + (H - s.y0) * s.ld + 2; };
+    int flip = 0;
+    // the sum over the cluster of every thread's v, the same bits in every thread
+    auto all_sum = [&](Df v) {
+        arm(&bS[flip], 8u * G);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v = df_add(v, df_shfl_xor(v, o));
+        Df* const ws = reinterpret_cast<Df*>(wsum);
+        if (cx.lane == 0) ws[cx.warp] = v;
+        gone = __syncthreads_or(lost);
+        if (cx.warp == 0) {
+            Df t = ws[cx.lane & (kResWarps - 1)];
+#pragma unroll
+            for (int o = kResWarps / 2; o > 0; o >>= 1) t = df_add(t, df_shfl_xor(t, o));
+            if (cx.lane < G) put2(&slots[flip][g], cx.lane, &bS[flip], t.h, t.l);
+        }
+        await(&bS[flip], uS, flip);
+        Df t = reinterpret_cast<Df*>(slots[flip])[cx.lane & 15];
+        if ((cx.lane & 15) >= G) t = Df{0.f, 0.f};
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) t = df_add(t, df_shfl_xor(t, o));
+        flip ^= 1;
+        return t;
+    };
+    // the same in FP64 (norms of the refinement): warp 0 adds the partials; the sum is returned in warp 0 only.
+    // `extra` more bytes are due on the barrier.
+    auto all_sum64 = [&](double v, unsigned extra) {
+        arm(&bS[flip], 8u * G + extra);
+        double* const pd = reinterpret_cast<double*>(sm + a.o_d);
+        pd[tid] = v;
+        gone = __syncthreads_or(lost);
+        if (cx.warp == 0) {
+            double t = 0.0;
+#pragma unroll
+            for (int k = 0; k < kResWarps; k += 4)
+                t += (pd[k * 32 + cx.lane] + pd[(k + 1) * 32 + cx.lane]) + (pd[(k + 2) * 32 + cx.lane] + pd[(k + 3) * 32 + cx.lane]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (cx.lane < G)
+                put2(&slots[flip][g], cx.lane, &bS[flip], __int_as_float(__double2loint(t)), __int_as_float(__double2hiint(t)));
+        }
+        await(&bS[flip], uS, flip);
+        double t = 0.0;
+        if (cx.warp == 0) {
+            t = cx.lane < G ? slots[flip][cx.lane] : 0.0;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            t = __shfl_sync(0xffffffffu, t, 0);
+        }
+        flip ^= 1;
+        return t;
+    };
+
+    const Slab s0 = range(0);
+    const int np = (s0.y1 - s0.y0) * s0.nx;  // own points of level 0, numbered along the rows
+    const int ld0 = s0.ld, ldx = even(s0.nx);
+    float* const R0 = at(a.lev[0].oR, kHR, s0);
+    float* const P0 = at(a.o_p, kHP, s0);
+    double* const r64 = reinterpret_cast<double*>(sm + a.o_r64);     // own points (over P, X, Y, D: free between inner solves)
+    double* const vg = a.v + (size_t)sys * a.N;
+    double* const vs = reinterpret_cast<double*>(sm + a.o_vs);       // v of the own points for the residual
+    double* const vh = reinterpret_cast<double*>(sm + a.o_vh);       // v on the rows below and above the slab
+    // x of the own points, rows of ldx
+    float* const xs = (a.o_x >= 0 ? sm + a.o_x : a.x + ((size_t)sys * s0.ny + s0.y0) * ldx) - (size_t)s0.y0 * ldx;
+    const size_t gofs = (size_t)s0.y0 * s0.nx;
+
+    if (cx.warp == kResWarps - 1) {
+        // this system's relative threshold need_j, reached in n_j = ceil(log need_j / log inner_rtol - 1e-9) steps of
+        // need_j^(1/n_j) each; n_j by comparing with the powers of inner_rtol (rtol_slack = inner_rtol^1e-9)
+        const OuterCfg& c = *a.cfg;
+        const double t = c.lambda_lo > 0 ? tol * (c.lambda_lo - c.d[sys]) / (c.K * c.c[sys]) : tol;
+        double st2 = 1.0;  // the square of a step's share
+        if (t < 1.0) {
+            double r = c.inner_rtol;
+            int n = 1;
+            for (; t < r * c.rtol_slack && r > 0.0; ++n) r *= c.inner_rtol;
+            st2 = n == 1 ? t * t : n == 2 ? t : pow(t, 2.0 / n);
+        }
+        if (cx.lane == 0) {
+            bc[5] = t;
+            bc[2] = 0.25 * st2;
+        }
+    }
+    // ||f||^2
+    double part = 0.0;
+    for (int i = tid; i < np; i += kResThreads) {
+        const double v = __ldg(f + gofs + i);
+        part = fma(v, v, part);
+    }
+    if (tid < G) put(reinterpret_cast<float*>(&late_in[g]), tid, &bS[0], __int_as_float(faulted));
+    const double sum_f = all_sum64(part, 4u * G);
+    for (int t = 0; t < G; ++t) faulted |= late_in[t];
+    if (tid == 0) {
+        bc[0] = sum_f;
+        bc[1] = bc[5] * bc[5] * sum_f;
+    }
+    __syncthreads();
+    const double fn2 = bc[0], thr64 = bc[1];
+    const int max_outer = a.cfg->max_outer, max_iters = a.cfg->max_iters;
+
+    // ---- pieces of the V-cycle
+    // way down level l: x2 (both pre-smoothing steps from zero) on the own rows and two halo rows, the residual
+    // in Y on the fine rows the slab restricts, its full weighting into R of level l + 1
+    auto down = [&](int l) {
+        const ResLevel& L = a.lev[l];
+        const Slab s = range(l), sc = range(l + 1);
+        const int ld = s.ld, nx = s.nx;
+        const float wx = L.wx, wy = L.wy, diag = wx + wx + wy + wy;
+        const float c20 = coef[l][0], c1 = coef[l][1], c2 = coef[l][2];
+        const bool more = l + 1 < le;  // the exact level reads its own rows only
+        if (more) arm(&bR[l + 1], sc.halo_bytes(kHR));
+        if (s.some()) {
+            const float* R = at(L.oR, kHR, s);
+            float* X = at(L.oX, kHX, s);
+            cx.strips(split[l], 3, max(0, s.y0 - 2), min(s.ny, s.y1 + 2), nx, [&](int y, int n, int x) {
+                const float* q = R + y * ld + x;
+                float* o = X + y * ld + x;
+                const bool last = x + 1 >= nx;
+                float2 b = ld2(q), c = __fmul2_rn(dup(c20), b), u = __fmul2_rn(dup(c20), ld2(q - ld));
+                for (int i = 0; i < n; ++i, q += ld, o += ld) {
+                    const float2 bn = ld2(q + ld), w = __fmul2_rn(dup(c20), bn);
+                    const float2 t = stencil2(wx, wy, diag, c, c20 * q[-1], c20 * q[2], u, w);
+                    const float2 tt = __ffma2_rn(dup(-d), c, t);
+                    const float2 res = make_float2(b.x - tt.x, b.y - tt.y);
+                    float2 v = __fadd2_rn(c, __ffma2_rn(dup(c1), c, __fmul2_rn(dup(c2), res)));
+                    if (last) v.y = 0.f;
+                    st2(o, v);
+                    u = c; c = w; b = bn;
+                }
+            });
+        }
+        __syncthreads();
+        if (s.some()) {
+            const float *R = at(L.oR, kHR, s), *X = at(L.oX, kHX, s);
+            float* Y = at(L.oY, kHY, s);
+            cx.strips(split[l], 1, s.y0, min(s.ny, s.y1 + 1), nx, [&](int y, int n, int x) {
+                const float* q = X + y * ld + x;
+                const float* rb = R + y * ld + x;
+                float* o = Y + y * ld + x;
+                float2 u = ld2(q - ld), c = ld2(q);
+                for (int i = 0; i < n; ++i, q += ld, rb += ld, o += ld) {
+                    const float2 w = ld2(q + ld);
+                    const float2 t = __ffma2_rn(dup(-d), c, stencil2(wx, wy, diag, c, q[-1], q[2], u, w));
+                    const float2 b = ld2(rb);
+                    st2(o, make_float2(b.x - t.x, b.y - t.y));
+                    u = c; c = w;
+                }
+            });
+        }
+        __syncthreads();
+        if (sc.some()) {
+            const float* Y = at(L.oY, kHY, s);
+            const int oRc = a.lev[l + 1].oR;
+            float* Rc = at(oRc, kHR, sc);
+            cx.strips(split[l + 1], 0, sc.y0, sc.y1, sc.nx, [&](int J, int n, int I) {
+                const float* q = Y + 2 * J * ld + 2 * I;
+                const bool last = I + 1 >= sc.nx;
+                for (int i = 0; i < n; ++i, ++J, q += 2 * ld) {
+                    float2 t = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {  // columns 2I .. 2I + 4 of rows 2J .. 2J + 2
+                        const float2 p = ld2(q + k * ld), m = ld2(q + k * ld + 2);
+                        const float e = q[k * ld + 4];
+                        const float w0 = k == 1 ? 0.125f : 0.0625f, w1 = k == 1 ? 0.25f : 0.125f;
+                        t.x = fmaf(w0, m.x, fmaf(w1, p.y, fmaf(w0, p.x, t.x)));
+                        t.y = fmaf(w0, e, fmaf(w1, m.y, fmaf(w0, m.x, t.y)));
+                    }
+                    if (last) t.y = 0.f;
+                    st2(Rc + J * sc.ld + I, t);
+                    if (more) cx.share(l + 1, oRc, kHR, sc, &bR[l + 1], J, I, t);
+                }
+            });
+        }
+        __syncthreads();
+        if (more) await(&bR[l + 1], uR, l + 1);
+    };
+    // way up level l: x2 + P (result of level l + 1) on two halo rows, the first post-smoothing step on one, the
+    // second on the own rows into D; returns this thread's part of r.z
+    auto up = [&](int l) {
+        const ResLevel& L = a.lev[l];
+        const Slab s = range(l), sc = range(l + 1);
+        const int ld = s.ld, ldc = sc.ld, nx = s.nx;
+        const float wx = L.wx, wy = L.wy, diag = wx + wx + wy + wy;
+        const float c20 = coef[l][0], c1 = coef[l][1], c2 = coef[l][2];
+        const float* R = at(L.oR, kHR, s);
+        float *X = at(L.oX, kHX, s), *Y = at(L.oY, kHY, s), *D = at(L.oD, kHD, s);
+        const float* E = at(a.lev[l + 1].oD, kHD, sc);
+        Df tot{0.f, 0.f};
+        arm(&bD[l], s.halo_bytes(kHD));
+        if (s.some()) {
+            cx.strips(split[l], 3, max(0, s.y0 - 2), min(s.ny, s.y1 + 2), nx, [&](int y, int n, int x) {
+                const bool last = x + 1 >= nx;
+                float* o = X + y * ld + x;
+                for (int i = 0; i < n; ++i, ++y, o += ld) {
+                    // column x reads coarse columns x/2 - 1 and x/2, column x + 1 reads x/2
+                    const float* e = E + ((y & 1) ? y >> 1 : (y >> 1) - 1) * ldc + (x >> 1);
+                    const float e0 = e[-1], e1 = e[0];
+                    float2 t;
+                    if (y & 1) {
+                        t.x = fmaf(0.5f, e1, 0.5f * e0);
+                        t.y = e1;
+                    } else {
+                        const float f0 = e[ldc - 1], f1 = e[ldc];
+                        t.x = fmaf(0.25f, f1, fmaf(0.25f, f0, fmaf(0.25f, e1, 0.25f * e0)));
+                        t.y = fmaf(0.5f, f1, 0.5f * e1);
+                    }
+                    if (last) t.y = 0.f;
+                    st2(o, __fadd2_rn(ld2(o), t));
+                }
+            });
+        }
+        __syncthreads();
+        if (s.some()) {
+            cx.strips(split[l], 2, max(0, s.y0 - 1), min(s.ny, s.y1 + 1), nx, [&](int y, int n, int x) {
+                const bool last = x + 1 >= nx;
+                const int k = y * ld + x;
+                const float *q = X + k, *rb = R + k;
+                float *oy = Y + k, *od = D + k;
+                float2 u = ld2(q - ld), c = ld2(q);
+                for (int i = 0; i < n; ++i, q += ld, rb += ld, oy += ld, od += ld) {
+                    const float2 w = ld2(q + ld), b = ld2(rb);
+                    const float2 t = __ffma2_rn(dup(-d), c, stencil2(wx, wy, diag, c, q[-1], q[2], u, w));
+                    float2 dv = __fmul2_rn(dup(c20), make_float2(b.x - t.x, b.y - t.y));
+                    if (last) dv.y = 0.f;
+                    st2(oy, __fadd2_rn(c, dv));
+                    if (y + i >= s.y0 && y + i < s.y1) st2(od, dv);
+                    u = c; c = w;
+                }
+            });
+        }
+        __syncthreads();
+        if (s.some()) {
+            cx.strips(split[l], 0, s.y0, s.y1, nx, [&](int y, int n, int x) {
+                const bool last = x + 1 >= nx;
+                const int k = y * ld + x;
+                const float *q = Y + k, *rb = R + k;
+                float* od = D + k;
+                float2 u = ld2(q - ld), c = ld2(q), p2 = make_float2(0.f, 0.f);
+                for (int i = 0; i < n; ++i, q += ld, rb += ld, od += ld) {
+                    const float2 w = ld2(q + ld), b = ld2(rb);
+                    const float2 t = __ffma2_rn(dup(-d), c, stencil2(wx, wy, diag, c, q[-1], q[2], u, w));
+                    const float2 res = make_float2(b.x - t.x, b.y - t.y);
+                    float2 z = __fadd2_rn(c, __ffma2_rn(dup(c1), ld2(od), __fmul2_rn(dup(c2), res)));
+                    if (last) z.y = 0.f;
+                    st2(od, z);
+                    cx.share(l, L.oD, kHD, s, &bD[l], y + i, x, z);
+                    p2 = __ffma2_rn(b, z, p2);
+                    u = c; c = w;
+                }
+                tot = df_add(tot, p2.x + p2.y);
+            });
+        }
+        __syncthreads();
+        await(&bD[l], uD, l);
+        return tot;
+    };
+    // out[q][m] = sum_k S[k][m] C[q][k] (k in increasing order) for m < M, q < Q, handed to epi(q, value) by a thread with
+    // tid mod kSP = m; C has rows of kSP floats, zero from Kd on (so that k may run on to a multiple of 4: the bases are
+    // followed by finite values).  A thread takes two q, so a value of S is loaded once for both; a warp shares them, so
+    // its loads of C are broadcasts of four at a time.
+    const int m = tid & (kSP - 1);
+    const int own_c = m / a.ce, own_r = m / a.re;  // the slabs that own column and row m of the exact level
+    auto product = [&](const float* S, const float* C, int Kd, int M, int Q, auto&& epi) {
+        if (m >= M) return;
+        const float* Sm = S + m;
+        for (int q = 2 * (tid / kSP); q < Q; q += 2 * (kResThreads / kSP)) {
+            const bool two = q + 1 < Q;
+            const float4 *A4 = reinterpret_cast<const float4*>(C + q * kSP), *B4 = A4 + (two ? kSP / 4 : 0);
+            float v = 0.f, w = 0.f;
+#pragma unroll 4
+            for (int k = 0; k < Kd; k += 4) {
+                const float4 c = A4[k >> 2], e = B4[k >> 2];
+                const float s0 = Sm[k * kSP], s1 = Sm[(k + 1) * kSP], s2 = Sm[(k + 2) * kSP], s3 = Sm[(k + 3) * kSP];
+                v = fmaf(s0, c.x, v);
+                w = fmaf(s0, e.x, w);
+                v = fmaf(s1, c.y, v);
+                w = fmaf(s1, e.y, w);
+                v = fmaf(s2, c.z, v);
+                w = fmaf(s2, e.z, w);
+                v = fmaf(s3, c.w, v);
+                w = fmaf(s3, e.w, w);
+            }
+            epi(q, v);
+            if (two) epi(q + 1, w);
+        }
+    };
+    // exact solve of level le: D = (A - d I)^{-1} R there; returns this thread's part of R.D (the CG r.z when le = 0)
+    auto exact = [&]() {
+        const ResLevel& L = a.lev[le];
+        const Slab s = range(le);
+        const int ld = s.ld, nx = s.nx, ny = s.ny, rows = s.y1 - s.y0;
+        const float* R = at(L.oR, kHR, s);
+        float* D = at(L.oD, kHD, s);
+        const float *SX = sm + a.o_sx, *SY = sm + a.o_sy;
+        float *Bt = sm + a.o_bt, *Br = sm + a.o_br, *Cc = sm + a.o_cc, *Cd = sm + a.o_cd;
+        const int c0 = min(nx, g * a.ce), cw = min(nx, c0 + a.ce) - c0;
+        arm(&bC, 4u * ny * cw);
+        arm(&bB, 4u * rows * nx);
+        arm(&bD[le], s.halo_bytes(kHD));
+        for (int i = tid; i < rows * kSP; i += kResThreads) {
+            const int r = i / kSP, k = i & (kSP - 1);
+            Bt[i] = k < nx ? R[(s.y0 + r) * ld + k] : 0.f;
+        }
+        __syncthreads();
+        // rows of R S_x, each value to the slab that owns its column
+        product(SX, Bt, nx, nx, rows, [&](int r, float v) {
+            put(Cc + (m - own_c * a.ce) * kSP + s.y0 + r, own_c, &bC, v);
+        });
+        await(&bC, uC, 0);
+        product(SY, Cc, ny, ny, cw, [&](int c, float v) {
+            Cd[c * kSP + m] = v / ((sm[a.o_lam + c0 + c] + sm[a.o_lam + kSP + m]) - d);
+        });
+        __syncthreads();
+        product(SY, Cd, ny, ny, cw, [&](int c, float v) {
+            put(Br + (m - own_r * a.re) * kSP + c0 + c, own_r, &bB, v);
+        });
+        await(&bB, uB, 0);
+        Df tot{0.f, 0.f};
+        product(SX, Br, nx, nx, rows, [&](int r, float v) {
+            const int y = s.y0 + r;
+            D[y * ld + m] = v;
+            tot = df_add(tot, v * R[y * ld + m]);
+        });
+        __syncthreads();
+        if (s.some())  // the edge rows, in pairs
+            for (int i = tid; i < rows * (kSP / 2); i += kResThreads) {
+                const int r = i / (kSP / 2), x = 2 * (i & (kSP / 2 - 1));
+                if (x < nx && (r < kHD || r >= rows - kHD)) cx.share(le, L.oD, kHD, s, &bD[le], s.y0 + r, x, ld2(D + (s.y0 + r) * ld + x));
+            }
+        await(&bD[le], uD, le);
+        return tot;
+    };
+
+    // ---- the refinement loop
+    const double c0_64 = 2.0 * (a.wx + a.wy) - a.cfg->d[sys];
+    double rr64 = fn2;  // uniform: every decision below is taken alike by all threads of the cluster
+    int outer = 0, siters = 0, status = -5;
+    if (faulted) status = -6;
+    ResOut& out = a.out[sys];
+    const ResLevel& L0 = a.lev[0];
+    for (; !faulted;) {
+        if (!isfinite(rr64)) { status = -4; break; }
+        if (!(rr64 > thr64)) { status = 0; break; }
+        if (outer >= max_outer) break;
+        // the scale, its reciprocal and the inner target on ||r||^2 (a step's share or what is left, with a margin of 2), by
+        // a warp each: FP64 roots and divisions are long chains on GB300
+        if (cx.warp == 0) {
+            const double h = sqrt(rr64);
+            if (cx.lane == 0) bc[3] = h;
+        } else if (cx.warp == 1) {
+            const double h = rsqrt(rr64);
+            if (cx.lane == 0) bc[4] = h;
+        } else if (cx.warp == 2) {
+            const double t = fmax(bc[2], 0.25 * (thr64 / rr64));
+            if (cx.lane == 0) bc[5] = t;
+        }
+        arm(&bR[0], s0.halo_bytes(kHR));
+        __syncthreads();
+        const double hs = bc[3], is = bc[4];
+        const Df thr{(float)bc[5], (float)(bc[5] - (double)(float)bc[5])};
+        // the inner right-hand side r / ||r|| in FP32, with its halo rows
+        if (s0.some())
+            cx.strips(split[0], 0, s0.y0, s0.y1, s0.nx, [&](int y, int n, int x) {
+                const bool last = x + 1 >= s0.nx;
+                for (int i = 0; i < n; ++i, ++y) {
+                    const int k = (y - s0.y0) * s0.nx + x;
+                    const double* src = outer == 0 ? f + gofs : r64;
+                    float2 v;
+                    v.x = (float)(src[k] * is);
+                    v.y = last ? 0.f : (float)(src[k + 1] * is);
+                    st2(R0 + y * ld0 + x, v);
+                    cx.share(0, L0.oR, kHR, s0, &bR[0], y, x, v);
+                }
+            });
+        // P, X, Y, D held the FP64 residual and the norm's partials: their zero columns and rows are restored
+        __syncthreads();
+        for (int i = a.o_r64 / 4 + tid; i < a.o_r64_end / 4; i += kResThreads)
+            reinterpret_cast<float4*>(sm)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        __syncthreads();
+        await(&bR[0], uR, 0);
+        Df rz{1.f, 0.f};
+        int it = 0, breakdown = 0;
+        for (;;) {
+            // z = M r into D
+            Df t;
+            for (int l = 0; l < le; ++l) down(l);
+            t = exact();
+            for (int l = le - 1; l >= 0; --l) t = up(l);
+            const Df rzn = all_sum(t);
+            if (!isfinite(rzn.h)) breakdown = 1;
+            const float beta = df_div(rzn, rz);
+            rz = rzn;
+            // p = z + beta p on the own rows and one halo row, q = (A - d I) p into Y
+            const float* Z = at(L0.oD, kHD, s0);
+            float* Q = at(L0.oY, kHY, s0);
+            if (s0.some())
+                cx.strips(split[0], 2, max(0, s0.y0 - 1), min(s0.ny, s0.y1 + 1), s0.nx, [&](int y, int n, int x) {
+                    const int k = y * ld0 + x;
+                    const float* z = Z + k;
+                    float* o = P0 + k;
+                    for (int i = 0; i < n; ++i, z += ld0, o += ld0)
+                        st2(o, it == 0 ? ld2(z) : __ffma2_rn(dup(beta), ld2(o), ld2(z)));
+                });
+            __syncthreads();
+            t = Df{0.f, 0.f};
+            if (s0.some()) {
+                const float wx = L0.wx, wy = L0.wy, diag = wx + wx + wy + wy;
+                cx.strips(split[0], 0, s0.y0, s0.y1, s0.nx, [&](int y, int n, int x) {
+                    const int k = y * ld0 + x;
+                    const float* q = P0 + k;
+                    float* o = Q + k;
+                    float2 u = ld2(q - ld0), c = ld2(q), p2 = make_float2(0.f, 0.f);
+                    for (int i = 0; i < n; ++i, q += ld0, o += ld0) {
+                        const float2 w = ld2(q + ld0);
+                        const float2 v = __ffma2_rn(dup(-d), c, stencil2(wx, wy, diag, c, q[-1], q[2], u, w));
+                        st2(o, v);
+                        p2 = __ffma2_rn(c, v, p2);  // c is zero in the padding column
+                        u = c; c = w;
+                    }
+                    t = df_add(t, p2.x + p2.y);
+                });
+            }
+            const Df pq = all_sum(t);
+            float af = 0.f;
+            if (!(pq.h > 0.f) || !isfinite(pq.h)) breakdown = 1;
+            else af = df_div(rz, pq);
+            // x += alpha p, r -= alpha q with the halo rows of r
+            arm(&bR[0], s0.halo_bytes(kHR));
+            t = Df{0.f, 0.f};
+            if (s0.some())
+                cx.strips(split[0], 0, s0.y0, s0.y1, s0.nx, [&](int y, int n, int x) {
+                    const bool last = x + 1 >= s0.nx;
+                    const int k = y * ld0 + x;
+                    const float *p = P0 + k, *q = Q + k;
+                    float *r = R0 + k, *xp = xs + y * ldx + x;
+                    float2 p2 = make_float2(0.f, 0.f);
+                    for (int i = 0; i < n; ++i, p += ld0, q += ld0, r += ld0, xp += ldx) {
+                        const float2 pv = ld2(p);
+                        st2(xp, it == 0 ? __fmul2_rn(dup(af), pv) : __ffma2_rn(dup(af), pv, ld2(xp)));
+                        float2 rv = __ffma2_rn(dup(-af), ld2(q), ld2(r));
+                        if (last) rv.y = 0.f;
+                        st2(r, rv);
+                        cx.share(0, L0.oR, kHR, s0, &bR[0], y + i, x, rv);
+                        p2 = __ffma2_rn(rv, rv, p2);
+                    }
+                    t = df_add(t, p2.x + p2.y);
+                });
+            const Df rr = all_sum(t);
+            await(&bR[0], uR, 0);
+            ++it;
+            ++siters;
+            if (!isfinite(rr.h)) breakdown = 1;
+            if (rr.h < thr.h || (rr.h == thr.h && rr.l <= thr.l) || breakdown || it >= max_iters || gone) break;
+        }
+        if (tid == 0 && g == 0) out.its[outer] = it;
+        ++outer;
+        if (gone) { status = -6; break; }
+        if (breakdown) { status = -4; break; }
+        // v += ||r|| x, its edge rows into the neighbours' vh, then the true residual f - (A - d I) v and its norm, in FP64
+        arm(&bV, s0.some() ? (unsigned)((s0.y0 > 0) + (s0.y1 < s0.ny)) * s0.nx * 8u : 0u);
+        __syncthreads();
+        for (int i = tid; i < np; i += kResThreads) {
+            const int r = i / s0.nx, x = i - r * s0.nx;
+            const double xv = (double)xs[(s0.y0 + r) * ldx + x];
+            const double v = outer == 1 ? hs * xv : fma(hs, xv, vg[gofs + i]);
+            vg[gofs + i] = v;
+            vs[i] = v;
+            if (r == 0 && s0.y0 > 0) put2(vh + s0.nx + x, g - 1, &bV, __int_as_float(__double2loint(v)), __int_as_float(__double2hiint(v)));
+            if (r == s0.y1 - s0.y0 - 1 && s0.y1 < s0.ny)
+                put2(vh + x, g + 1, &bV, __int_as_float(__double2loint(v)), __int_as_float(__double2hiint(v)));
+        }
+        __syncthreads();
+        await(&bV, uV, 0);
+        double t = 0.0;
+        for (int i = tid; i < np; i += kResThreads) {
+            const int r = i / s0.nx, x = i - r * s0.nx, y = s0.y0 + r;
+            const double* q = vs + i;
+            const double sx = (x > 0 ? q[-1] : 0.0) + (x < s0.nx - 1 ? q[1] : 0.0);
+            const double lo = y == 0 ? 0.0 : r == 0 ? vh[x] : q[-s0.nx];
+            const double hi = y == s0.ny - 1 ? 0.0 : y == s0.y1 - 1 ? vh[s0.nx + x] : q[s0.nx];
+            double v = fma(-c0_64, q[0], __ldg(f + gofs + i));
+            v = fma(a.wx, sx, v);
+            v = fma(a.wy, lo + hi, v);
+            r64[i] = v;
+            t = fma(v, v, t);
+        }
+        t = all_sum64(t, 0u);
+        if (tid == 0) bc[0] = t;
+        __syncthreads();
+        rr64 = bc[0];
+    }
+    if (outer == 0)
+        for (int i = tid; i < np; i += kResThreads) vg[gofs + i] = 0.0;
+    if (tid == 0 && g == 0) {
+        out.rr = rr64;
+        out.fnorm2 = fn2;
+        out.outer = outer;
+        out.siters = siters;
+    }
+    if (tid == 0 && g == 0) out.status = status;
+    cl.sync();  // no CTA leaves while another may still store into its shared memory
+    if (tid == 0 && gone) out.status = -6;
+}
+
+// The output stage: u = sum_j c_j v_j (FP64, j = 0..K-1 in order) or the systems themselves into V, and the solve's
+// outcome from the systems' records (page-locked host memory): the counts of the lockstep solve, in which a
+// refinement step lasts as long as its slowest system.
+__global__ void k_resident_out(ResArgs a, int K, const double* c, double* u, double* V, int accumulate, OuterState* st) {
+    pdl_wait();
+    const size_t N = a.N;
+    if (blockIdx.x == 0 && threadIdx.x < 32) {  // lane j: system j
+        const int j = threadIdx.x;
+        const bool on = j < K;
+        const ResOut& o = a.out[on ? j : 0];
+        const int mine = o.outer;
+        int rank = o.status == -6 ? 3 : o.status == -4 ? 2 : o.status == -5 ? 1 : 0, outer = mine;
+        for (int w = 16; w > 0; w >>= 1) {
+            rank = max(rank, __shfl_xor_sync(0xffffffffu, rank, w));
+            outer = max(outer, __shfl_xor_sync(0xffffffffu, outer, w));
+        }
+        int total = 0;
+        for (int q = 0; q < outer; ++q) {
+            int m = q < mine ? o.its[q] : 0;
+            for (int w = 16; w > 0; w >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, w));
+            total += m;
+        }
+        if (on) {
+            st->siters[j] = o.siters;
+            st->rr[j] = o.rr;
+        }
+        if (j == 0) {
+            st->fnorm2 = o.fnorm2;
+            st->outer = outer;
+            st->total_it = total;
+            st->status = rank == 3 ? -6 : rank == 2 ? -4 : rank == 1 ? -5 : 0;
+            st->done = 1;
+        }
+    }
+    for (size_t P = blockIdx.x * (size_t)blockDim.x + threadIdx.x; P < N; P += (size_t)gridDim.x * blockDim.x) {
+        double s = 0.0;
+        for (int j = 0; j < K; ++j) {
+            const double v = a.v[j * N + P];
+            if (V) V[j * N + P] = v;
+            s = fma(c[j], v, s);
+        }
+        if (u) u[P] = accumulate ? u[P] + s : s;
+    }
+}
+
+namespace {
+
+int up4(int v) { return (v + 3) / 4 * 4; }
+
+// Shared-memory layout of one CTA for clusters of G; false if it does not fit (or has no rows to give a CTA).
+bool res_layout(ResArgs& a, int G) {
+    a.re = (a.ne + G - 1) / G;
+    a.ce = (a.lev[a.le].nx + G - 1) / G;
+    const int nxe = a.lev[a.le].nx;
+    const int last = a.ne - a.re * ((a.ne + a.re - 1) / a.re - 1);  // rows of the exact level in the last slab
+    long long own0 = 0;
+    int o = 0;
+    auto take = [&](long long n) {
+        const int at = o;
+        o = (int)std::min<long long>(1 << 28, up4((int)std::min<long long>(1 << 28, o + n)));
+        return at;
+    };
+    a.o_sx = take((long long)nxe * kSP);
+    a.o_sy = take((long long)a.ne * kSP);
+    a.o_lam = take(2 * kSP);
+    a.img_bytes = (unsigned)(res_image_floats(nxe, a.ne) * sizeof(float));
+    a.o_zero = o;
+    for (int l = 0; l <= a.le; ++l) {
+        ResLevel& L = a.lev[l];
+        const int ld = row_floats(L.nx);
+        const int sh = a.le - l;
+        const int tail = ((last << sh) + (1 << sh) - 1);  // the last slab's rows
+        const int most = std::min(std::max(a.re << sh, tail), L.ny);
+        L.oR = take((long long)(most + 2 * kHR) * ld);
+        if (l == 0) {
+            a.o_r64 = o;
+            a.o_p = take((long long)(most + 2 * kHP) * ld);
+        }
+        L.oX = l < a.le ? take((long long)(most + 2 * kHX) * ld) : o;
+        L.oY = l < a.le || l == 0 ? take((long long)(most + 2 * kHY) * ld) : o;
+        L.oD = take((long long)(most + 2 * kHD) * ld);
+        if (l == 0) {  // between inner solves: the FP64 residual, v with its neighbours' edge rows, the partials of a norm
+            own0 = (long long)most * even(L.nx);
+            const int end = o;
+            o = a.o_r64;
+            take(2 * own0);
+            a.o_vs = take(2 * own0);
+            a.o_vh = take(4 * L.nx);
+            a.o_d = take(2 * 32 * kResMostWarps);
+            a.o_r64_end = o = std::max(o, end);
+        }
+    }
+    a.o_bt = take((long long)a.re * kSP);
+    a.o_br = take((long long)a.re * kSP);
+    a.o_cc = take((long long)a.ce * kSP);
+    a.o_cd = take((long long)a.ce * kSP);
+    a.floats = o;
+    a.o_x = -1;
+    const size_t room = (size_t)o * sizeof(float) <= kResSmemHalf ? kResSmemHalf : kResSmemMax;
+    if ((size_t)(o + own0) * sizeof(float) <= room) {
+        a.o_x = take(own0);
+        a.floats = o;
+    }
+    return (size_t)a.floats * sizeof(float) <= kResSmemMax;
+}
+
+using ResKernel = void (*)(const ResArgs, const double*, double);
+ResKernel res_kernel(const ResArgs& a) { return a.threads == 256 ? k_resident<256> : k_resident<512>; }
+
+// The limits are properties of the function: always the largest, whatever a plan takes.
+cudaError_t res_attributes(ResKernel k) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemMax);
+}
+
+cudaLaunchConfig_t res_config(const ResArgs& a, int blocks, cudaLaunchAttribute* attr, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(a.threads);
+    cfg.dynamicSmemBytes = (size_t)a.floats * sizeof(float);
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = a.G;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+}  // namespace
+
+size_t res_image_floats(int nx, int ny) { return (size_t)(nx + ny + 2) * kSP; }
+
+void res_image(int nx, int ny, const double* sx, const double* sy, const float* lx, const float* ly, float* img) {
+    std::fill(img, img + res_image_floats(nx, ny), 0.f);
+    for (int i = 0; i < nx; ++i)
+        for (int k = 0; k < nx; ++k) img[(size_t)i * kSP + k] = (float)sx[(size_t)i * nx + k];
+    for (int i = 0; i < ny; ++i)
+        for (int k = 0; k < ny; ++k) img[(size_t)(nx + i) * kSP + k] = (float)sy[(size_t)i * ny + k];
+    std::copy(lx, lx + nx, img + (size_t)(nx + ny) * kSP);
+    std::copy(ly, ly + ny, img + (size_t)(nx + ny + 1) * kSP);
+}
+
+// The largest cluster of up to 16 CTAs (the device holds 7 clusters of 16 at one CTA per SM; more systems than that
+// run as the first clusters finish: 255^2 with 13 systems 989 -> 420 us).  Slabs small enough for two CTAs per SM
+// take 256 threads each, so that 14 clusters are resident (63^2, k = 9: 80 us with 512 threads, 49 with 256; 32
+// problems of up to 127^2 as one batch: 1772 and 993 us); larger ones take 512 (255^2, k = 5: 173 us, 189 with 256).
+bool resident_plan(ResArgs& a) {
+    for (int G = 16; G >= 1; G /= 2) {
+        if (G > a.ne || G > a.lev[a.le].nx) continue;
+        if (!res_layout(a, G)) return false;
+        a.G = G;
+        a.threads = (size_t)a.floats * sizeof(float) <= kResSmemHalf ? 256 : 512;
+        if (res_attributes(res_kernel(a)) != cudaSuccess) { cudaGetLastError(); return false; }
+        cudaLaunchAttribute attr[1];
+        cudaLaunchConfig_t cfg = res_config(a, G, attr, nullptr);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, res_kernel(a), &cfg) != cudaSuccess) { cudaGetLastError(); continue; }
+        if (n >= 1) return true;
+    }
+    return false;
+}
+
+cudaError_t launch_resident(const ResArgs& a, int K, const double* f, double tol, cudaStream_t s) {
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = res_config(a, K * a.G, attr, s);
+    return cudaLaunchKernelEx(&cfg, res_kernel(a), a, f, tol);
+}
+
+cudaError_t launch_resident_out(const ResArgs& a, int K, const double* c, double* u, double* V, int accumulate,
+                                OuterState* st, cudaStream_t s) {
+    const long long b = ((long long)a.N + 255) / 256;
+    launch_pdl(k_resident_out, dim3((unsigned)std::min<long long>(b, 152 * 8)), dim3(256), 0, s, a, K, c, u, V, accumulate, st);
+    return cudaGetLastError();
+}
+
+}  // namespace bura

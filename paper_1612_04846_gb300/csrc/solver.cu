@@ -212,6 +212,8 @@ struct bura_plan {
     cudaGraph_t sgraph = nullptr;
     cudaGraphExec_t sexec = nullptr;
     long long s_fixed = 0, s_outer = 0, s_body = 0;  // launches: once, per refinement step, per PCG iteration
+    bool res_on = false;         // the whole solve is one launch (resident.cu)
+    ResArgs res{};
     bool pending = false;        // a device-driven solve's outcome has not been read into st yet
     int last_status = BURA_OK;   // status of the last solve whose outcome was read
     bura_stats st{};
@@ -599,26 +601,33 @@ double smoother_ratio(const bura_plan* p) {
 // sine basis S_ik = sqrt(2/(n+1)) sin(pi (i+1)(k+1)/(n+1)) and the eigenvalues w (2 - 2 cos(pi (k+1)/(n+1)))
 // = 4 w sin^2(pi (k+1) / (2 (n+1))) of w tridiag(-1, 2, -1), in FP64, rounded to T.
 template <class T>
+void sine_axis(const HostLevel& h, int a, std::vector<double>& S, std::vector<T>& lam) {
+    const int n = h.n[a];
+    const double pi = 3.14159265358979323846;
+    const double sc = std::sqrt(2.0 / (n + 1));
+    S.resize((size_t)n * n);
+    for (int i = 0; i < n; ++i)
+        for (int k = 0; k < n; ++k) {
+            // (i+1)(k+1) reduced modulo 2 (n+1): the same angle, with no large argument
+            const long long m = (long long)(i + 1) * (k + 1) % (2LL * (n + 1));
+            S[(size_t)i * n + k] = sc * std::sin(pi * (double)m / (n + 1));
+        }
+    lam.resize(n);
+    for (int k = 0; k < n; ++k) {
+        const double sk = std::sin(pi * (k + 1) / (2.0 * (n + 1)));
+        lam[k] = (T)(4.0 * h.w[a] * sk * sk);
+    }
+}
+
+template <class T>
 int upload_fdiag(bura_plan* p, Work<T>& w) {
     const HostLevel& h = p->hl[w.lc];
     std::vector<double> S[2];
     T** dst_l[2] = {&w.fd_lx, &w.fd_ly};
     for (int a = 0; a < 2; ++a) {
         const int n = h.n[a];
-        const double pi = 3.14159265358979323846;
-        const double sc = std::sqrt(2.0 / (n + 1));
-        S[a].resize((size_t)n * n);
-        for (int i = 0; i < n; ++i)
-            for (int k = 0; k < n; ++k) {
-                // (i+1)(k+1) reduced modulo 2 (n+1): the same angle, with no large argument
-                const long long m = (long long)(i + 1) * (k + 1) % (2LL * (n + 1));
-                S[a][(size_t)i * n + k] = sc * std::sin(pi * (double)m / (n + 1));
-            }
-        std::vector<T> lam(n);
-        for (int k = 0; k < n; ++k) {
-            const double sk = std::sin(pi * (k + 1) / (2.0 * (n + 1)));
-            lam[k] = (T)(4.0 * h.w[a] * sk * sk);
-        }
+        std::vector<T> lam;
+        sine_axis<T>(h, a, S[a], lam);
         CA(dalloc(p, dst_l[a], (size_t)n * sizeof(T)));
         CK(cudaMemcpy(*dst_l[a], lam.data(), lam.size() * sizeof(T), cudaMemcpyHostToDevice));
     }
@@ -875,6 +884,56 @@ int build_work(bura_plan* p, Work<T>& w, bool full = true) {
     if (sizeof(T) == 4 && p->dim == 2 && !p->var && w.Kp <= 16) CK(strip_prepare(w.Kp));
     if (sizeof(T) == 4 && p->dim == 3 && w.Kp <= 16) CK(cheb3s_prepare(w.Kp, p->var));
     w.ready = true;
+    return BURA_OK;
+}
+
+// The one-launch solve: 2-D constant coefficients in mixed precision with FP64 refinement and the default
+// smoothing, whose hierarchy ends in the fast-diagonalization level and whose slabs fit the shared memory of a
+// cluster.  Options that ask for particular sweeps keep the graph of kernels.  It keeps its solutions in the
+// plan's v64 buffer, system by system.
+int build_resident(bura_plan* p) {
+    const bura_options& o = p->opt;
+    Work<float>& w = p->w32;
+    if (o.precision != BURA_PREC_MIXED || o.refine != BURA_REFINE_FP64 || p->dim != 2 || p->var) return BURA_OK;
+    if (w.coarse_kind != BURA_COARSE_FDIAG || w.lc < 0 || w.lc >= kResMaxLevels) return BURA_OK;
+    if ((w.lc > 0 && o.smoother_degree != 2) || o.sweeps != BURA_SWEEP_AUTO || o.post_smooth_split != 0 || o.tma_stages != 0 ||
+        o.max_outer > kResMaxOuter)
+        return BURA_OK;
+    ResArgs& a = p->res;
+    a.le = w.lc;
+    a.ne = p->hl[w.lc].n[1];
+    a.Kp = w.Kp;
+    a.N = (size_t)p->hl[0].N;
+    a.wx = p->hl[0].w[0];
+    a.wy = p->hl[0].w[1];
+    for (int l = 0; l <= w.lc; ++l) {
+        ResLevel& L = a.lev[l];
+        L.nx = p->hl[l].n[0];
+        L.ny = p->hl[l].n[1];
+        L.wx = (float)p->hl[l].w[0];
+        L.wy = (float)p->hl[l].w[1];
+        L.c1 = w.c1[l];
+        L.c2 = w.c2[l];
+    }
+    if (!resident_plan(a)) return BURA_OK;
+    const int nx = p->hl[w.lc].n[0], ny = p->hl[w.lc].n[1];
+    std::vector<double> S[2];
+    std::vector<float> lam[2];
+    for (int q = 0; q < 2; ++q) sine_axis<float>(p->hl[w.lc], q, S[q], lam[q]);
+    std::vector<float> img(res_image_floats(nx, ny));
+    res_image(nx, ny, S[0].data(), S[1].data(), lam[0].data(), lam[1].data(), img.data());
+    float* di = nullptr;
+    CA(dalloc(p, &di, img.size() * sizeof(float)));
+    CK(cudaMemcpy(di, img.data(), img.size() * sizeof(float), cudaMemcpyHostToDevice));
+    CA(dalloc(p, &a.out, (size_t)p->K * sizeof(ResOut)));
+    a.img = di;
+    a.dsh = w.dsh;
+    a.cfg = p->ocfg;
+    a.x = nullptr;
+    if (a.o_x < 0)
+        CA(dalloc(p, &a.x, (size_t)p->K * p->hl[0].n[1] * ((p->hl[0].n[0] + 1) / 2 * 2) * sizeof(float)));
+    a.v = p->v64;
+    p->res_on = true;
     return BURA_OK;
 }
 
@@ -1681,6 +1740,7 @@ int upload_outer(bura_plan* p) {
         }
         oc.lambda_lo = p->lambda_lo;
         oc.inner_rtol = p->opt.inner_rtol;
+        oc.rtol_slack = std::pow(p->opt.inner_rtol, 1e-9);
         oc.wait_cycles = p->wait_cycles;
         oc.K = p->K;
         oc.max_outer = p->opt.max_outer;
@@ -1914,7 +1974,7 @@ int read_outcome(bura_plan* p) {
     double rr[KMAXP] = {0};
     for (int j = 0; j < p->K; ++j) rr[j] = o.rr[j];
     finish_stats(p, rr, o.fnorm2);
-    p->st.launches = 2 + p->s_fixed + (long long)o.outer * p->s_outer + (long long)o.total_it * p->s_body;
+    p->st.launches = p->res_on ? 2 : 2 + p->s_fixed + (long long)o.outer * p->s_outer + (long long)o.total_it * p->s_body;
     p->last_status = o.status;
     return o.status;
 }
@@ -2063,6 +2123,7 @@ int setup_device(bura_plan* p, long long N, bura_plan** out) {
     if (cudaMallocHost(&p->hstate, sizeof(OuterState)) != cudaSuccess) { p->hstate = nullptr; return fail(BURA_ENOMEM); }
     std::memset(p->hstate, 0, sizeof(OuterState));
     if ((rc = upload_outer(p)) != BURA_OK) return fail(rc);
+    if ((rc = build_resident(p)) != BURA_OK) return fail(rc);
     if (cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming) != cudaSuccess) {
         p->done = nullptr;
         return fail(BURA_ECUDA);
@@ -2342,6 +2403,13 @@ namespace {
 int enqueue_device_solve(bura_plan* p, const double* f, double* u, double* V, double tol, cudaStream_t s, int accumulate) {
     if (!(tol > 0)) return BURA_EINVAL;
     CK(cudaSetDevice(p->dev));
+    if (p->res_on) {
+        CK(launch_resident(p->res, p->K, f, tol, s));
+        CK(launch_resident_out(p->res, p->K, p->cdev, u, V, accumulate, p->hstate, s));
+        CK(cudaEventRecord(p->done, s));
+        p->pending = true;
+        return BURA_OK;
+    }
     CA(solve_device(p, f, tol, s));
     const long long N = p->hl[0].N;
     if (V) launch_gather_systems(N, p->w64.Kp, p->K, solution_vectors(p), V, s);
@@ -2542,6 +2610,13 @@ int build_batch(bura_batch* b, const double* const* f, double* const* u, double 
         const bool was_on = p->tr.on;
         const long long before = p->tr.launches;
         p->tr.on = false;
+        if (p->res_on) {
+            e = launch_resident(p->res, p->K, f[i], tol, s);
+            if (e == cudaSuccess) e = launch_resident_out(p->res, p->K, p->cdev, u[i], nullptr, 0, p->hstate, s);
+            p->tr.on = was_on;
+            if (e != cudaSuccess) { g_last = e; rc = BURA_ECUDA; }
+            continue;
+        }
         launch_solve_params(p->ostate, f[i], tol, s);
         rc = capture_solve_top(p, s, tasks);
         p->tr.on = was_on;
