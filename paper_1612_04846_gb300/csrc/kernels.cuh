@@ -223,24 +223,13 @@ cudaError_t launch_post2_strip(const StripGeo& g, int nsm, const float* x, const
                                ChebStepT<float> cs0, ChebStepT<float> cs1, const float* dsh, const Red& red,
                                cudaStream_t s);
 
-// The 3-D FP32 Chebyshev step with its inputs staged plane by plane in a shared-memory ring (sweep3d.cu);
-// face weights in FP32 (not bf16).  cheb3s_prepare sets the kernel's shared-memory limit (plan setup).
-#ifndef BURA_CHEB3S
-#define BURA_CHEB3S 1
+// The 3-D FP32 sweeps staged plane by plane in shared memory (sweep3d.cu) run on levels at least this wide (else the
+// z-marching grid sweeps): with 63 instead of 127 a 63^3 variable-coefficient solve (k = 5) takes 3.42 ms instead of 3.93.
+#ifndef BURA_SWEEP3_MIN_N
+#define BURA_SWEEP3_MIN_N 63
 #endif
-#ifndef BURA_CHEB3S_MIN_N
-#define BURA_CHEB3S_MIN_N 127
-#endif
-constexpr bool kCheb3s = BURA_CHEB3S != 0;     // 3-D Chebyshev steps of levels >= kCheb3sMinN wide staged
-constexpr int kCheb3sMinN = BURA_CHEB3S_MIN_N;  // in shared memory (else the z-marching grid sweep)
-size_t cheb3s_smem_bytes(int Kp, bool var);
-cudaError_t cheb3s_prepare(int Kp, bool var);
-cudaError_t launch_cheb_step3s(const Lev& L, int Kp, bool var, int nsm, const float* xin, const float* din,
-                               const float* b, float* xout, float* dout, ChebStepT<float> cs, const float* dsh,
-                               const Red& red, cudaStream_t s);
-// r = b - (A - d_j I) x with the same staging
-cudaError_t launch_residual3s(const Lev& L, int Kp, bool var, int nsm, const float* x, const float* b, float* r,
-                              const float* dsh, cudaStream_t s);
+constexpr int kSweep3MinN = BURA_SWEEP3_MIN_N;
+cudaError_t sweep3_prepare(int Kp, bool var);  // the kernels' shared-memory limits (plan setup)
 
 // Exact coarsest-level solve of a 2-D constant-coefficient operator by fast diagonalization (fdiag.cu):
 // one thread-block cluster of G CTAs per shifted system; every array holds element type T.

@@ -894,8 +894,9 @@ TmaGeo tma_geo(const Lev& L, const Lev* Lc, int Kp) {
     return g;
 }
 
-cudaError_t tma_encode(CUtensorMap* m, const float* base, int Kp, int nx, int ny, int boxkind) {
-    // resolved once per process (a thread-safe static initialisation: plans may be set up concurrently)
+// cuTensorMapEncodeTiled, resolved once per process (a thread-safe static initialisation: plans may be set up
+// concurrently); null if the driver has none.
+static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     static const PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
         void* fn = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -903,6 +904,24 @@ cudaError_t tma_encode(CUtensorMap* m, const float* base, int Kp, int nx, int ny
         return (e == cudaSuccess && q == cudaDriverEntryPointSuccess) ? reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn)
                                                                         : nullptr;
     }();
+    return encode;
+}
+
+cudaError_t tma_encode3(CUtensorMap* m, const void* base, long long row, int ny, int nz, int bx, int by) {
+    const PFN_cuTensorMapEncodeTiled_v12000 encode = encode_fn();
+    if (!encode) return cudaErrorNotSupported;
+    const cuuint64_t dims[3] = {(cuuint64_t)row, (cuuint64_t)ny, (cuuint64_t)nz};
+    const cuuint64_t strides[2] = {(cuuint64_t)row * 8, (cuuint64_t)row * 8 * ny};
+    const cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    const CUresult r = encode(m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, const_cast<void*>(base), dims, strides, box, estr,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+cudaError_t tma_encode(CUtensorMap* m, const float* base, int Kp, int nx, int ny, int boxkind) {
+    const PFN_cuTensorMapEncodeTiled_v12000 encode = encode_fn();
     if (!encode) return cudaErrorNotSupported;
     int bx = 0, by = 0;
     tma_box_dims(boxkind, &bx, &by);

@@ -130,6 +130,18 @@ struct Work {
         }
     };
     std::vector<TmaLev> tma;
+    // TMA-staged sweeps of the large 3-D levels (FP32): geometry and the maps of the level's vectors by box
+    struct S3Lev {
+        bool on = false;
+        Sweep3Lev geo{};
+        std::vector<typename TmaLev::Ent> maps;
+        const CUtensorMap& at(int box, const void* buf) const {
+            for (const auto& e : maps)
+                if (e.box == box && e.buf == buf) return e.map;
+            return maps[0].map;  // (every pair that a sweep asks for is in the list)
+        }
+    };
+    std::vector<S3Lev> s3;
     bool ready = false;
     // the PCG loop captured once as a graph with a device-side conditional WHILE node
     cudaGraph_t graph = nullptr;
@@ -726,6 +738,92 @@ int upload_faces(bura_plan* p, const HostLevel& h, Lev& L, bool bf16) {
     return BURA_OK;
 }
 
+// The packed weights of a variable-coefficient level for the staged 3-D sweeps: a float4 per point of the grid extended
+// by one point along each axis (the faces below the point along x, y and z, and the diagonal summed from the stored
+// weights as upload_faces does; zero where a face or a point does not exist), and its maps.
+int upload_packed(bura_plan* p, const HostLevel& h, Sweep3Lev& g) {
+    const int nx = h.n[0], ny = h.n[1], nz = h.n[2];
+    std::vector<float> v((size_t)(nx + 1) * (ny + 1) * (nz + 1) * 4, 0.f);
+    for (int l = 0; l <= nz; ++l)
+        for (int j = 0; j <= ny; ++j) {
+            float* o = &v[((size_t)l * (ny + 1) + j) * (nx + 1) * 4];
+            const double* ax = h.a[0].data() + ((size_t)l * ny + j) * (nx + 1);  // read where the face exists only
+            const double* ay = h.a[1].data() + ((size_t)l * (ny + 1) + j) * nx;
+            const double* az = h.a[2].data() + ((size_t)l * ny + j) * nx;
+            const size_t up = (size_t)ny * nx;
+            for (int i = 0; i <= nx; ++i, o += 4) {
+                const bool in = i < nx && j < ny && l < nz;
+                if (j < ny && l < nz) o[0] = (float)(ax[i] * h.w[0]);
+                if (i < nx && l < nz) o[1] = (float)(ay[i] * h.w[1]);
+                if (i < nx && j < ny) o[2] = (float)(az[i] * h.w[2]);
+                if (in) {
+                    double s = (double)o[0] + (double)(float)(ax[i + 1] * h.w[0]);
+                    s += (double)o[1] + (double)(float)(ay[i + nx] * h.w[1]);
+                    s += (double)o[2] + (double)(float)(az[i + up] * h.w[2]);
+                    o[3] = (float)s;
+                }
+            }
+        }
+    float* d = nullptr;
+    CA(dalloc(p, &d, v.size() * sizeof(float)));
+    CK(cudaMemcpy(d, v.data(), v.size() * sizeof(float), cudaMemcpyHostToDevice));
+    for (int q = 0; q < 2; ++q) {
+        int bx = 0, by = 0;
+        sweep3_box(q ? S3B_RHALO : S3B_HALO, &bx, &by);
+        CK(tma_encode3(q ? &g.wr : &g.w, d, (long long)(nx + 1) * 2, ny + 1, nz + 1, bx * 2, by));
+    }
+    return BURA_OK;
+}
+
+// Whether level l of an FP32 work set runs the staged 3-D sweeps (kSweep3MinN points along x, half that along the other
+// axes: below, an item's fill of its ring costs more than the sweep saves), and its maps.  The buffers exist.
+template <class T>
+int build_sweep3(bura_plan* p, Work<T>& w, int l) {
+    const int nlev = (int)p->hl.size();
+    const HostLevel& h = p->hl[l];
+    auto& t = w.s3[l];
+    if (sizeof(T) != 4 || p->dim != 3 || (p->var && p->opt.smoother_bf16) || w.Kp > 16 || l + 1 >= nlev || w.deg[l] < 2 ||
+        h.n[0] < kSweep3MinN || std::min(h.n[1], h.n[2]) < kSweep3MinN / 2)
+        return BURA_OK;
+    const HostLevel& hc = p->hl[l + 1];
+    Sweep3Lev& g = t.geo;
+    g.nx = h.n[0]; g.ny = h.n[1]; g.nz = h.n[2];
+    g.ncx = hc.n[0]; g.ncy = hc.n[1]; g.ncz = hc.n[2];
+    g.Kp = w.Kp;
+    g.nsm = p->nsm;
+    g.var = p->var;
+    g.wx = (float)h.w[0]; g.wy = (float)h.w[1]; g.wz = (float)h.w[2];
+    const void* bl = l == 0 ? (const void*)w.r : (const void*)w.b[l];
+    struct Want { int box; const void* buf; int lev; };
+    std::vector<Want> want = {{S3B_HALO, bl, l}, {S3B_TILE, bl, l}, {S3B_RTILE, bl, l}, {S3B_TILE, w.dd[l], l},
+                              {S3B_COARSE, w.xa[l + 1], l + 1}, {S3B_COARSE, w.xb[l + 1], l + 1}};
+    for (const void* x : {(const void*)w.xa[l], (const void*)w.xb[l]}) {
+        want.push_back({S3B_HALO, x, l});
+        want.push_back({S3B_RHALO, x, l});
+    }
+    if (l == 0) {
+        want.push_back({S3B_HALO, w.pa, 0});
+        want.push_back({S3B_HALO, w.pb, 0});
+    }
+    for (const Want& e : want) {
+        typename Work<T>::TmaLev::Ent ent;
+        ent.box = e.box;
+        ent.buf = e.buf;
+        int bx = 0, by = 0;
+        sweep3_box(e.box, &bx, &by);
+        const HostLevel& q = p->hl[e.lev];
+        if (tma_encode3(&ent.map, e.buf, (long long)q.n[0] * w.Kp / 2, q.n[1], q.n[2], bx * w.Kp / 2, by) != cudaSuccess) {
+            t = typename Work<T>::S3Lev();
+            return BURA_OK;  // a map the driver does not accept: the grid sweeps
+        }
+        t.maps.push_back(ent);
+    }
+    if (p->var) CA(upload_packed(p, h, g));
+    CK(sweep3_prepare(w.Kp, p->var));
+    t.on = true;
+    return BURA_OK;
+}
+
 // full = false: only what the mixed path's FP64 refinement and bura_apply_shifted use of the FP64 work
 // (level-0 launch shape, geometry and face coefficients, the shifts); no hierarchy, no PCG buffers.
 template <class T>
@@ -743,8 +841,30 @@ int build_work(bura_plan* p, Work<T>& w, bool full = true) {
     w.c1.assign(nlev, nullptr);
     w.c2.assign(nlev, nullptr);
     w.deg.resize(nlev);
+    w.s3.assign(nlev, typename Work<T>::S3Lev());
+    if (full) {  // the level vectors, the smoothing degrees and the CG's vectors
+        for (int l = 0; l < nlev; ++l) {
+            const HostLevel& h = p->hl[l];
+            const size_t vb = (size_t)h.N * w.Kp * sizeof(T);
+            CA(dalloc(p, &w.b[l], vb));  // level 0 uses the CG residual instead; kept for the coarse CTA
+            CA(dalloc(p, &w.xa[l], vb));
+            CA(dalloc(p, &w.xb[l], vb));
+            CA(dalloc(p, &w.dd[l], vb));
+            int deg = p->opt.smoother_degree;
+            if (l == nlev - 1)
+                deg = h.N == 1 ? 1 : (p->opt.coarse_degree > 0 ? p->opt.coarse_degree
+                                      : p->dim == 0 ? kCsrDegree : coarse_degree_auto(h, p->d[0]));
+            w.deg[l] = deg;
+            // the Chebyshev tables (deg x Kp each) depend on the shifts: filled by upload_tables
+            CA(dalloc(p, &w.c1[l], (size_t)deg * w.Kp * sizeof(T)));
+            CA(dalloc(p, &w.c2[l], (size_t)deg * w.Kp * sizeof(T)));
+        }
+        const size_t vb0 = (size_t)p->hl[0].N * w.Kp * sizeof(T);
+        for (T** q : {&w.x, &w.r, &w.pa, &w.pb, &w.q}) CA(dalloc(p, q, vb0));
+    }
     for (int l = 0; l < nlev; ++l) {
         const HostLevel& h = p->hl[l];
+        if (full) CA(build_sweep3(p, w, l));
         w.g[l] = make_launch(w.Kp, w.W, h.N, p->nsm, p->opt.block_points, p->opt.blocks_per_sm);
         Lev& L = w.L[l];
         L.nx = h.n[0];
@@ -781,25 +901,12 @@ int build_work(bura_plan* p, Work<T>& w, bool full = true) {
             // the CG operator's faces in T; the V-cycle's in bf16 when asked (FP32 path), with the diagonal
             // summed from the stored values so each level operator is the M-matrix of its stored faces
             const bool bf = sizeof(T) == 4 && p->opt.smoother_bf16;
-            if (!bf || l == 0) CA(upload_faces<T>(p, h, L, false));
+            if (!w.s3[l].on && (!bf || l == 0)) CA(upload_faces<T>(p, h, L, false));
             if (l == 0) w.Lop = L;
             if (bf) CA(upload_faces<T>(p, h, L, true));
         }
         if (l == 0 && !p->var) w.Lop = L;
         if (!full) break;
-        const size_t vb = (size_t)h.N * w.Kp * sizeof(T);
-        CA(dalloc(p, &w.b[l], vb));  // level 0 uses the CG residual instead; kept for the coarse CTA
-        CA(dalloc(p, &w.xa[l], vb));
-        CA(dalloc(p, &w.xb[l], vb));
-        CA(dalloc(p, &w.dd[l], vb));
-        const bool coarsest = (l == nlev - 1);
-        int deg = p->opt.smoother_degree;
-        if (coarsest) deg = h.N == 1 ? 1 : (p->opt.coarse_degree > 0 ? p->opt.coarse_degree
-                                            : p->dim == 0 ? kCsrDegree : coarse_degree_auto(h, p->d[0]));
-        w.deg[l] = deg;
-        // the Chebyshev tables (deg x Kp each) depend on the shifts: filled by upload_tables
-        CA(dalloc(p, &w.c1[l], (size_t)deg * w.Kp * sizeof(T)));
-        CA(dalloc(p, &w.c2[l], (size_t)deg * w.Kp * sizeof(T)));
     }
     if (!full) {
         CA(dalloc(p, &w.dsh, KMAXP * sizeof(T)));
@@ -870,19 +977,12 @@ int build_work(bura_plan* p, Work<T>& w, bool full = true) {
     if (w.lc >= 0 && w.coarse_kind == BURA_COARSE_CTA)
         CK(Ops<T>::prepare_coarse(p->dim, p->var,
                                   w.coarse_smem + kCoarseTables + KMAXP * sizeof(double) + w.minv_smem));
-    const size_t vb0 = (size_t)p->hl[0].N * w.Kp * sizeof(T);
-    CA(dalloc(p, &w.x, vb0));
-    CA(dalloc(p, &w.r, vb0));
-    CA(dalloc(p, &w.pa, vb0));
-    CA(dalloc(p, &w.pb, vb0));
-    CA(dalloc(p, &w.q, vb0));
     CA(dalloc(p, &w.dsh, KMAXP * sizeof(T)));
     CA(upload_tables<T>(p, w));
     CA(dalloc(p, &w.scal, sizeof(Scal)));
     CK(cudaMemset(w.scal, 0, sizeof(Scal)));
     CA(build_tma(p, w));
     if (sizeof(T) == 4 && p->dim == 2 && !p->var && w.Kp <= 16) CK(strip_prepare(w.Kp));
-    if (sizeof(T) == 4 && p->dim == 3 && w.Kp <= 16) CK(cheb3s_prepare(w.Kp, p->var));
     w.ready = true;
     return BURA_OK;
 }
@@ -1112,6 +1212,8 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
     T* cur = A;
     T* oth = B;
     const auto& tl = w.tma[l];
+    const auto& s3l = w.s3[l];
+    const bool s3 = s3l.on;
     // one Chebyshev step, TMA-staged where the level has tensor maps
     auto cheb = [&](const T* xin, const T* din, T* xout, T* dout, ChebStepT<T> cs, const Red& red) {
         const CUtensorMap* mx = tl.on ? tl.find(TB_HALO, xin) : nullptr;
@@ -1120,10 +1222,10 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
         if (mx && mb && (md || !din))
             (void)tma_cheb_step(tl.geo, p->nsm, *mx, md, *mb, reinterpret_cast<float*>(xout),
                                 reinterpret_cast<float*>(dout), f32_step(cs), f32_ptr(w.dsh), red, s);
-        else if (f32 && dim == 3 && kCheb3s && !L.cbf16 && L.nx >= kCheb3sMinN)
-            (void)launch_cheb_step3s(L, w.Kp, var, p->nsm, f32_ptr(xin), f32_ptr(din), f32_ptr(b),
-                                     reinterpret_cast<float*>(xout), reinterpret_cast<float*>(dout), f32_step(cs),
-                                     f32_ptr(w.dsh), red, s);
+        else if (s3)
+            (void)sweep3_step(s3l.geo, s3l.at(S3B_HALO, xin), din ? &s3l.at(S3B_TILE, din) : nullptr, s3l.at(S3B_TILE, b),
+                              reinterpret_cast<float*>(xout), reinterpret_cast<float*>(dout), f32_step(cs), f32_ptr(w.dsh),
+                              red, s);
         else
             Ops<T>::cheb_step(g, L, dim, var, xin, din, b, xout, dout, cs, w.dsh, red, s);
     };
@@ -1196,6 +1298,18 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
     if (deg == 1) {
         traced(p, K_CHEB0, f32, fine, vbytes<T>(p, l, 2.0, var), s,
                [&] { Ops<T>::cheb_zero(g, L, dim, var, b, A, step_of(w, l, 0), w.dsh, s); });
+    } else if (s3) {  // both steps from zero in one staged sweep
+        traced(p, K_PRE2, f32, fine, vbytes<T>(p, l, deg > 2 ? 3.0 : 2.0, true), s, [&] {
+            (void)sweep3_pre(s3l.geo, s3l.at(S3B_HALO, b), reinterpret_cast<float*>(A),
+                             reinterpret_cast<float*>(deg > 2 ? D : nullptr), f32_step(step_of(w, l, 0)),
+                             f32_step(step_of(w, l, 1)), f32_ptr(w.dsh), none, s);
+        });
+        for (int m = 2; m < deg; ++m) {
+            T* dout = m < deg - 1 ? D : nullptr;
+            traced(p, K_CHEB, f32, fine, vbytes<T>(p, l, 4.0 + (dout ? 1.0 : 0.0), true), s,
+                   [&] { cheb(cur, D, oth, dout, step_of(w, l, m), none); });
+            std::swap(cur, oth);
+        }
     } else if (!tl.on && split_sweeps(p)) {
         traced(p, K_CHEB0, f32, fine, vbytes<T>(p, l, 2.0, var), s,
                [&] { Ops<T>::cheb_zero(g, L, dim, var, b, A, step_of(w, l, 0), w.dsh, s); });
@@ -1237,15 +1351,14 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
     // coarse-grid correction: residual + restriction, then the coarser levels.  In 3-D and with variable
     // coefficients the residual is stored (in D, free between pre- and post-smoothing) and restricted by a
     // second sweep: 27 (3-D) stencil evaluations per coarse point cost more than the extra vector pass.
-    if (dim == 3 || var) {
+    if (s3) {
+        traced(p, K_RESTRICT, f32, fine, vbytes<T>(p, l, 2.0, true) + vbytes<T>(p, l + 1, 1.0, false), s, [&] {
+            (void)sweep3_residual_restrict(s3l.geo, s3l.at(S3B_RHALO, cur), s3l.at(S3B_RTILE, b),
+                                           reinterpret_cast<float*>(w.b[l + 1]), f32_ptr(w.dsh), none, s);
+        });
+    } else if (dim == 3 || var) {
         traced(p, K_RESID, f32, fine, vbytes<T>(p, l, 3.0, true), s,
-               [&] {
-                   if (f32 && dim == 3 && kCheb3s && !L.cbf16 && L.nx >= kCheb3sMinN)
-                       (void)launch_residual3s(L, w.Kp, var, p->nsm, f32_ptr(cur), f32_ptr(b),
-                                               reinterpret_cast<float*>(D), f32_ptr(w.dsh), s);
-                   else
-                       Ops<T>::residual(g, L, dim, var, cur, b, D, w.dsh, s);
-               });
+               [&] { Ops<T>::residual(g, L, dim, var, cur, b, D, w.dsh, s); });
         traced(p, K_RESTRICT, f32, fine, vbytes<T>(p, l, 1.0, false) + vbytes<T>(p, l + 1, 1.0, false), s,
                [&] { Ops<T>::restrict_r(w.g[l + 1], L, w.L[l + 1], dim, D, w.b[l + 1], s); });
     } else {
@@ -1254,10 +1367,21 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
         });
     }
     T* ec = vcycle<T>(p, w, l + 1, w.b[l + 1], false, s);
-    traced(p, K_PROLONG, f32, fine, vbytes<T>(p, l, 2.0, false) + vbytes<T>(p, l + 1, 1.0, false), s,
-           [&] { Ops<T>::prolong_add(g, L, w.L[l + 1], dim, ec, cur, s); });
+    int m0 = 0;
+    if (s3) {  // the correction and the first post-smoothing step in one staged sweep
+        traced(p, K_PROCHEB, f32, fine, vbytes<T>(p, l, 4.0, true) + vbytes<T>(p, l + 1, 1.0, false), s, [&] {
+            (void)sweep3_prolong_step(s3l.geo, s3l.at(S3B_HALO, cur), s3l.at(S3B_COARSE, ec), s3l.at(S3B_TILE, b),
+                                      reinterpret_cast<float*>(oth), reinterpret_cast<float*>(D),
+                                      f32_step(step_of(w, l, 0, false)), f32_ptr(w.dsh), none, s);
+        });
+        std::swap(cur, oth);
+        m0 = 1;
+    } else {
+        traced(p, K_PROLONG, f32, fine, vbytes<T>(p, l, 2.0, false) + vbytes<T>(p, l + 1, 1.0, false), s,
+               [&] { Ops<T>::prolong_add(g, L, w.L[l + 1], dim, ec, cur, s); });
+    }
     // post-smoothing with the same polynomial (symmetric preconditioner)
-    for (int m = 0; m < deg; ++m) {
+    for (int m = m0; m < deg; ++m) {
         const bool last = (m == deg - 1);
         T* din = m == 0 ? nullptr : D;
         T* dout = last ? nullptr : D;
@@ -1281,16 +1405,22 @@ int pcg_body(bura_plan* p, Work<T>& w, unsigned long long cond, cudaStream_t s) 
     const Red rconv = deferred(p, Red{p->partial, p->tickets, w.scal, nullptr, RED_CONV, cond});
     T* z = vcycle<T>(p, w, 0, w.r, true, s);
     const auto& tl = w.tma[0];
-    if (!tl.on && split_sweeps(p))  // p = z + beta p as its own pointwise sweep
+    const auto& s3l = w.s3[0];
+    const bool s3 = s3l.on;
+    if (!tl.on && split_sweeps(p) && !s3)  // p = z + beta p as its own pointwise sweep
         traced(p, K_PUPD, f32, true, vbytes<T>(p, 0, 3.0, false), s,
                [&] { Ops<T>::pupdate(g, L.N, z, w.pa, w.pb, ralpha, s); });
-    traced(p, K_SPMV, f32, true, vbytes<T>(p, 0, !tl.on && split_sweeps(p) ? 2.0 : 4.0, true), s, [&] {
+    traced(p, K_SPMV, f32, true, vbytes<T>(p, 0, !tl.on && split_sweeps(p) && !s3 ? 2.0 : 4.0, true), s, [&] {
         const CUtensorMap* mz = tl.on ? tl.find(TB_HALO, z) : nullptr;
         const CUtensorMap* ma = tl.on ? tl.find(TB_HALO, w.pa) : nullptr;
         const CUtensorMap* mbb = tl.on ? tl.find(TB_HALO, w.pb) : nullptr;
         if (mz && ma && mbb)
             (void)tma_spmv_p(tl.geo, p->nsm, *mz, *ma, *mbb, reinterpret_cast<float*>(w.pa),
                              reinterpret_cast<float*>(w.pb), reinterpret_cast<float*>(w.q), ralpha, s);
+        else if (s3)
+            (void)sweep3_spmv(s3l.geo, s3l.at(S3B_HALO, z), s3l.at(S3B_HALO, w.pa), s3l.at(S3B_HALO, w.pb),
+                              reinterpret_cast<float*>(w.pa), reinterpret_cast<float*>(w.pb), reinterpret_cast<float*>(w.q),
+                              ralpha, s);
         else if (split_sweeps(p))
             Ops<T>::spmv_q(g, L, p->dim, p->var, w.pa, w.pb, w.q, ralpha, s);
         else

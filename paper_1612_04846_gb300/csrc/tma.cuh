@@ -220,4 +220,37 @@ cudaError_t tma_cg_update(const TmaGeo& g, int nsm, const CUtensorMap& mx, const
 cudaError_t tma_spmv_p(const TmaGeo& g, int nsm, const CUtensorMap& mz, const CUtensorMap& mpa,
                        const CUtensorMap& mpb, float* pa, float* pb, float* q, const Red& red, cudaStream_t s);
 
+// Tensor map of ny x nz rows of `row` eight-byte elements (a row a multiple of 16 bytes), box bx x by elements and rows
+// of one plane; zero fill outside.
+cudaError_t tma_encode3(CUtensorMap* m, const void* base, long long row, int ny, int nz, int bx, int by);
+
+// The 3-D sweeps staged by TMA (sweep3d.cu): modes, the boxes of their maps (in grid points), and a level's geometry.
+enum Sweep3Mode { S3_STEP = 0, S3_PRE = 1, S3_RESR = 2, S3_PROL = 3, S3_SPMV = 4 };
+enum Sweep3Box { S3B_HALO = 0, S3B_TILE = 1, S3B_RHALO = 2, S3B_RTILE = 3, S3B_COARSE = 4 };
+void sweep3_box(int box, int* bx, int* by);
+struct Sweep3Lev {
+    int nx, ny, nz, ncx, ncy, ncz;  // the level and the next coarser one
+    int Kp, nsm;
+    bool var;
+    float wx, wy, wz;               // constant coefficients
+    CUtensorMap w, wr;              // variable coefficients: the packed weights, [nz + 1][ny + 1][nx + 1] float4 (the faces
+                                    // below a point along x, y, z and its diagonal), with the halo boxes HALO and RHALO
+};
+// x: HALO map; din (may be null) and b: TILE maps
+cudaError_t sweep3_step(const Sweep3Lev& g, const CUtensorMap& x, const CUtensorMap* din, const CUtensorMap& b, float* xout,
+                        float* dout, ChebStepT<float> cs, const float* dsh, const Red& red, cudaStream_t s);
+// both pre-smoothing steps from a zero guess (d_2 into dout unless null); b: HALO map
+cudaError_t sweep3_pre(const Sweep3Lev& g, const CUtensorMap& b, float* xout, float* dout, ChebStepT<float> c0,
+                       ChebStepT<float> c1, const float* dsh, const Red& none, cudaStream_t s);
+// bc = R (b - (A - d_j I) x), full weighting; x: RHALO map, b: RTILE map
+cudaError_t sweep3_residual_restrict(const Sweep3Lev& g, const CUtensorMap& x, const CUtensorMap& b, float* bc, const float* dsh,
+                                     const Red& none, cudaStream_t s);
+// a Chebyshev step without previous direction on x + P ec; x: HALO map, ec: the coarse level's COARSE map, b: TILE map
+cudaError_t sweep3_prolong_step(const Sweep3Lev& g, const CUtensorMap& x, const CUtensorMap& ec, const CUtensorMap& b,
+                                float* xout, float* dout, ChebStepT<float> cs, const float* dsh, const Red& none,
+                                cudaStream_t s);
+// p = z + beta p (into the buffer the parity selects) and q = (A - d_j I) p with p . q; z, pa, pb: HALO maps
+cudaError_t sweep3_spmv(const Sweep3Lev& g, const CUtensorMap& z, const CUtensorMap& mpa, const CUtensorMap& mpb, float* pa,
+                        float* pb, float* q, const Red& red, cudaStream_t s);
+
 }  // namespace bura
