@@ -313,14 +313,24 @@ __device__ __forceinline__ void stencil(const Lev& L, int Kp, int P, int off, co
 // per-thread partial sums are deterministic.
 constexpr int kZRun = 16;
 
+// Planes per work item: kZRun on levels whose items fill the grid, fewer on small ones (down to `least`), where a chain
+// of dependent planes costs more than the reuse saves: a 31^3 level has 62 items of 16 planes (10 to 17 us a sweep) and
+// 496 of 2.
+__device__ __forceinline__ int z_run(int per_z, int nz, int nb, int least) {
+    int zr = kZRun;
+    while (zr > least && per_z * ((nz + zr - 1) / zr) < nb) zr >>= 1;
+    return zr;
+}
+
 template <class T, bool VAR, class Body>
 __device__ __forceinline__ void zmarch(const Lev& L, int Kp, const T* __restrict__ x, int b0, int nb, Body&& body) {
     constexpr int W = VecT<T>::W;
     const int off = threadIdx.x * W;
     const int PX = (int)blockDim.y;
     const int nxs = (L.nx + PX - 1) / PX;
-    const int nzc = (L.nz + kZRun - 1) / kZRun;
     const int per_z = nxs * L.ny;
+    const int zr = z_run(per_z, L.nz, nb, 1);
+    const int nzc = (L.nz + zr - 1) / zr;
     const int items = per_z * nzc;
     const size_t sx = (size_t)Kp, sy = (size_t)L.nx * Kp, sz = (size_t)L.plane * Kp;
     const T wxc = sizeof(T) == 4 ? (T)L.wxf : (T)L.wx, wyc = sizeof(T) == 4 ? (T)L.wyf : (T)L.wy;
@@ -331,8 +341,8 @@ __device__ __forceinline__ void zmarch(const Lev& L, int Kp, const T* __restrict
         const int j = rem / nxs;
         const int i = (rem - j * nxs) * PX + (int)threadIdx.y;
         if (i >= L.nx) continue;
-        const int l0 = zc * kZRun;
-        const int l1 = min(L.nz, l0 + kZRun);
+        const int l0 = zc * zr;
+        const int l1 = min(L.nz, l0 + zr);
         int P = (l0 * L.ny + j) * L.nx + i;
         size_t base = (size_t)P * Kp + off;
         T xm1[W], x0[W], xp1[W];
@@ -1024,8 +1034,9 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_min_blocks<3, true>()) k_
     const int off = threadIdx.x * W;
     const int PX = (int)blockDim.y;
     const int nxs = (Lf.nx + PX - 1) / PX;
-    const int nzc = (Lf.nz + kZRun - 1) / kZRun;
     const int per_z = nxs * Lf.ny;
+    const int zr = z_run(per_z, Lf.nz, gridDim.x, 2);
+    const int nzc = (Lf.nz + zr - 1) / zr;
     const int items = per_z * nzc;
     for (int item = blockIdx.x; item < items; item += gridDim.x) {
         const int zc = item / per_z;
@@ -1059,8 +1070,8 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_min_blocks<3, true>()) k_
                 sv[v] = t;
             }
         };
-        const int l0 = zc * kZRun;  // even
-        const int l1 = min(Lf.nz, l0 + kZRun);
+        const int l0 = zc * zr;  // even
+        const int l1 = min(Lf.nz, l0 + zr);
         T sp[W], sc[W];             // the interpolations on coarse planes l / 2 - 1 and l / 2 (l even)
         T en[4][W];                 // the footprint of the next coarse plane, fetched one fine plane early
         fetch((l0 >> 1) - 1, en);

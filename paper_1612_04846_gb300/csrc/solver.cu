@@ -865,7 +865,10 @@ int build_work(bura_plan* p, Work<T>& w, bool full = true) {
     for (int l = 0; l < nlev; ++l) {
         const HostLevel& h = p->hl[l];
         if (full) CA(build_sweep3(p, w, l));
-        w.g[l] = make_launch(w.Kp, w.W, h.N, p->nsm, p->opt.block_points, p->opt.blocks_per_sm);
+        // a row segment of the 3-D column sweeps is a CTA's points: no more of them than a short row has
+        int points = p->opt.block_points;
+        if (points == 0 && l > 0 && p->dim == 3 && h.n[0] <= 32) points = h.n[0] <= 16 ? 16 : 32;
+        w.g[l] = make_launch(w.Kp, w.W, h.N, p->nsm, points, p->opt.blocks_per_sm);
         Lev& L = w.L[l];
         L.nx = h.n[0];
         L.ny = h.n[1];
