@@ -258,10 +258,11 @@ cudaError_t fdiag_launch(const FdiagArgs& a, int G, size_t smem, int nsys, cudaS
 
 // A whole mixed-precision solve of a small 2-D constant-coefficient plan in one launch (resident.cu): a
 // thread-block cluster per system runs the refinement and CG loops on vectors kept in shared memory.
-constexpr int kResMaxLevels = 8;
+constexpr int kResMaxLevels = 10;
 constexpr int kResMaxOuter = 64;                 // refinement steps whose iteration counts a record holds
-constexpr size_t kResSmemMax = 230912;           // dynamic shared memory of a CTA (227 KB less the static arrays)
-constexpr size_t kResSmemHalf = 114176;          // ... of one of two CTAs that share an SM
+constexpr size_t kResSmemMax = 230400;           // dynamic shared memory of a CTA (227 KB less the static arrays)
+constexpr size_t kResSmemHalf = 113920;          // ... of one of two CTAs that share an SM
+constexpr int kResCycleMaxN = 127;               // a larger plan's V-cycle runs resident from the first level this small
 struct ResOut {                                  // a system's outcome
     double rr, fnorm2;
     int outer, siters, status;
@@ -271,17 +272,21 @@ struct ResLevel {
     int nx, ny;
     float wx, wy;
     const float *c1, *c2;                        // Chebyshev tables of the level, [step][Kp]
+    const float *fx, *fy, *dg;                   // variable coefficients: scaled faces and diagonal (as Lev)
     int oR, oX, oY, oD;                          // shared-memory offsets (floats)
+    int oW, wsz;                                 // of the weights: fx, fy, dg, wsz floats each
 };
 struct ResArgs {
-    int le, ne;                                  // the exact level (the last one) and its rows
+    bool var, vonly;                             // variable coefficients; one V-cycle only
+    int le, ne;                                  // the last level in slabs (the exact one, or the first of the tail), its rows
+    int ld;                                      // variable coefficients: the tail's last level, solved with dense inverses
     int re, ce;                                  // rows and columns of it per CTA
     int G, threads;                              // CTAs per system, threads per CTA
     int Kp;
     size_t N;
     double wx, wy;                               // level-0 weights in FP64
-    ResLevel lev[kResMaxLevels];
-    int o_sx, o_sy, o_lam, o_zero, o_p, o_r64, o_r64_end, o_d, o_vs, o_vh, o_bt, o_br, o_cc, o_cd, o_x, floats;
+    ResLevel lev[kResMaxLevels], tail[kResMaxLevels];  // in slabs; the tail's whole levels (le .. ld)
+    int o_inv, o_sx, o_sy, o_lam, o_zero, o_p, o_r64, o_r64_end, o_d, o_vs, o_vh, o_bt, o_br, o_cc, o_cd, o_x, floats;
     unsigned img_bytes;
     const float* img;                            // sine bases and eigenvalues of the exact level (res_image)
     const float* dsh;                            // shifts
@@ -290,12 +295,17 @@ struct ResArgs {
                                                  // no room for them (o_x < 0)
     double* v;                                   // [system][N] solutions
     ResOut* out;                                 // [system]
+    const float* minv;                           // variable coefficients: dense inverses of level ld, [row][col][Kp]
+    const double *fx64, *fy64, *dg64;            // and the level-0 weights in FP64
+    const float* vb;                             // one V-cycle: right-hand side and result of level 0, [point][Kp]
+    float* vx;
+    Scal* scal;                                  // ... and the record of a fault
 };
 size_t res_image_floats(int nx, int ny);
 void res_image(int nx, int ny, const double* sx, const double* sy, const float* lx, const float* ly, float* img);
 // Chooses the cluster size and lays out the shared memory of a plan whose levels are filled in; false if the
 // plan does not fit.  Called at plan setup, outside any capture.
-bool resident_plan(ResArgs& a);
+bool resident_plan(ResArgs& a, int K);
 cudaError_t launch_resident(const ResArgs& a, int K, const double* f, double tol, cudaStream_t s);
 // u = sum_j c_j v_j (or V: the systems) and the outcome into st (page-locked host memory)
 cudaError_t launch_resident_out(const ResArgs& a, int K, const double* c, double* u, double* V, int accumulate,

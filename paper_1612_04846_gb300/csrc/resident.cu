@@ -35,6 +35,9 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <array>
+#include <map>
+#include <mutex>
 
 #include "kernels_impl.cuh"
 #include "tma.cuh"
@@ -108,6 +111,11 @@ __device__ __forceinline__ bool wait_bytes(uint64_t* bar, unsigned parity) {
         if (clock64() - t0 > kTmaWaitCycles) return false;
     }
 }
+// One float from global to shared memory, asynchronously; copies_done() waits for this thread's.
+__device__ __forceinline__ void copy4(float* dst, const float* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
 __device__ __forceinline__ void st2(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
 __device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
@@ -196,7 +204,9 @@ struct Ctx {
 
 }  // namespace
 
-template <int kResThreads>
+// VAR: variable coefficients.  VONLY: one V-cycle from level 0 of the arguments for the interleaved right-hand side a.vb
+// into a.vx, instead of the whole solve.
+template <int kResThreads, bool VAR, bool VONLY>
 __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(const __grid_constant__ ResArgs a, const double* f, double tol) {
     constexpr int kResWarps = kResThreads / 32;
     extern __shared__ __align__(16) float rsm[];
@@ -204,7 +214,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
     __shared__ double slots[2][16];      // a reduction's partial sums of every CTA (FP64, or Df pairs)
     __shared__ double wsum[kResWarps];
     __shared__ double bc[6];             // FP64 scalars that one warp computes for all
-    __shared__ Split<kResWarps> split[kResMaxLevels];
+    __shared__ Split<kResWarps> split[kResMaxLevels], tsplit[VAR ? kResMaxLevels : 1];  // of the slabs; of the tail's levels
     __shared__ float coef[kResMaxLevels][3];  // c2 of the first Chebyshev step, c1 and c2 of the second
     __shared__ int late_in[16];          // each CTA's copy timed out
     __shared__ __align__(8) uint64_t bimg, bR[kResMaxLevels], bD[kResMaxLevels], bC, bB, bV, bS[2];
@@ -228,43 +238,93 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         mbar_init(&bS[0], 1);
         mbar_init(&bS[1], 1);
         mbar_fence_init();
-        const long long w = a.cfg->wait_cycles;
-        mbar_expect_tx(&bimg, a.img_bytes);
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(smem_u32(sm + a.o_sx)), "l"(a.img), "r"(a.img_bytes), "r"(smem_u32(&bimg))
-                     : "memory");
-        // a wait budget of the caller's starts at the copy's issue; the default one after the buffers are cleared
-        if (w > 0) late = !mbar_wait_bounded(&bimg, 0, w);
+        if (!VAR) {
+            const long long w = a.cfg->wait_cycles;
+            mbar_expect_tx(&bimg, a.img_bytes);
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(smem_u32(sm + a.o_sx)), "l"(a.img), "r"(a.img_bytes), "r"(smem_u32(&bimg))
+                         : "memory");
+            // a wait budget of the caller's starts at the copy's issue; the default one after the buffers are cleared
+            if (w > 0) late = !mbar_wait_bounded(&bimg, 0, w);
+        }
     }
     __syncthreads();
-    if (tid < 4 * (le + 1)) {  // thread (level, kind)
-        const int l = tid >> 2, k = tid & 3, nch = (a.lev[l].nx + 63) >> 6;
-        int y0, y1;
-        slab(g, a.re, a.ne, le - l, a.lev[l].ny, y0, y1);
-        const int rows = y1 - y0 + (k == 3 ? 4 : k);
-        int h = 1, best = 1 << 30;
-        for (int q = 1; q <= kStrip; ++q) {
-            const int cost = (((rows + q - 1) / q) * nch + kResWarps - 1) / kResWarps * (q + 1);
-            if (cost < best) { best = cost; h = q; }
+    const int lend = VAR ? a.ld : le;  // the last level
+    if (tid < 8 * (lend + 1)) {  // thread (level, slabs or tail, kind)
+        const int l = tid >> 3, k = tid & 3, nch = (a.lev[l].nx + 63) >> 6;
+        const bool tail = (tid & 4) != 0;
+        if (tail ? VAR && l >= le : l <= le) {
+            int y0 = 0, y1 = a.lev[l].ny;
+            if (!tail) slab(g, a.re, a.ne, le - l, a.lev[l].ny, y0, y1);
+            const int rows = y1 - y0 + (k == 3 ? 4 : k);
+            int h = 1, best = 1 << 30;
+            for (int q = 1; q <= kStrip; ++q) {
+                const int cost = (((rows + q - 1) / q) * nch + kResWarps - 1) / kResWarps * (q + 1);
+                if (cost < best) { best = cost; h = q; }
+            }
+            Split<kResWarps>& sp = tail ? tsplit[VAR ? l : 0] : split[l];
+            sp.h[k] = h;
+            for (int w = k; w < kResWarps; w += 4) {
+                sp.s[w] = (unsigned char)(w / nch);
+                sp.ch[w] = (unsigned char)(w % nch);
+            }
+            if (k == 0) {
+                sp.nch = nch;
+                sp.q = kResWarps / nch;
+                sp.m = kResWarps % nch;
+            }
         }
-        Split<kResWarps>& sp = split[l];
-        sp.h[k] = h;
-        for (int w = k; w < kResWarps; w += 4) {
-            sp.s[w] = (unsigned char)(w / nch);
-            sp.ch[w] = (unsigned char)(w % nch);
-        }
-        if (k == 0) {
-            sp.nch = nch;
-            sp.q = kResWarps / nch;
-            sp.m = kResWarps % nch;
-        }
-        if (l < le && k < 3) coef[l][k] = k == 0 ? a.lev[l].c2[sys] : k == 1 ? a.lev[l].c1[a.Kp + sys] : a.lev[l].c2[a.Kp + sys];
+        if (!tail && l < lend && k < 3)
+            coef[l][k] = k == 0 ? a.lev[l].c2[sys] : k == 1 ? a.lev[l].c1[a.Kp + sys] : a.lev[l].c2[a.Kp + sys];
     }
     // everything but the bases starts at zero: the zero columns and the rows outside the grid stay zero
     for (int i = a.o_zero / 4 + tid; i < a.floats / 4; i += kResThreads)
         reinterpret_cast<float4*>(sm)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (!mbar_wait_bounded(&bimg, 0, kTmaWaitCycles)) late = true;  // (a late copy lands before the kernel goes on)
+    if (!VAR && !mbar_wait_bounded(&bimg, 0, kTmaWaitCycles)) late = true;  // (a late copy lands before the kernel goes on)
     int faulted = __syncthreads_or(late);
+    if constexpr (VAR) {
+        // the weights (faces negated) of the own rows and three halo rows, the tail's whole levels and its dense inverse in
+        // CTA 0; 1 on the diagonal where there is no point
+        auto weights = [&](const ResLevel& L, int y0, int y1) {
+            const int ld = row_floats(L.nx), rows = y1 - y0 + 2 * kHR, nx = L.nx;
+            float *wx = sm + L.oW, *wy = wx + L.wsz, *wd = wy + L.wsz;
+            for (int r = cx.warp; r <= rows; r += kResWarps) {
+                const int y = y0 - kHR + r;
+                const bool iny = y >= 0 && y < L.ny;
+                for (int x = cx.lane; x <= nx; x += 32) {
+                    const int i = r * ld + x + 2;
+                    if (iny && r < rows) copy4(wx + i, L.fx + (size_t)y * (nx + 1) + x);
+                    if (x < nx && y >= 0 && y <= L.ny) copy4(wy + i, L.fy + (size_t)y * nx + x);
+                    if (x < nx && iny && r < rows) copy4(wd + i, L.dg + (size_t)y * nx + x);
+                }
+            }
+        };
+        auto each = [&](auto&& fn) {  // fn(level, first row, end) for every level whose weights this CTA keeps
+            for (int l = 0; l < le; ++l) {
+                int y0, y1;
+                slab(g, a.re, a.ne, le - l, a.lev[l].ny, y0, y1);
+                if (y1 > y0) fn(a.lev[l], y0, y1);
+            }
+            if (g == 0)
+                for (int l = le; l < lend; ++l) fn(a.tail[l], 0, a.tail[l].ny);
+        };
+        each([&](const ResLevel& L, int, int) {
+            for (int i = tid; i < L.wsz; i += kResThreads) sm[L.oW + 2 * L.wsz + i] = 1.f;
+        });
+        __syncthreads();
+        each(weights);
+        if (g == 0) {
+            const int n = a.tail[lend].nx * a.tail[lend].ny;
+            for (int i = tid; i < n * n; i += kResThreads) copy4(sm + a.o_inv + i, a.minv + (size_t)i * a.Kp + sys);
+        }
+        copies_done();
+        __syncthreads();
+        each([&](const ResLevel& L, int, int) {
+            for (int i = tid; i < 2 * L.wsz; i += kResThreads) sm[L.oW + i] = -sm[L.oW + i];
+        });
+        __syncthreads();
+    }
+    if (VONLY) pdl_wait();  // what is read so far does not depend on the kernel before
     cl.sync();  // every CTA runs and has cleared its buffers and barriers before the first remote store
 
     unsigned uR = 0, uD = 0, uC = 0, uB = 0, uV = 0, uS = 0;  // the parity of each barrier's next phase
@@ -286,6 +346,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         s.ld = row_floats(s.nx);
         return s;
     };
+    auto whole = [&](int l) { return Slab{0, a.lev[l].ny, a.lev[l].nx, a.lev[l].ny, row_floats(a.lev[l].nx)}; };
     // (y, x) of a buffer at base + y * ld + x
     auto at = [&](int ofs, int H, const Slab& s) { return sm + ofs + (H - s.y0) * s.ld + 2; };
     int flip = 0;
@@ -340,78 +401,71 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         return t;
     };
 
-    const Slab s0 = range(0);
-    const int np = (s0.y1 - s0.y0) * s0.nx;  // own points of level 0, numbered along the rows
-    const int ld0 = s0.ld, ldx = even(s0.nx);
-    float* const R0 = at(a.lev[0].oR, kHR, s0);
-    float* const P0 = at(a.o_p, kHP, s0);
-    double* const r64 = reinterpret_cast<double*>(sm + a.o_r64);     // own points (over P, X, Y, D: free between inner solves)
-    double* const vg = a.v + (size_t)sys * a.N;
-    double* const vs = reinterpret_cast<double*>(sm + a.o_vs);       // v of the own points for the residual
-    double* const vh = reinterpret_cast<double*>(sm + a.o_vh);       // v on the rows below and above the slab
-    // x of the own points, rows of ldx
-    float* const xs = (a.o_x >= 0 ? sm + a.o_x : a.x + ((size_t)sys * s0.ny + s0.y0) * ldx) - (size_t)s0.y0 * ldx;
-    const size_t gofs = (size_t)s0.y0 * s0.nx;
-
-    if (cx.warp == kResWarps - 1) {
-        // this system's relative threshold need_j, reached in n_j = ceil(log need_j / log inner_rtol - 1e-9) steps of
-        // need_j^(1/n_j) each; n_j by comparing with the powers of inner_rtol (rtol_slack = inner_rtol^1e-9)
-        const OuterCfg& c = *a.cfg;
-        const double t = c.lambda_lo > 0 ? tol * (c.lambda_lo - c.d[sys]) / (c.K * c.c[sys]) : tol;
-        double st2 = 1.0;  // the square of a step's share
-        if (t < 1.0) {
-            double r = c.inner_rtol;
-            int n = 1;
-            for (; t < r * c.rtol_slack && r > 0.0; ++n) r *= c.inner_rtol;
-            st2 = n == 1 ? t * t : n == 2 ? t : pow(t, 2.0 / n);
+    // ---- pieces of the V-cycle, on slabs or (loc) on the tail's whole levels in CTA 0
+    // the operator at pair index k of a level: A c (no shift) and the pair's diagonal (variable coefficients)
+    struct Op {
+        const float *fx, *fy, *dg;
+        int ld;
+        float wx, wy, diag;
+        __device__ __forceinline__ float2 apply(int k, float2 c, float l, float r, float2 u, float2 w, float2& dv) const {
+            if constexpr (VAR) {
+                const float2 xm = ld2(fx + k), ym = ld2(fy + k), yp = ld2(fy + k + ld);
+                dv = ld2(dg + k);
+                float2 t = __fmul2_rn(dv, c);
+                t.x = fmaf(xm.x, l, t.x);
+                t.y = fmaf(xm.y, c.x, t.y);
+                t.x = fmaf(xm.y, c.y, t.x);
+                t.y = fmaf(fx[k + 2], r, t.y);
+                t = __ffma2_rn(ym, u, t);
+                return __ffma2_rn(yp, w, t);
+            } else {
+                return stencil2(wx, wy, diag, c, l, r, u, w);
+            }
         }
-        if (cx.lane == 0) {
-            bc[5] = t;
-            bc[2] = 0.25 * st2;
-        }
-    }
-    // ||f||^2
-    double part = 0.0;
-    for (int i = tid; i < np; i += kResThreads) {
-        const double v = __ldg(f + gofs + i);
-        part = fma(v, v, part);
-    }
-    if (tid < G) put(reinterpret_cast<float*>(&late_in[g]), tid, &bS[0], __int_as_float(faulted));
-    const double sum_f = all_sum64(part, 4u * G);
-    for (int t = 0; t < G; ++t) faulted |= late_in[t];
-    if (tid == 0) {
-        bc[0] = sum_f;
-        bc[1] = bc[5] * bc[5] * sum_f;
-    }
-    __syncthreads();
-    const double fn2 = bc[0], thr64 = bc[1];
-    const int max_outer = a.cfg->max_outer, max_iters = a.cfg->max_iters;
-
-    // ---- pieces of the V-cycle
+    };
+    auto op_of = [&](const ResLevel& L, const Slab& s) {
+        Op o;
+        o.ld = s.ld;
+        o.wx = L.wx;
+        o.wy = L.wy;
+        o.diag = L.wx + L.wx + L.wy + L.wy;
+        o.fx = sm + L.oW + (kHR - s.y0) * s.ld + 2;
+        o.fy = o.fx + L.wsz;
+        o.dg = o.fy + L.wsz;
+        return o;
+    };
+    // the Jacobi scaling: the constant operator's is part of the coefficients
+    auto jac = [&](float2 v, float2 dv) { return VAR ? make_float2(jdiv(v.x, dv.x - d), jdiv(v.y, dv.y - d)) : v; };
+    auto jac1 = [&](float v, const float* dg) { return VAR ? jdiv(v, *dg - d) : v; };
     // way down level l: x2 (both pre-smoothing steps from zero) on the own rows and two halo rows, the residual
     // in Y on the fine rows the slab restricts, its full weighting into R of level l + 1
-    auto down = [&](int l) {
-        const ResLevel& L = a.lev[l];
-        const Slab s = range(l), sc = range(l + 1);
+    auto down = [&](int l, bool loc) {
+        const ResLevel &L = loc ? a.tail[VAR ? l : 0] : a.lev[l];
+        const Slab s = loc ? whole(l) : range(l), sc = loc ? whole(l + 1) : range(l + 1);
+        const Split<kResWarps>&sp = loc ? tsplit[VAR ? l : 0] : split[l], &spc = loc ? tsplit[VAR ? l + 1 : 0] : split[l + 1];
         const int ld = s.ld, nx = s.nx;
-        const float wx = L.wx, wy = L.wy, diag = wx + wx + wy + wy;
+        const Op A = op_of(L, s);
         const float c20 = coef[l][0], c1 = coef[l][1], c2 = coef[l][2];
-        const bool more = l + 1 < le;  // the exact level reads its own rows only
+        const bool more = !loc && l + 1 < le;  // the last slab level's readers take their own rows only
         if (more) arm(&bR[l + 1], sc.halo_bytes(kHR));
+        if (VAR && !loc && l + 1 == le && g == 0) arm(&bC, (unsigned)(sc.ny * even(sc.nx) * 4));
         if (s.some()) {
             const float* R = at(L.oR, kHR, s);
             float* X = at(L.oX, kHX, s);
-            cx.strips(split[l], 3, max(0, s.y0 - 2), min(s.ny, s.y1 + 2), nx, [&](int y, int n, int x) {
-                const float* q = R + y * ld + x;
-                float* o = X + y * ld + x;
+            cx.strips(sp, 3, max(0, s.y0 - 2), min(s.ny, s.y1 + 2), nx, [&](int y, int n, int x) {
+                int k = y * ld + x;
+                const float* q = R + k;
+                float* o = X + k;
                 const bool last = x + 1 >= nx;
-                float2 b = ld2(q), c = __fmul2_rn(dup(c20), b), u = __fmul2_rn(dup(c20), ld2(q - ld));
-                for (int i = 0; i < n; ++i, q += ld, o += ld) {
-                    const float2 bn = ld2(q + ld), w = __fmul2_rn(dup(c20), bn);
-                    const float2 t = stencil2(wx, wy, diag, c, c20 * q[-1], c20 * q[2], u, w);
+                auto first = [&](float2 b, int kk) { return jac(__fmul2_rn(dup(c20), b), VAR ? ld2(A.dg + kk) : b); };
+                float2 b = ld2(q), c = first(b, k), u = first(ld2(q - ld), k - ld);
+                for (int i = 0; i < n; ++i, q += ld, o += ld, k += ld) {
+                    const float2 bn = ld2(q + ld), w = first(bn, k + ld);
+                    float2 dv;
+                    const float2 t = A.apply(k, c, jac1(c20 * q[-1], A.dg + k - 1), jac1(c20 * q[2], A.dg + k + 2), u, w, dv);
                     const float2 tt = __ffma2_rn(dup(-d), c, t);
                     const float2 res = make_float2(b.x - tt.x, b.y - tt.y);
-                    float2 v = __fadd2_rn(c, __ffma2_rn(dup(c1), c, __fmul2_rn(dup(c2), res)));
+                    float2 v = __fadd2_rn(c, __ffma2_rn(dup(c1), c, jac(__fmul2_rn(dup(c2), res), dv)));
                     if (last) v.y = 0.f;
                     st2(o, v);
                     u = c; c = w; b = bn;
@@ -422,14 +476,15 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         if (s.some()) {
             const float *R = at(L.oR, kHR, s), *X = at(L.oX, kHX, s);
             float* Y = at(L.oY, kHY, s);
-            cx.strips(split[l], 1, s.y0, min(s.ny, s.y1 + 1), nx, [&](int y, int n, int x) {
-                const float* q = X + y * ld + x;
-                const float* rb = R + y * ld + x;
-                float* o = Y + y * ld + x;
+            cx.strips(sp, 1, s.y0, min(s.ny, s.y1 + 1), nx, [&](int y, int n, int x) {
+                int k = y * ld + x;
+                const float *q = X + k, *rb = R + k;
+                float* o = Y + k;
                 float2 u = ld2(q - ld), c = ld2(q);
-                for (int i = 0; i < n; ++i, q += ld, rb += ld, o += ld) {
+                for (int i = 0; i < n; ++i, q += ld, rb += ld, o += ld, k += ld) {
                     const float2 w = ld2(q + ld);
-                    const float2 t = __ffma2_rn(dup(-d), c, stencil2(wx, wy, diag, c, q[-1], q[2], u, w));
+                    float2 dv;
+                    const float2 t = __ffma2_rn(dup(-d), c, A.apply(k, c, q[-1], q[2], u, w, dv));
                     const float2 b = ld2(rb);
                     st2(o, make_float2(b.x - t.x, b.y - t.y));
                     u = c; c = w;
@@ -439,9 +494,9 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         __syncthreads();
         if (sc.some()) {
             const float* Y = at(L.oY, kHY, s);
-            const int oRc = a.lev[l + 1].oR;
+            const int oRc = loc ? a.tail[VAR ? l + 1 : 0].oR : a.lev[l + 1].oR;
             float* Rc = at(oRc, kHR, sc);
-            cx.strips(split[l + 1], 0, sc.y0, sc.y1, sc.nx, [&](int J, int n, int I) {
+            cx.strips(spc, 0, sc.y0, sc.y1, sc.nx, [&](int J, int n, int I) {
                 const float* q = Y + 2 * J * ld + 2 * I;
                 const bool last = I + 1 >= sc.nx;
                 for (int i = 0; i < n; ++i, ++J, q += 2 * ld) {
@@ -455,8 +510,12 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
                         t.y = fmaf(w0, e, fmaf(w1, m.y, fmaf(w0, m.x, t.y)));
                     }
                     if (last) t.y = 0.f;
-                    st2(Rc + J * sc.ld + I, t);
-                    if (more) cx.share(l + 1, oRc, kHR, sc, &bR[l + 1], J, I, t);
+                    if (VAR && !loc && l + 1 == le) {  // into CTA 0's whole level
+                        put2(sm + a.tail[le].oR + (J + kHR) * sc.ld + I + 2, 0, &bC, t.x, t.y);
+                    } else {
+                        st2(Rc + J * sc.ld + I, t);
+                        if (more) cx.share(l + 1, oRc, kHR, sc, &bR[l + 1], J, I, t);
+                    }
                 }
             });
         }
@@ -465,19 +524,20 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
     };
     // way up level l: x2 + P (result of level l + 1) on two halo rows, the first post-smoothing step on one, the
     // second on the own rows into D; returns this thread's part of r.z
-    auto up = [&](int l) {
-        const ResLevel& L = a.lev[l];
-        const Slab s = range(l), sc = range(l + 1);
+    auto up = [&](int l, bool loc) {
+        const ResLevel &L = loc ? a.tail[VAR ? l : 0] : a.lev[l];
+        const Slab s = loc ? whole(l) : range(l), sc = loc ? whole(l + 1) : range(l + 1);
+        const Split<kResWarps>& sp = loc ? tsplit[VAR ? l : 0] : split[l];
         const int ld = s.ld, ldc = sc.ld, nx = s.nx;
-        const float wx = L.wx, wy = L.wy, diag = wx + wx + wy + wy;
+        const Op A = op_of(L, s);
         const float c20 = coef[l][0], c1 = coef[l][1], c2 = coef[l][2];
         const float* R = at(L.oR, kHR, s);
         float *X = at(L.oX, kHX, s), *Y = at(L.oY, kHY, s), *D = at(L.oD, kHD, s);
-        const float* E = at(a.lev[l + 1].oD, kHD, sc);
+        const float* E = at(loc ? a.tail[VAR ? l + 1 : 0].oD : a.lev[l + 1].oD, kHD, sc);
         Df tot{0.f, 0.f};
-        arm(&bD[l], s.halo_bytes(kHD));
+        if (!loc) arm(&bD[l], s.halo_bytes(kHD));
         if (s.some()) {
-            cx.strips(split[l], 3, max(0, s.y0 - 2), min(s.ny, s.y1 + 2), nx, [&](int y, int n, int x) {
+            cx.strips(sp, 3, max(0, s.y0 - 2), min(s.ny, s.y1 + 2), nx, [&](int y, int n, int x) {
                 const bool last = x + 1 >= nx;
                 float* o = X + y * ld + x;
                 for (int i = 0; i < n; ++i, ++y, o += ld) {
@@ -500,16 +560,17 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         }
         __syncthreads();
         if (s.some()) {
-            cx.strips(split[l], 2, max(0, s.y0 - 1), min(s.ny, s.y1 + 1), nx, [&](int y, int n, int x) {
+            cx.strips(sp, 2, max(0, s.y0 - 1), min(s.ny, s.y1 + 1), nx, [&](int y, int n, int x) {
                 const bool last = x + 1 >= nx;
-                const int k = y * ld + x;
+                int k = y * ld + x;
                 const float *q = X + k, *rb = R + k;
                 float *oy = Y + k, *od = D + k;
                 float2 u = ld2(q - ld), c = ld2(q);
-                for (int i = 0; i < n; ++i, q += ld, rb += ld, oy += ld, od += ld) {
+                for (int i = 0; i < n; ++i, q += ld, rb += ld, oy += ld, od += ld, k += ld) {
                     const float2 w = ld2(q + ld), b = ld2(rb);
-                    const float2 t = __ffma2_rn(dup(-d), c, stencil2(wx, wy, diag, c, q[-1], q[2], u, w));
-                    float2 dv = __fmul2_rn(dup(c20), make_float2(b.x - t.x, b.y - t.y));
+                    float2 dg;
+                    const float2 t = __ffma2_rn(dup(-d), c, A.apply(k, c, q[-1], q[2], u, w, dg));
+                    float2 dv = jac(__fmul2_rn(dup(c20), make_float2(b.x - t.x, b.y - t.y)), dg);
                     if (last) dv.y = 0.f;
                     st2(oy, __fadd2_rn(c, dv));
                     if (y + i >= s.y0 && y + i < s.y1) st2(od, dv);
@@ -519,20 +580,21 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         }
         __syncthreads();
         if (s.some()) {
-            cx.strips(split[l], 0, s.y0, s.y1, nx, [&](int y, int n, int x) {
+            cx.strips(sp, 0, s.y0, s.y1, nx, [&](int y, int n, int x) {
                 const bool last = x + 1 >= nx;
-                const int k = y * ld + x;
+                int k = y * ld + x;
                 const float *q = Y + k, *rb = R + k;
                 float* od = D + k;
                 float2 u = ld2(q - ld), c = ld2(q), p2 = make_float2(0.f, 0.f);
-                for (int i = 0; i < n; ++i, q += ld, rb += ld, od += ld) {
+                for (int i = 0; i < n; ++i, q += ld, rb += ld, od += ld, k += ld) {
                     const float2 w = ld2(q + ld), b = ld2(rb);
-                    const float2 t = __ffma2_rn(dup(-d), c, stencil2(wx, wy, diag, c, q[-1], q[2], u, w));
+                    float2 dg;
+                    const float2 t = __ffma2_rn(dup(-d), c, A.apply(k, c, q[-1], q[2], u, w, dg));
                     const float2 res = make_float2(b.x - t.x, b.y - t.y);
-                    float2 z = __fadd2_rn(c, __ffma2_rn(dup(c1), ld2(od), __fmul2_rn(dup(c2), res)));
+                    float2 z = __fadd2_rn(c, __ffma2_rn(dup(c1), ld2(od), jac(__fmul2_rn(dup(c2), res), dg)));
                     if (last) z.y = 0.f;
                     st2(od, z);
-                    cx.share(l, L.oD, kHD, s, &bD[l], y + i, x, z);
+                    if (!loc) cx.share(l, L.oD, kHD, s, &bD[l], y + i, x, z);
                     p2 = __ffma2_rn(b, z, p2);
                     u = c; c = w;
                 }
@@ -540,8 +602,49 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
             });
         }
         __syncthreads();
-        await(&bD[l], uD, l);
+        if (!loc) await(&bD[l], uD, l);
         return tot;
+    };
+    // variable coefficients: CTA 0 runs the V-cycle of levels le .. lend (dense inverse on the last) on whole levels and
+    // sends every slab its rows of the result with two halo rows
+    auto tail = [&]() {
+        const Slab s = whole(le), mine = range(le);
+        if (mine.some()) arm(&bB, (unsigned)((min(mine.ny, mine.y1 + kHD) - max(0, mine.y0 - kHD)) * even(s.nx) * 4));
+        if (g == 0) {
+            await(&bC, uC, 0);
+            __syncthreads();
+            for (int l = le; l < lend; ++l) down(l, true);
+            const ResLevel& L = a.tail[lend];
+            const int nx = L.nx, n = nx * L.ny, ld = row_floats(nx);
+            float* const b = sm + a.o_bt;
+            for (int i = tid; i < n; i += kResThreads) b[i] = sm[L.oR + (i / nx + kHR) * ld + i % nx + 2];
+            __syncthreads();
+            if (tid < n) {
+                const float* m = sm + a.o_inv + tid * n;
+                float v = 0.f;
+                for (int j = 0; j < n; ++j) v = fmaf(m[j], b[j], v);
+                sm[L.oD + (tid / nx + kHD) * ld + tid % nx + 2] = v;
+            }
+            __syncthreads();
+            for (int l = lend - 1; l >= le; --l) (void)up(l, true);
+            const float* D = at(a.tail[le].oD, kHD, s);
+            const int half = even(s.nx) / 2;
+            for (int i = tid; i < s.ny * half; i += kResThreads) {
+                const int y = i / half, x = 2 * (i - y * half);
+                const float2 v = ld2(D + y * s.ld + x);
+                for (int t = max(0, (y - kHD) / a.re - 1); t < G; ++t) {
+                    int u0, u1;
+                    slab(t, a.re, a.ne, 0, s.ny, u0, u1);
+                    if (u0 >= s.ny || y < u0 - kHD) break;
+                    if (y < u1 + kHD) put2(sm + a.lev[le].oD + (y - u0 + kHD) * s.ld + x + 2, t, &bB, v.x, v.y);
+                }
+            }
+        } else {
+            uC ^= 1u;
+        }
+        if (mine.some()) await(&bB, uB, 0);
+        else uB ^= 1u;
+        __syncthreads();
     };
     // out[q][m] = sum_k S[k][m] C[q][k] (k in increasing order) for m < M, q < Q, handed to epi(q, value) by a thread with
     // tid mod kSP = m; C has rows of kSP floats, zero from Kd on (so that k may run on to a multiple of 4: the bases are
@@ -620,8 +723,87 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         return tot;
     };
 
+    // z = M r into D of level 0; returns this thread's part of r.z
+    auto cycle = [&]() {
+        Df t{0.f, 0.f};
+        for (int l = 0; l < le; ++l) down(l, false);
+        if constexpr (VAR) tail();
+        else t = exact();
+        for (int l = le - 1; l >= 0; --l) t = up(l, false);
+        return t;
+    };
+
+    if constexpr (VONLY) {
+        // the right-hand side on the own rows and the halo rows, one V-cycle, the result's own rows
+        const Slab s = range(0);
+        float* const R = at(a.lev[0].oR, kHR, s);
+        const float* const D = at(a.lev[0].oD, kHD, s);
+        if (s.some()) {
+            for (int y = max(0, s.y0 - kHR) + cx.warp; y < min(s.ny, s.y1 + kHR); y += kResWarps)
+                for (int x = cx.lane; x < s.nx; x += 32) copy4(R + y * s.ld + x, a.vb + ((size_t)y * s.nx + x) * a.Kp + sys);
+        }
+        copies_done();
+        __syncthreads();
+        (void)cycle();
+        if (s.some())
+            for (int y = s.y0 + cx.warp; y < s.y1; y += kResWarps)
+                for (int x = cx.lane; x < s.nx; x += 32) a.vx[((size_t)y * s.nx + x) * a.Kp + sys] = D[y * s.ld + x];
+        if (lost || faulted) atomicExch(&a.scal->fault, 1);
+        pdl_trigger();
+        cl.sync();  // no CTA leaves while another may still store into its shared memory
+        return;
+    }
+
+    // ---- the whole solve
+    const Slab s0 = range(0);
+    const int np = (s0.y1 - s0.y0) * s0.nx;  // own points of level 0, numbered along the rows
+    const int ld0 = s0.ld, ldx = even(s0.nx);
+    float* const R0 = at(a.lev[0].oR, kHR, s0);
+    float* const P0 = at(a.o_p, kHP, s0);
+    double* const r64 = reinterpret_cast<double*>(sm + a.o_r64);     // own points (over P, X, Y, D: free between inner solves)
+    double* const vg = a.v + (size_t)sys * a.N;
+    double* const vs = reinterpret_cast<double*>(sm + a.o_vs);       // v of the own points for the residual
+    double* const vh = reinterpret_cast<double*>(sm + a.o_vh);       // v on the rows below and above the slab
+    // x of the own points, rows of ldx
+    float* const xs = (a.o_x >= 0 ? sm + a.o_x : a.x + ((size_t)sys * s0.ny + s0.y0) * ldx) - (size_t)s0.y0 * ldx;
+    const size_t gofs = (size_t)s0.y0 * s0.nx;
+
+    if (cx.warp == kResWarps - 1) {
+        // this system's relative threshold need_j, reached in n_j = ceil(log need_j / log inner_rtol - 1e-9) steps of
+        // need_j^(1/n_j) each; n_j by comparing with the powers of inner_rtol (rtol_slack = inner_rtol^1e-9)
+        const OuterCfg& c = *a.cfg;
+        const double t = c.lambda_lo > 0 ? tol * (c.lambda_lo - c.d[sys]) / (c.K * c.c[sys]) : tol;
+        double st2 = 1.0;  // the square of a step's share
+        if (t < 1.0) {
+            double r = c.inner_rtol;
+            int n = 1;
+            for (; t < r * c.rtol_slack && r > 0.0; ++n) r *= c.inner_rtol;
+            st2 = n == 1 ? t * t : n == 2 ? t : pow(t, 2.0 / n);
+        }
+        if (cx.lane == 0) {
+            bc[5] = t;
+            bc[2] = 0.25 * st2;
+        }
+    }
+    // ||f||^2
+    double part = 0.0;
+    for (int i = tid; i < np; i += kResThreads) {
+        const double v = __ldg(f + gofs + i);
+        part = fma(v, v, part);
+    }
+    if (tid < G) put(reinterpret_cast<float*>(&late_in[g]), tid, &bS[0], __int_as_float(faulted));
+    const double sum_f = all_sum64(part, 4u * G);
+    for (int t = 0; t < G; ++t) faulted |= late_in[t];
+    if (tid == 0) {
+        bc[0] = sum_f;
+        bc[1] = bc[5] * bc[5] * sum_f;
+    }
+    __syncthreads();
+    const double fn2 = bc[0], thr64 = bc[1];
+    const int max_outer = a.cfg->max_outer, max_iters = a.cfg->max_iters;
+
     // ---- the refinement loop
-    const double c0_64 = 2.0 * (a.wx + a.wy) - a.cfg->d[sys];
+    const double d64 = a.cfg->d[sys], c0_64 = 2.0 * (a.wx + a.wy) - d64;
     double rr64 = fn2;  // uniform: every decision below is taken alike by all threads of the cluster
     int outer = 0, siters = 0, status = -5;
     if (faulted) status = -6;
@@ -672,9 +854,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         for (;;) {
             // z = M r into D
             Df t;
-            for (int l = 0; l < le; ++l) down(l);
-            t = exact();
-            for (int l = le - 1; l >= 0; --l) t = up(l);
+            t = cycle();
             const Df rzn = all_sum(t);
             if (!isfinite(rzn.h)) breakdown = 1;
             const float beta = df_div(rzn, rz);
@@ -693,15 +873,16 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
             __syncthreads();
             t = Df{0.f, 0.f};
             if (s0.some()) {
-                const float wx = L0.wx, wy = L0.wy, diag = wx + wx + wy + wy;
+                const Op A = op_of(L0, s0);
                 cx.strips(split[0], 0, s0.y0, s0.y1, s0.nx, [&](int y, int n, int x) {
-                    const int k = y * ld0 + x;
+                    int k = y * ld0 + x;
                     const float* q = P0 + k;
                     float* o = Q + k;
                     float2 u = ld2(q - ld0), c = ld2(q), p2 = make_float2(0.f, 0.f);
-                    for (int i = 0; i < n; ++i, q += ld0, o += ld0) {
+                    for (int i = 0; i < n; ++i, q += ld0, o += ld0, k += ld0) {
                         const float2 w = ld2(q + ld0);
-                        const float2 v = __ffma2_rn(dup(-d), c, stencil2(wx, wy, diag, c, q[-1], q[2], u, w));
+                        float2 dv;
+                        const float2 v = __ffma2_rn(dup(-d), c, A.apply(k, c, q[-1], q[2], u, w, dv));
                         st2(o, v);
                         p2 = __ffma2_rn(c, v, p2);  // c is zero in the padding column
                         u = c; c = w;
@@ -764,12 +945,24 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         for (int i = tid; i < np; i += kResThreads) {
             const int r = i / s0.nx, x = i - r * s0.nx, y = s0.y0 + r;
             const double* q = vs + i;
-            const double sx = (x > 0 ? q[-1] : 0.0) + (x < s0.nx - 1 ? q[1] : 0.0);
             const double lo = y == 0 ? 0.0 : r == 0 ? vh[x] : q[-s0.nx];
             const double hi = y == s0.ny - 1 ? 0.0 : y == s0.y1 - 1 ? vh[s0.nx + x] : q[s0.nx];
-            double v = fma(-c0_64, q[0], __ldg(f + gofs + i));
-            v = fma(a.wx, sx, v);
-            v = fma(a.wy, lo + hi, v);
+            const double fv = __ldg(f + gofs + i);
+            double v;
+            if constexpr (VAR) {  // f - (A - d I) v, the grid kernel's order
+                const size_t P = gofs + i, F = (size_t)y * (s0.nx + 1) + x;
+                v = __ldg(a.dg64 + P) * q[0];
+                v = fma(-__ldg(a.fx64 + F), x > 0 ? q[-1] : 0.0, v);
+                v = fma(-__ldg(a.fx64 + F + 1), x < s0.nx - 1 ? q[1] : 0.0, v);
+                v = fma(-__ldg(a.fy64 + P), lo, v);
+                v = fma(-__ldg(a.fy64 + P + s0.nx), hi, v);
+                v = fv - fma(-d64, q[0], v);
+            } else {
+                const double sx = (x > 0 ? q[-1] : 0.0) + (x < s0.nx - 1 ? q[1] : 0.0);
+                v = fma(-c0_64, q[0], fv);
+                v = fma(a.wx, sx, v);
+                v = fma(a.wy, lo + hi, v);
+            }
             r64[i] = v;
             t = fma(v, v, t);
         }
@@ -853,10 +1046,12 @@ bool res_layout(ResArgs& a, int G) {
         o = (int)std::min<long long>(1 << 28, up4((int)std::min<long long>(1 << 28, o + n)));
         return at;
     };
-    a.o_sx = take((long long)nxe * kSP);
-    a.o_sy = take((long long)a.ne * kSP);
-    a.o_lam = take(2 * kSP);
-    a.img_bytes = (unsigned)(res_image_floats(nxe, a.ne) * sizeof(float));
+    if (!a.var) {
+        a.o_sx = take((long long)nxe * kSP);
+        a.o_sy = take((long long)a.ne * kSP);
+        a.o_lam = take(2 * kSP);
+        a.img_bytes = (unsigned)(res_image_floats(nxe, a.ne) * sizeof(float));
+    }
     a.o_zero = o;
     for (int l = 0; l <= a.le; ++l) {
         ResLevel& L = a.lev[l];
@@ -864,15 +1059,16 @@ bool res_layout(ResArgs& a, int G) {
         const int sh = a.le - l;
         const int tail = ((last << sh) + (1 << sh) - 1);  // the last slab's rows
         const int most = std::min(std::max(a.re << sh, tail), L.ny);
-        L.oR = take((long long)(most + 2 * kHR) * ld);
-        if (l == 0) {
+        const bool smoothed = l < a.le, cg = l == 0 && !a.vonly;
+        L.oR = smoothed || !a.var ? take((long long)(most + 2 * kHR) * ld) : o;
+        if (cg) {
             a.o_r64 = o;
             a.o_p = take((long long)(most + 2 * kHP) * ld);
         }
-        L.oX = l < a.le ? take((long long)(most + 2 * kHX) * ld) : o;
-        L.oY = l < a.le || l == 0 ? take((long long)(most + 2 * kHY) * ld) : o;
+        L.oX = smoothed ? take((long long)(most + 2 * kHX) * ld) : o;
+        L.oY = smoothed || cg ? take((long long)(most + 2 * kHY) * ld) : o;
         L.oD = take((long long)(most + 2 * kHD) * ld);
-        if (l == 0) {  // between inner solves: the FP64 residual, v with its neighbours' edge rows, the partials of a norm
+        if (cg) {  // between inner solves: the FP64 residual, v with its neighbours' edge rows, the partials of a norm
             own0 = (long long)most * even(L.nx);
             const int end = o;
             o = a.o_r64;
@@ -882,11 +1078,31 @@ bool res_layout(ResArgs& a, int G) {
             a.o_d = take(2 * 32 * kResMostWarps);
             a.o_r64_end = o = std::max(o, end);
         }
+        L.wsz = (most + 2 * kHR + 1) * ld;
+        if (a.var && smoothed) L.oW = take(3LL * L.wsz);
     }
-    a.o_bt = take((long long)a.re * kSP);
-    a.o_br = take((long long)a.re * kSP);
-    a.o_cc = take((long long)a.ce * kSP);
-    a.o_cd = take((long long)a.ce * kSP);
+    if (a.var) {  // the tail's whole levels, the dense inverse of its last one
+        for (int l = a.le; l <= a.ld; ++l) {
+            ResLevel& L = a.tail[l];
+            L = a.lev[l];
+            const int ld = row_floats(L.nx);
+            L.oR = take((long long)(L.ny + 2 * kHR) * ld);
+            L.oD = take((long long)(L.ny + 2 * kHD) * ld);
+            if (l == a.ld) break;
+            L.oX = take((long long)(L.ny + 2 * kHX) * ld);
+            L.oY = take((long long)(L.ny + 2 * kHY) * ld);
+            L.wsz = (L.ny + 2 * kHR + 1) * ld;
+            L.oW = take(3LL * L.wsz);
+        }
+        const int n = a.lev[a.ld].nx * a.lev[a.ld].ny;
+        a.o_inv = take((long long)n * n);
+        a.o_bt = take(n);
+    } else {
+        a.o_bt = take((long long)a.re * kSP);
+        a.o_br = take((long long)a.re * kSP);
+        a.o_cc = take((long long)a.ce * kSP);
+        a.o_cd = take((long long)a.ce * kSP);
+    }
     a.floats = o;
     a.o_x = -1;
     const size_t room = (size_t)o * sizeof(float) <= kResSmemHalf ? kResSmemHalf : kResSmemMax;
@@ -898,13 +1114,11 @@ bool res_layout(ResArgs& a, int G) {
 }
 
 using ResKernel = void (*)(const ResArgs, const double*, double);
-ResKernel res_kernel(const ResArgs& a) { return a.threads == 256 ? k_resident<256> : k_resident<512>; }
-
-// The limits are properties of the function: always the largest, whatever a plan takes.
-cudaError_t res_attributes(ResKernel k) {
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemMax);
+template <bool VAR, bool VONLY>
+ResKernel res_kernel_t(const ResArgs& a) { return a.threads == 256 ? k_resident<256, VAR, VONLY> : k_resident<512, VAR, VONLY>; }
+ResKernel res_kernel(const ResArgs& a) {
+    return a.var ? (a.vonly ? res_kernel_t<true, true>(a) : res_kernel_t<true, false>(a))
+                 : (a.vonly ? res_kernel_t<false, true>(a) : res_kernel_t<false, false>(a));
 }
 
 cudaLaunchConfig_t res_config(const ResArgs& a, int blocks, cudaLaunchAttribute* attr, cudaStream_t s) {
@@ -919,6 +1133,11 @@ cudaLaunchConfig_t res_config(const ResArgs& a, int blocks, cudaLaunchAttribute*
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    if (a.vonly) {  // within a chain of dependent launches: the setup overlaps the kernel before
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.numAttrs = 2;
+    }
     return cfg;
 }
 
@@ -936,28 +1155,51 @@ void res_image(int nx, int ny, const double* sx, const double* sy, const float* 
     std::copy(ly, ly + ny, img + (size_t)(nx + ny + 1) * kSP);
 }
 
+// Clusters of a plan's shape that the current device holds at once (0: none), after setting the kernel's limits, which are
+// properties of the function: always the largest, whatever a plan takes.  The counts are kept: a query costs more than the
+// rest of a small plan's setup, and there are few shapes.
+int resident_clusters(const ResArgs& a) {
+    static std::mutex m;
+    static std::map<std::array<int, 5>, int> known;
+    const ResKernel k = res_kernel(a);
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemMax) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    const std::array<int, 5> key = {dev, (a.var ? 2 : 0) + (a.vonly ? 1 : 0), a.threads, a.G, a.floats};
+    std::lock_guard<std::mutex> lock(m);
+    const auto it = known.find(key);
+    if (it != known.end()) return it->second;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = res_config(a, a.G, attr, nullptr);
+    if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (known.size() < 4096) known[key] = n;
+    return n;
+}
+
 // The largest cluster of up to 16 CTAs (the device holds 7 clusters of 16 at one CTA per SM; more systems than that
 // run as the first clusters finish: 255^2 with 13 systems 989 -> 420 us).  Slabs small enough for two CTAs per SM
 // take 256 threads each, so that 14 clusters are resident (63^2, k = 9: 80 us with 512 threads, 49 with 256; 32
 // problems of up to 127^2 as one batch: 1772 and 993 us); larger ones take 512 (255^2, k = 5: 173 us, 189 with 256).
-bool resident_plan(ResArgs& a) {
+bool resident_plan(ResArgs& a, int K) {
     for (int G = 16; G >= 1; G /= 2) {
         if (G > a.ne || G > a.lev[a.le].nx) continue;
         if (!res_layout(a, G)) return false;
         a.G = G;
         a.threads = (size_t)a.floats * sizeof(float) <= kResSmemHalf ? 256 : 512;
-        if (res_attributes(res_kernel(a)) != cudaSuccess) { cudaGetLastError(); return false; }
-        cudaLaunchAttribute attr[1];
-        cudaLaunchConfig_t cfg = res_config(a, G, attr, nullptr);
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, res_kernel(a), &cfg) != cudaSuccess) { cudaGetLastError(); continue; }
-        if (n >= 1) return true;
+        const int n = resident_clusters(a);
+        if (n >= (a.vonly ? K : 1)) return true;  // a V-cycle inside an iteration takes one round of clusters
     }
     return false;
 }
 
 cudaError_t launch_resident(const ResArgs& a, int K, const double* f, double tol, cudaStream_t s) {
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = res_config(a, K * a.G, attr, s);
     return cudaLaunchKernelEx(&cfg, res_kernel(a), a, f, tol);
 }

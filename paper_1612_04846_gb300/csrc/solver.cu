@@ -47,7 +47,7 @@ struct HostLevel {
 // Kernel types for launch counting and per-kernel timing (fine level only).
 enum KId { K_SPMV, K_CGUPD, K_CHEB0, K_CHEB, K_RESTRICT, K_PRE2, K_PROLONG, K_COARSE, K_DOT, K_BCAST, K_NORM,
            K_RES64, K_CAST, K_CORR64, K_WSUM, K_GATHER, K_CLUSTER, K_PRE2R, K_PROCHEB, K_RESDF, K_CASTDF, K_REDFIN,
-           K_POST2, K_RESID, K_PUPD, K_FDIAG, K_POST2S, K_NK };
+                  K_POST2, K_RESID, K_PUPD, K_FDIAG, K_POST2S, K_RESV, K_NK };
 // [kernel][f32][coarser level]
 const char* const kNames[K_NK][2][2] = {
     {{"spmv_p_f64", "spmv_p_f64@coarse"}, {"spmv_p_f32", "spmv_p_f32@coarse"}},
@@ -76,7 +76,8 @@ const char* const kNames[K_NK][2][2] = {
     {{"residual_f64", "residual_f64@coarse"}, {"residual_f32", "residual_f32@coarse"}},
     {{"p_update_f64", "p_update_f64"}, {"p_update_f32", "p_update_f32"}},
     {{"coarse_fdiag_f64", "coarse_fdiag_f64@coarse"}, {"coarse_fdiag_f32", "coarse_fdiag_f32@coarse"}},
-    {{"post2_strip_f64", "post2_strip_f64@coarse"}, {"post2_strip_f32", "post2_strip_f32@coarse"}}};
+    {{"post2_strip_f64", "post2_strip_f64@coarse"}, {"post2_strip_f32", "post2_strip_f32@coarse"}},
+    {{"coarse_resident_f64", "coarse_resident_f64@coarse"}, {"coarse_resident_f32", "coarse_resident_f32@coarse"}}};
 constexpr int kSlots = K_NK * 4;
 
 struct Tracer {
@@ -90,6 +91,7 @@ struct Tracer {
     long long launches = 0;  // every launch of the current solve
 };
 constexpr size_t kMaxTimed = 16384;
+constexpr int kCoarseResident = 100;  // a coarse kind that only AUTO chooses
 
 template <class T>
 struct Work {
@@ -102,7 +104,8 @@ struct Work {
     std::vector<T*> c1, c2;       // [level] -> deg rows of Kp coefficients, in the kernels' precision
     std::vector<int> deg;
     int lc = -1;                  // first level run by the coarse kernel (-1: none, grid kernels to the end)
-    int coarse_kind = 0;          // BURA_COARSE_CLUSTER, BURA_COARSE_CTA or BURA_COARSE_FDIAG
+    int coarse_kind = 0;          // BURA_COARSE_CLUSTER, BURA_COARSE_CTA, BURA_COARSE_FDIAG or kCoarseResident
+    ResArgs rv{};                 // kCoarseResident: the V-cycle from level lc down (resident.cu)
     int csize = 0;                // CTAs of the cluster (cluster kind)
     int le = -1;                  // level solved exactly with dense inverses inside that kernel (-1: none)
     T* minv = nullptr;            // the inverses, [row][col][Kp]
@@ -683,7 +686,7 @@ int upload_tables(bura_plan* p, Work<T>& w) {
     if (w.minv) {
         std::vector<double> inv;
         dense_inverses(p->hl[w.le], p->dim, p->var, p->d, p->K, w.Kp, inv);
-        const std::vector<T> tv(inv.begin(), inv.end());
+        const std::vector<T> tv(inv.begin(), inv.end());  // (w.le: its level)
         CK(cudaMemcpy(w.minv, tv.data(), tv.size() * sizeof(T), cudaMemcpyHostToDevice));
     }
     return BURA_OK;
@@ -824,6 +827,124 @@ int build_sweep3(bura_plan* p, Work<T>& w, int l) {
     return BURA_OK;
 }
 
+// The arguments of the resident kernels (resident.cu) for the 2-D hierarchy from level l0 down: geometry, tables,
+// coefficients, and for constant ones the image of the exact level's sine bases.  False in *fits where the hierarchy has
+// no such form: it has to reach a level of at most 63 points per axis (constant coefficients, solved by fast
+// diagonalization) or, below a level of at most 31, one of at most kExactPoints points (dense inverses).
+int resident_args(bura_plan* p, Work<float>& w, int l0, bool vonly, ResArgs& a, bool* fits) {
+    *fits = false;
+    const int nlev = (int)p->hl.size();
+    auto size = [&](int l) { return std::max(p->hl[l].n[0], p->hl[l].n[1]); };
+    int le = p->var ? l0 + 1 : l0;
+    while (le < nlev && size(le) > (p->var ? 31 : kFdiagMaxN<float>)) ++le;
+    if (le >= nlev) return BURA_OK;
+    int ld = le;
+    if (p->var) {
+        while (ld < nlev && p->hl[ld].N > kExactPoints) ++ld;
+        if (ld >= nlev || p->hl[l0].N <= kExactPoints || ld != w.le || !w.minv) return BURA_OK;
+    }
+    if (ld - l0 >= kResMaxLevels) return BURA_OK;
+    a.var = p->var;
+    a.vonly = vonly;
+    a.le = le - l0;
+    a.ld = ld - l0;
+    a.ne = p->hl[le].n[1];
+    a.Kp = w.Kp;
+    a.N = (size_t)p->hl[l0].N;
+    a.wx = p->hl[l0].w[0];
+    a.wy = p->hl[l0].w[1];
+    for (int l = l0; l <= ld; ++l) {
+        ResLevel& L = a.lev[l - l0];
+        L.nx = p->hl[l].n[0];
+        L.ny = p->hl[l].n[1];
+        L.wx = (float)p->hl[l].w[0];
+        L.wy = (float)p->hl[l].w[1];
+        L.c1 = w.c1[l];
+        L.c2 = w.c2[l];
+        L.fx = reinterpret_cast<const float*>(w.L[l].fx);
+        L.fy = reinterpret_cast<const float*>(w.L[l].fy);
+        L.dg = reinterpret_cast<const float*>(w.L[l].dg);
+    }
+    a.minv = w.minv;
+    a.dsh = w.dsh;
+    if (!resident_plan(a, p->K)) return BURA_OK;
+    if (!p->var) {
+        const int nx = p->hl[le].n[0], ny = p->hl[le].n[1];
+        std::vector<double> S[2];
+        std::vector<float> lam[2];
+        for (int q = 0; q < 2; ++q) sine_axis<float>(p->hl[le], q, S[q], lam[q]);
+        std::vector<float> img(res_image_floats(nx, ny));
+        res_image(nx, ny, S[0].data(), S[1].data(), lam[0].data(), lam[1].data(), img.data());
+        float* di = nullptr;
+        CA(dalloc(p, &di, img.size() * sizeof(float)));
+        CK(cudaMemcpy(di, img.data(), img.size() * sizeof(float), cudaMemcpyHostToDevice));
+        a.img = di;
+    }
+    *fits = true;
+    return BURA_OK;
+}
+
+// Plans that the resident kernels serve: 2-D FP32 work of a mixed plan with the default smoothing.  Options that ask for
+// particular sweeps or coarse kernels keep them.
+bool resident_options(const bura_plan* p) {
+    const bura_options& o = p->opt;
+    return p->dim == 2 && p->cluster_ok && o.precision == BURA_PREC_MIXED && o.sweeps == BURA_SWEEP_AUTO && !o.smoother_bf16;
+}
+
+// The one-launch solve of a small plan with FP64 refinement, whose slabs fit the shared memory of a cluster.  It keeps
+// its solutions in the plan's v64 buffer, system by system.
+int build_resident(bura_plan* p) {
+    const bura_options& o = p->opt;
+    Work<float>& w = p->w32;
+    if (!resident_options(p) || o.refine != BURA_REFINE_FP64 || o.post_smooth_split != 0 || o.tma_stages != 0 ||
+        o.max_outer > kResMaxOuter)
+        return BURA_OK;
+    if (!(o.coarse_kernel == BURA_COARSE_AUTO || (o.coarse_kernel == BURA_COARSE_FDIAG && !p->var))) return BURA_OK;
+    const bool smooths = p->var || std::max(p->hl[0].n[0], p->hl[0].n[1]) > kFdiagMaxN<float>;
+    if (smooths && o.smoother_degree != 2) return BURA_OK;
+    ResArgs& a = p->res;
+    CA(resident_args(p, w, 0, false, a, &p->res_on));
+    if (!p->res_on) return BURA_OK;
+    CA(dalloc(p, &a.out, (size_t)p->K * sizeof(ResOut)));
+    a.cfg = p->ocfg;
+    a.x = nullptr;
+    if (a.o_x < 0)
+        CA(dalloc(p, &a.x, (size_t)p->K * p->hl[0].n[1] * ((p->hl[0].n[0] + 1) / 2 * 2) * sizeof(float)));
+    a.v = p->v64;
+    const Lev& L64 = p->w64.L[0];
+    a.fx64 = reinterpret_cast<const double*>(L64.fx);
+    a.fy64 = reinterpret_cast<const double*>(L64.fy);
+    a.dg64 = reinterpret_cast<const double*>(L64.dg);
+    return BURA_OK;
+}
+
+// The lower part of a larger plan's V-cycle as one launch of a cluster per system: the first level (below the finest)
+// that lets every system's cluster be resident at once.  Sets w.lc and the kind on success.
+template <class T>
+int build_resident_cycle(bura_plan* p, Work<T>& w) {
+    if constexpr (sizeof(T) == 4) {
+        if (!resident_options(p) || p->opt.coarse_kernel != BURA_COARSE_AUTO || p->opt.smoother_degree != 2) return BURA_OK;
+        const int nlev = (int)p->hl.size();
+        // (a grid that is the exact level itself is one exact solve)
+        if (!p->var && std::max(p->hl[0].n[0], p->hl[0].n[1]) <= kFdiagMaxN<float>) return BURA_OK;
+        for (int l = 1; l < nlev; ++l) {
+            if (std::max(p->hl[l].n[0], p->hl[l].n[1]) > kResCycleMaxN) continue;
+            bool fits = false;
+            CA(resident_args(p, w, l, true, w.rv, &fits));
+            if (!fits) continue;
+            w.coarse_kind = kCoarseResident;
+            w.lc = l;
+            w.rv.vb = w.b[l];
+            w.rv.vx = w.xa[l];
+            w.rv.cfg = nullptr;  // (p->ocfg, once it exists)
+            // the padding systems of the result are never written
+            CK(cudaMemset(w.xa[l], 0, (size_t)p->hl[l].N * w.Kp * sizeof(T)));
+            return BURA_OK;
+        }
+    }
+    return BURA_OK;
+}
+
 // full = false: only what the mixed path's FP64 refinement and bura_apply_shifted use of the FP64 work
 // (level-0 launch shape, geometry and face coefficients, the shifts); no hierarchy, no PCG buffers.
 template <class T>
@@ -861,6 +982,7 @@ int build_work(bura_plan* p, Work<T>& w, bool full = true) {
         }
         const size_t vb0 = (size_t)p->hl[0].N * w.Kp * sizeof(T);
         for (T** q : {&w.x, &w.r, &w.pa, &w.pb, &w.q}) CA(dalloc(p, q, vb0));
+        CA(dalloc(p, &w.dsh, KMAXP * sizeof(T)));
     }
     for (int l = 0; l < nlev; ++l) {
         const HostLevel& h = p->hl[l];
@@ -929,6 +1051,11 @@ int build_work(bura_plan* p, Work<T>& w, bool full = true) {
     // points per axis replaces that level and every coarser one.  Otherwise, as measured on GB300 (2-D
     // 1023^2, k = 7), the single CTA over shared memory beats the cluster, whose sweeps each pay an L2
     // round trip and a cluster barrier (about 3 us of fixed cost per sweep).
+    if (p->var && p->dim == 2 && w.le >= 0) {  // dense inverses, whichever of the kernels below runs the coarse levels
+        const size_t n = (size_t)p->hl[w.le].N;
+        CA(dalloc(p, &w.minv, n * n * w.Kp * sizeof(T)));
+    }
+    CA(build_resident_cycle<T>(p, w));
     if (w.coarse_kind == BURA_COARSE_AUTO)
         w.coarse_kind = (p->dim == 2 && !p->var && p->cluster_ok) ? BURA_COARSE_FDIAG : BURA_COARSE_CTA;
     if (p->dim == 0) w.coarse_kind = BURA_COARSE_NONE;  // one level: the polynomial preconditioner alone
@@ -962,8 +1089,9 @@ int build_work(bura_plan* p, Work<T>& w, bool full = true) {
             }
         }
     }
-    if (w.lc < 0 || w.coarse_kind == BURA_COARSE_FDIAG) w.le = -1;  // the dense solve lives in the CTA / cluster kernels only
-    if (w.le >= 0) {  // [row][col][Kp] dense inverses of the exact level, filled by upload_tables
+    if (w.lc < 0 || w.coarse_kind == BURA_COARSE_FDIAG || (w.coarse_kind == kCoarseResident && !p->var))
+        w.le = -1;  // no dense solve
+    if (w.le >= 0 && !w.minv) {  // [row][col][Kp] dense inverses of the exact level, filled by upload_tables
         const size_t n = (size_t)p->hl[w.le].N;
         CA(dalloc(p, &w.minv, n * n * w.Kp * sizeof(T)));
     }
@@ -980,63 +1108,12 @@ int build_work(bura_plan* p, Work<T>& w, bool full = true) {
     if (w.lc >= 0 && w.coarse_kind == BURA_COARSE_CTA)
         CK(Ops<T>::prepare_coarse(p->dim, p->var,
                                   w.coarse_smem + kCoarseTables + KMAXP * sizeof(double) + w.minv_smem));
-    CA(dalloc(p, &w.dsh, KMAXP * sizeof(T)));
     CA(upload_tables<T>(p, w));
     CA(dalloc(p, &w.scal, sizeof(Scal)));
     CK(cudaMemset(w.scal, 0, sizeof(Scal)));
     CA(build_tma(p, w));
     if (sizeof(T) == 4 && p->dim == 2 && !p->var && w.Kp <= 16) CK(strip_prepare(w.Kp));
     w.ready = true;
-    return BURA_OK;
-}
-
-// The one-launch solve: 2-D constant coefficients in mixed precision with FP64 refinement and the default
-// smoothing, whose hierarchy ends in the fast-diagonalization level and whose slabs fit the shared memory of a
-// cluster.  Options that ask for particular sweeps keep the graph of kernels.  It keeps its solutions in the
-// plan's v64 buffer, system by system.
-int build_resident(bura_plan* p) {
-    const bura_options& o = p->opt;
-    Work<float>& w = p->w32;
-    if (o.precision != BURA_PREC_MIXED || o.refine != BURA_REFINE_FP64 || p->dim != 2 || p->var) return BURA_OK;
-    if (w.coarse_kind != BURA_COARSE_FDIAG || w.lc < 0 || w.lc >= kResMaxLevels) return BURA_OK;
-    if ((w.lc > 0 && o.smoother_degree != 2) || o.sweeps != BURA_SWEEP_AUTO || o.post_smooth_split != 0 || o.tma_stages != 0 ||
-        o.max_outer > kResMaxOuter)
-        return BURA_OK;
-    ResArgs& a = p->res;
-    a.le = w.lc;
-    a.ne = p->hl[w.lc].n[1];
-    a.Kp = w.Kp;
-    a.N = (size_t)p->hl[0].N;
-    a.wx = p->hl[0].w[0];
-    a.wy = p->hl[0].w[1];
-    for (int l = 0; l <= w.lc; ++l) {
-        ResLevel& L = a.lev[l];
-        L.nx = p->hl[l].n[0];
-        L.ny = p->hl[l].n[1];
-        L.wx = (float)p->hl[l].w[0];
-        L.wy = (float)p->hl[l].w[1];
-        L.c1 = w.c1[l];
-        L.c2 = w.c2[l];
-    }
-    if (!resident_plan(a)) return BURA_OK;
-    const int nx = p->hl[w.lc].n[0], ny = p->hl[w.lc].n[1];
-    std::vector<double> S[2];
-    std::vector<float> lam[2];
-    for (int q = 0; q < 2; ++q) sine_axis<float>(p->hl[w.lc], q, S[q], lam[q]);
-    std::vector<float> img(res_image_floats(nx, ny));
-    res_image(nx, ny, S[0].data(), S[1].data(), lam[0].data(), lam[1].data(), img.data());
-    float* di = nullptr;
-    CA(dalloc(p, &di, img.size() * sizeof(float)));
-    CK(cudaMemcpy(di, img.data(), img.size() * sizeof(float), cudaMemcpyHostToDevice));
-    CA(dalloc(p, &a.out, (size_t)p->K * sizeof(ResOut)));
-    a.img = di;
-    a.dsh = w.dsh;
-    a.cfg = p->ocfg;
-    a.x = nullptr;
-    if (a.o_x < 0)
-        CA(dalloc(p, &a.x, (size_t)p->K * p->hl[0].n[1] * ((p->hl[0].n[0] + 1) / 2 * 2) * sizeof(float)));
-    a.v = p->v64;
-    p->res_on = true;
     return BURA_OK;
 }
 
@@ -1186,6 +1263,16 @@ T* fdiag_part(bura_plan* p, Work<T>& w, const T* b, cudaStream_t s) {
     return w.xa[w.lc];
 }
 
+// The V-cycle from level lc down as one launch (its right-hand side is that level's b).
+template <class T>
+T* resident_part(bura_plan* p, Work<T>& w, cudaStream_t s) {
+    w.rv.cfg = p->ocfg;
+    w.rv.scal = w.scal;
+    traced(p, K_RESV, sizeof(T) == 4, w.lc == 0, vbytes<T>(p, w.lc, 2.0, false), s,
+           [&] { (void)launch_resident(w.rv, p->K, nullptr, 0.0, s); });  // errors: cudaGetLastError
+    return w.xa[w.lc];
+}
+
 // Symmetric V-cycle on level l for rhs b; returns the buffer holding the result.  With rz_fused
 // (level 0 only) the last smoothing step also forms r^T z and the CG beta of every system.
 template <class T>
@@ -1202,6 +1289,7 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
     if (l == w.lc) {  // the rest of the hierarchy in one kernel
         T* res = w.coarse_kind == BURA_COARSE_CLUSTER ? cluster_part(p, w, b, s)
                  : w.coarse_kind == BURA_COARSE_FDIAG ? fdiag_part(p, w, b, s)
+                 : w.coarse_kind == kCoarseResident   ? resident_part(p, w, s)
                                                       : coarse_part(p, w, b, s);
         if (rz_fused) {
             traced(p, K_DOT, f32, fine, vbytes<T>(p, l, 2.0, false), s, [&] { Ops<T>::dot(g, L.N, b, res, beta, s); });

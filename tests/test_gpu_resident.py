@@ -9,7 +9,7 @@ iterations within one (the dot products are grouped differently).
 import numpy as np
 import pytest
 
-from oracle import exact, tables
+from oracle import direct, exact, operators, tables
 from paper_1612_04846_gb300 import workloads as W
 
 torch = pytest.importorskip("torch")
@@ -85,3 +85,51 @@ def test_one_launch_outcomes(lib):
         lib.bura_destroy(plan)
     rc, _, st = _solve(lib, shape, k, f, 1e-6, max_iters=1, max_outer=3)
     assert rc == lib.BURA_ENOCONV and st["outer"] == 3 and st["iters"] == 3
+
+
+@pytest.mark.parametrize("shape,k,tol", [((11, 9), 4, 1e-9), ((31, 31), 10, 1e-6), ((63, 23), 5, 1e-8), ((127, 31), 5, 1e-6),
+                                         ((79, 79), 9, 1e-6), ((191, 191), 6, 1e-6)])
+def test_one_launch_solve_variable(lib, shape, k, tol):
+    """Variable coefficients: the tail of the hierarchy in CTA 0, its dense level, slabs of one row to all of them."""
+    nps = tuple(reversed(shape))
+    faces = W.block_lognormal_faces(nps, 4, 1e-2, 1.0, 6)
+    fh = W.rhs_uniform(nps, 63)
+    plan = lib.bura_setup(shape, 0.5, k, faces=faces)
+    try:
+        f = torch.from_numpy(fh).cuda()
+        u = torch.zeros_like(f)
+        assert lib.bura_solve(plan, f, u, tol) == lib.BURA_OK
+        torch.cuda.synchronize()
+        assert lib.bura_get_stats(plan)["launches"] == 2
+    finally:
+        lib.bura_destroy(plan)
+    A, _ = operators.scaled_matrix(nps, faces)
+    e = tables.entry(0.5, k)
+    ur = direct.bura_sparse(A, fh, e["c"], e["d"])
+    assert _rel(u.cpu().numpy(), ur) <= tol
+
+
+@pytest.mark.parametrize("shape,k,var,kind", [((255, 255), 6, True, "CTA"), ((255, 127), 9, True, "CTA"),
+                                              ((511, 255), 10, False, "FDIAG"), ((1023, 511), 7, False, "FDIAG")])
+def test_resident_cycle(lib, shape, k, var, kind):
+    """The lower V-cycle as one launch inside a larger plan against the coarse kernel it replaces: the same operations in
+    the same order per point, so the same iterations and (to the rounding of the FP32 cycle) the same result."""
+    nps, tol = tuple(reversed(shape)), 1e-6
+    faces = W.block_lognormal_faces(nps, 8, 1e-2, 1.0, 7) if var else None
+    f = torch.from_numpy(W.rhs_uniform(nps, 64)).cuda()
+    got = []
+    for coarse in (lib.BURA_COARSE_AUTO, getattr(lib, "BURA_COARSE_" + kind)):
+        o = lib.bura_default_options()
+        o.coarse_kernel = coarse
+        o.tma_stages = 2  # (the graph of kernels)
+        plan = lib.bura_setup(shape, 0.5, k, faces=faces, options=o)
+        try:
+            u = torch.zeros_like(f)
+            assert lib.bura_solve(plan, f, u, tol) == lib.BURA_OK
+            torch.cuda.synchronize()
+            st = lib.bura_get_stats(plan)
+            got.append((u.cpu().numpy(), st["iters"], st["outer"], st["launches"]))
+        finally:
+            lib.bura_destroy(plan)
+    assert got[0][1:3] == got[1][1:3] and got[0][3] < got[1][3]
+    assert _rel(got[0][0], got[1][0]) <= 1e-8
