@@ -1,5 +1,5 @@
-// A whole mixed-precision solve of a small 2-D constant-coefficient plan in one launch, with every vector of
-// the inner solver resident in shared memory.
+// A whole mixed-precision solve of a small 2-D plan in one launch, with every vector of the inner solver resident in
+// shared memory (constant and variable coefficients), and the lower part of a larger 2-D plan's V-cycle as one launch.
 //
 // The shifted systems never exchange values, so each system gets a thread-block cluster of G CTAs of its own
 // that runs the refinement loop, the multigrid-preconditioned CG inside it and all their decisions: the
@@ -32,6 +32,16 @@
 // Measured (GB300, one solve, tol 1e-6, graph of kernels -> here): 63^2, k = 5: 168 -> 45 us; 127^2, k = 6: 372 -> 100;
 // 255^2, k = 7: 550 -> 201; 383 x 255, k = 8: 812 -> 280.  What is left is latency: a 127^2 iteration is 9.5 us, of
 // which the exact solve's four products and three exchanges take 3.6.
+//
+// Variable coefficients: every level's face and diagonal weights stay in the owner's shared memory too (three floats a
+// point, so the largest grid is about 2 / 3 as wide), copied in while the first residual is taken.  The exact level is one
+// dense product per system; grids above 31 put their last levels on the cluster's first CTA, which then runs them without
+// an exchange (a boundary at 15 instead: 127^2 376 -> 403 us, and 191^2 no longer fits).  63^2, k = 5: 1477 -> 279 us;
+// 127^2, k = 6: 2198 -> 376; 191^2: 2819 -> 503.
+//
+// V-cycle only: an iteration of a larger plan launches its levels from the first one of at most kResCycleMaxN points a
+// side here.  About 10 of the launch's 25 us are its start (loading weights and tables), so it takes the place of five or
+// more launches only: var 511^2, k = 7: 4.72 -> 3.79 ms; constant 511^2, three problems: 3.05 -> 2.96; 1023^2: 1.985 -> 1.964.
 #include <cooperative_groups.h>
 
 #include <algorithm>
