@@ -1,4 +1,4 @@
-// TMA-staged sweeps of the large 2-D levels (FP32, constant coefficients).
+// TMA-staged sweeps of the large 2-D levels (FP32).
 //
 // A persistent grid walks tiles of kTX x kTY grid points (tile t = blockIdx.x + k * gridDim.x, a fixed
 // order, so the per-thread partial sums and hence the reductions are deterministic).  For each tile one
@@ -12,7 +12,16 @@
 // The arithmetic is the grid kernels' (kernels_impl.cuh), operation for operation: the stencil sums
 // diag*x and the four neighbours in the same order with the same fused multiply-adds, and a missing
 // neighbour contributes fma(-w, 0, acc) = acc.
+//
+// Variable coefficients take the fused V-cycle step and A p (k_pre2_restrict_tma, k_post2_tma, k_spmv_tma with VAR): one
+// more load per tile brings the weights, packed as a float4 per point (the faces below it along x and y, its diagonal) that
+// all systems of the tile share.  k_pre2_restrict_tma then keeps the first iterate c2 Dinv b of the tile in shared memory
+// (a division per point instead of one per use) and runs two CTAs per SM.  The grid kernels' nine passes a level were
+// launch-bound at 511^2 and read the weights through L1 per thread: 511^2, k = 7: 3.79 -> 2.90 ms; 1023^2: 11.4 -> 6.8;
+// 447 x 255, k = 9: 5.17 -> 3.05.
 #include <cudaTypedefs.h>
+
+#include <algorithm>
 
 #include "kernels_impl.cuh"
 #include "tma.cuh"
@@ -45,12 +54,15 @@ __host__ __device__ constexpr size_t vec_bytes(int pts, int Kp) { return align_u
 
 // Shared-memory bytes of one stage of each kernel kind, and of its unstaged scratch.
 enum TmaKind { TK_CHEB = 0, TK_CHEB_D = 1, TK_PRE2 = 2, TK_SPMV = 3, TK_PRE2R = 4, TK_PROCHEB = 5, TK_CG = 6,
-               TK_POST2 = 7, TK_NKIND = 8 };
+               TK_POST2 = 7, TK_PRE2R_V = 8, TK_POST2_V = 9, TK_SPMV_V = 10, TK_NKIND = 11 };
 __host__ __device__ constexpr size_t stage_bytes(int kind, int Kp) {
     return kind == TK_CHEB ? halo_bytes(Kp) + plain_bytes(Kp)
          : kind == TK_CHEB_D ? halo_bytes(Kp) + 2 * plain_bytes(Kp)
          : kind == TK_PRE2 ? halo_bytes(Kp)
          : kind == TK_SPMV ? 2 * halo_bytes(Kp)
+         : kind == TK_SPMV_V ? 2 * halo_bytes(Kp) + vec_bytes(kHaloPts, 4)
+         : kind == TK_PRE2R_V ? vec_bytes(kRsX * kRsY, Kp) + vec_bytes(kRsX * kRsY, 4)
+         : kind == TK_POST2_V ? vec_bytes(kH2X * kH2Y, Kp) + vec_bytes(kCp2X * kCp2Y, Kp) + halo_bytes(Kp) + vec_bytes(kH2X * kH2Y, 4)
          : kind == TK_PRE2R ? vec_bytes(kRsX * kRsY, Kp)
          : kind == TK_CG ? 4 * plain_bytes(Kp)
          : kind == TK_POST2 ? vec_bytes(kH2X * kH2Y, Kp) + vec_bytes(kCp2X * kCp2Y, Kp) + halo_bytes(Kp)
@@ -59,7 +71,8 @@ __host__ __device__ constexpr size_t stage_bytes(int kind, int Kp) {
 __host__ __device__ constexpr size_t scratch_bytes(int kind, int Kp) {
     return kind == TK_PRE2R ? vec_bytes(kE1X * kE1Y, Kp) + vec_bytes(kRX * kRY, Kp)
          : kind == TK_PROCHEB ? halo_bytes(Kp)
-         : kind == TK_POST2 ? halo_bytes(Kp) + plain_bytes(Kp)
+         : kind == TK_PRE2R_V ? vec_bytes(kE1X * kE1Y, Kp) + vec_bytes(kRX * kRY, Kp) + vec_bytes(kRsX * kRsY, Kp)
+         : kind == TK_POST2 || kind == TK_POST2_V ? halo_bytes(Kp) + plain_bytes(Kp)
          : 0;
 }
 __host__ __device__ constexpr size_t dyn_smem(int kind, int Kp, int S) {
@@ -174,6 +187,35 @@ __device__ __forceinline__ void stencil_tile(const TmaGeo& g, int hidx, const Va
     val(hidx + sy, n);
     for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wy, n[v], acc[v]);
     for (int v = 0; v < 4; ++v) Ax[v] = acc[v];
+}
+
+// The weights of a variable-coefficient point from a tile of packed ones (float4: the faces below the point along x and y,
+// its diagonal); ROW points per tile row.
+struct W5 {
+    float xm, xp, ym, yp, dg;
+};
+template <int ROW>
+__device__ __forceinline__ W5 tile_weights(const float* W, int h) {
+    const float4 w = *reinterpret_cast<const float4*>(W + 4 * h);
+    return {w.x, W[4 * (h + 1)], w.y, W[4 * (h + ROW) + 1], w.z};
+}
+// A x with the grid kernels' order of multiply-adds.
+__device__ __forceinline__ float apply5(const W5& w, float c, float l, float r, float d, float u) {
+    float a = w.dg * c;
+    a = fmaf(-w.xm, l, a);
+    a = fmaf(-w.xp, r, a);
+    a = fmaf(-w.ym, d, a);
+    return fmaf(-w.yp, u, a);
+}
+
+__global__ void k_pack_weights(const float* __restrict__ fx, const float* __restrict__ fy, const float* __restrict__ dg, int nx,
+                               int ny, float4* __restrict__ out) {
+    const size_t n = (size_t)(nx + 1) * (ny + 1);
+    for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (size_t)gridDim.x * blockDim.x) {
+        const int j = (int)(q / (nx + 1)), i = (int)(q - (size_t)j * (nx + 1));
+        const size_t row = (size_t)j * nx + i;
+        out[q] = make_float4(j < ny ? fx[q] : 0.f, i < nx ? fy[row] : 0.f, i < nx && j < ny ? dg[row] : 0.f, 0.f);
+    }
 }
 
 // One Chebyshev step, xout = xin + dnew with dnew = c1 din + c2 Dinv (b - (A - dI) xin); stages hold
@@ -310,14 +352,14 @@ __global__ void __launch_bounds__(kTmaThreads, kTmaMaxCtasPerSM)
 // p_new, and p_new . q per system; the stages hold z and p_old with their halos.  p_new is formed once
 // per halo point, in place over z in the stage, and the stencil then reads it from there.  The
 // direction buffers alternate by the parity in the Scal record, as in the grid kernel.
-template <int C>
+template <int C, bool VAR>
 __global__ void __launch_bounds__(kTmaThreads, kTmaMaxCtasPerSM)
     k_spmv_tma(const __grid_constant__ TmaMaps3 mp, TmaGeo g, float* pa, float* pb, float* __restrict__ q, Red red) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char* smem = aligned_ring(smem_raw);
     const int Kp = C * 4;
-    const size_t sb = stage_bytes(TK_SPMV, Kp);
+    const size_t sb = stage_bytes(VAR ? TK_SPMV_V : TK_SPMV, Kp);
     const int off = threadIdx.x * 4;
     const int par = red.scal->parity;
     const CUtensorMap* mold = par ? &mp.m[2] : &mp.m[1];
@@ -327,7 +369,7 @@ __global__ void __launch_bounds__(kTmaThreads, kTmaMaxCtasPerSM)
         beta[v] = red.scal->betaf[off + v];
         dsh[v] = red.scal->dshf[off + v];
     }
-    const unsigned tx_bytes = (unsigned)(2 * kHaloPts * Kp * 4);
+    const unsigned tx_bytes = (unsigned)(2 * kHaloPts * Kp * 4 + (VAR ? kHaloPts * 16 : 0));
     Accum<float> acc;
     tile_loop<true>(
         g.ntiles, g.stages, smem, sb, red.scal,
@@ -337,6 +379,7 @@ __global__ void __launch_bounds__(kTmaThreads, kTmaMaxCtasPerSM)
             mbar_expect_tx(bar, tx_bytes);
             tma_load_pt(st, &mp.m[0], g, x0 - 1, y0 - 1, bar);
             tma_load_pt(st + halo_bytes(Kp), mold, g, x0 - 1, y0 - 1, bar);
+            if (VAR) tma_load_2d(st + 2 * halo_bytes(Kp), &mp.w, (x0 - 1) * 2, y0 - 1, bar);
         },
         [&](unsigned char* st, int t) {
             int x0, y0;
@@ -360,7 +403,19 @@ __global__ void __launch_bounds__(kTmaThreads, kTmaMaxCtasPerSM)
                 if (gx >= g.nx || gy >= g.ny) continue;
                 const int hidx = ((ly + 1) * (kTX + 2) + lx + 1) * Kp + off;
                 float pc[4], Ax[4];
-                stencil_tile(g, hidx, [&](int h, float (&o)[4]) { ld4(Z + h, o); }, pc, Ax);
+                if constexpr (VAR) {
+                    const W5 w = tile_weights<kTX + 2>(reinterpret_cast<const float*>(st + 2 * halo_bytes(Kp)),
+                                                       (ly + 1) * (kTX + 2) + lx + 1);
+                    float l[4], r[4], dn[4], up[4];
+                    ld4(Z + hidx, pc);
+                    ld4(Z + hidx - Kp, l);
+                    ld4(Z + hidx + Kp, r);
+                    ld4(Z + hidx - (kTX + 2) * Kp, dn);
+                    ld4(Z + hidx + (kTX + 2) * Kp, up);
+                    for (int v = 0; v < 4; ++v) Ax[v] = apply5(w, pc[v], l[v], r[v], dn[v], up[v]);
+                } else {
+                    stencil_tile(g, hidx, [&](int h, float (&o)[4]) { ld4(Z + h, o); }, pc, Ax);
+                }
                 float qv[4];
                 for (int v = 0; v < 4; ++v) qv[v] = fmaf(-dsh[v], pc[v], Ax[v]);
                 const size_t gidx = ((size_t)gy * g.nx + gx) * Kp + off;
@@ -378,17 +433,18 @@ __global__ void __launch_bounds__(kTmaThreads, kTmaMaxCtasPerSM)
 // an axis also the last fine point).  x2 is computed, as k_pre2_tma does, on those points plus a
 // one-point halo (recomputed by neighbouring tiles, bit for bit the same), the residual on the fine
 // points the coarse tile's full weighting reads, and the weighted sums in the grid kernel's order.
-template <int C>
-__global__ void __launch_bounds__(kTmaThreads, kTmaMaxCtasPerSM)
+template <int C, bool VAR>
+__global__ void __launch_bounds__(kTmaThreads, VAR ? 2 : kTmaMaxCtasPerSM)
     k_pre2_restrict_tma(const __grid_constant__ TmaMaps3 mp, TmaGeo g, float* __restrict__ x2out,
                         float* __restrict__ bc, ChebStepT<float> cs0, ChebStepT<float> cs1, const float* __restrict__ dsh, Red none) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char* smem = aligned_ring(smem_raw);
     const int Kp = C * 4;
-    const size_t sb = stage_bytes(TK_PRE2R, Kp);
+    const size_t sb = stage_bytes(VAR ? TK_PRE2R_V : TK_PRE2R, Kp);
     float* X2s = reinterpret_cast<float*>(smem + g.stages * sb);
     float* Rs = reinterpret_cast<float*>(smem + g.stages * sb + vec_bytes(kE1X * kE1Y, Kp));
+    float* X1s = Rs + vec_bytes(kRX * kRY, Kp) / sizeof(float);  // VAR: the first iterate on b's box
     const int off = threadIdx.x * 4;
     float c20[4], c1[4], c2[4], d[4];
     for (int v = 0; v < 4; ++v) {
@@ -399,13 +455,14 @@ __global__ void __launch_bounds__(kTmaThreads, kTmaMaxCtasPerSM)
     }
     const float w1[3] = {0.25f, 0.5f, 0.25f};
     const float diag = g.wx + g.wx + g.wy + g.wy;
-    const unsigned tx_bytes = (unsigned)(kRsX * kRsY * Kp * 4);
+    const unsigned tx_bytes = (unsigned)(kRsX * kRsY * Kp * 4 + (VAR ? kRsX * kRsY * 16 : 0));
     tile_loop<true>(
         g.nctiles, g.stages, smem, sb, none.scal,
         [&](unsigned char* st, int t, uint64_t* bar) {
             const int cy = t / g.ncx, cx = t - cy * g.ncx;
             mbar_expect_tx(bar, tx_bytes);
             tma_load_pt(st, &mp.m[0], g, 2 * cx * kTXc - 2, 2 * cy * kTYc - 2, bar);
+            if (VAR) tma_load_2d(st + vec_bytes(kRsX * kRsY, Kp), &mp.w, (2 * cx * kTXc - 2) * 2, 2 * cy * kTYc - 2, bar);
         },
         [&](unsigned char* st, int t) {
             const int cy = t / g.ncx, cx = t - cy * g.ncx;
@@ -413,6 +470,17 @@ __global__ void __launch_bounds__(kTmaThreads, kTmaMaxCtasPerSM)
             const int ihi = X0 + kTXc >= g.nxc ? g.nx : 2 * X0 + 2 * kTXc;
             const int jhi = Y0 + kTYc >= g.nyc ? g.ny : 2 * Y0 + 2 * kTYc;
             const float* Bs = reinterpret_cast<const float*>(st);
+            const float* Ws = reinterpret_cast<const float*>(st + vec_bytes(kRsX * kRsY, Kp));
+            if constexpr (VAR) {  // the first iterate c2 Dinv b once per point (zero outside the grid, where the diagonal is)
+                for (int p = threadIdx.y; p < kRsX * kRsY; p += blockDim.y) {
+                    float v[4];
+                    ld4(Bs + p * Kp + off, v);
+                    const float dg = Ws[4 * p + 2];
+                    for (int q = 0; q < 4; ++q) v[q] = dg > 0.f ? jdiv(c20[q] * v[q], dg - d[q]) : 0.f;
+                    st4(X1s + p * Kp + off, v);
+                }
+                __syncthreads();
+            }
             // x2 on the owned fine points plus a one-point halo (zero outside the grid)
             for (int p = threadIdx.y; p < kE1X * kE1Y; p += blockDim.y) {
                 const int ey = p / kE1X, ex = p - ey * kE1X;
@@ -423,23 +491,40 @@ __global__ void __launch_bounds__(kTmaThreads, kTmaMaxCtasPerSM)
                     const int sy = kRsX * Kp;
                     float xc[4], acc[4], n[4], bv[4];
                     auto x1 = [&](int h, float (&o)[4]) {
-                        ld4(Bs + h, o);
-                        for (int v = 0; v < 4; ++v) o[v] *= c20[v];
+                        if constexpr (VAR) {
+                            ld4(X1s + h, o);
+                        } else {
+                            ld4(Bs + h, o);
+                            for (int v = 0; v < 4; ++v) o[v] *= c20[v];
+                        }
                     };
+                    float dg = 0.f;
                     x1(bidx, xc);
-                    for (int v = 0; v < 4; ++v) acc[v] = diag * xc[v];
-                    x1(bidx - Kp, n);
-                    for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wx, n[v], acc[v]);
-                    x1(bidx + Kp, n);
-                    for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wx, n[v], acc[v]);
-                    x1(bidx - sy, n);
-                    for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wy, n[v], acc[v]);
-                    x1(bidx + sy, n);
-                    for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wy, n[v], acc[v]);
+                    if constexpr (VAR) {
+                        const W5 w = tile_weights<kRsX>(Ws, (ey + 1) * kRsX + ex + 1);
+                        float l[4], r[4], dn[4];
+                        dg = w.dg;
+                        x1(bidx - Kp, l);
+                        x1(bidx + Kp, r);
+                        x1(bidx - sy, dn);
+                        x1(bidx + sy, n);
+                        for (int v = 0; v < 4; ++v) acc[v] = apply5(w, xc[v], l[v], r[v], dn[v], n[v]);
+                    } else {
+                        for (int v = 0; v < 4; ++v) acc[v] = diag * xc[v];
+                        x1(bidx - Kp, n);
+                        for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wx, n[v], acc[v]);
+                        x1(bidx + Kp, n);
+                        for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wx, n[v], acc[v]);
+                        x1(bidx - sy, n);
+                        for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wy, n[v], acc[v]);
+                        x1(bidx + sy, n);
+                        for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wy, n[v], acc[v]);
+                    }
                     ld4(Bs + bidx, bv);
                     for (int v = 0; v < 4; ++v) {
                         const float res = bv[v] - fmaf(-d[v], xc[v], acc[v]);
-                        const float gg = c2[v] * res;
+                        float gg = c2[v] * res;
+                        if (VAR) gg = jdiv(gg, dg - d[v]);
                         const float dv = fmaf(c1[v], xc[v], gg);
                         x2[v] = xc[v] + dv;
                     }
@@ -456,15 +541,25 @@ __global__ void __launch_bounds__(kTmaThreads, kTmaMaxCtasPerSM)
                 const int sy = kE1X * Kp;
                 float xc[4], acc[4], n[4], bv[4], r[4];
                 ld4(X2s + eidx, xc);
-                for (int v = 0; v < 4; ++v) acc[v] = diag * xc[v];
-                ld4(X2s + eidx - Kp, n);
-                for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wx, n[v], acc[v]);
-                ld4(X2s + eidx + Kp, n);
-                for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wx, n[v], acc[v]);
-                ld4(X2s + eidx - sy, n);
-                for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wy, n[v], acc[v]);
-                ld4(X2s + eidx + sy, n);
-                for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wy, n[v], acc[v]);
+                if constexpr (VAR) {
+                    const W5 w = tile_weights<kRsX>(Ws, (ry + 2) * kRsX + rx + 2);
+                    float l[4], r2[4], dn[4];
+                    ld4(X2s + eidx - Kp, l);
+                    ld4(X2s + eidx + Kp, r2);
+                    ld4(X2s + eidx - sy, dn);
+                    ld4(X2s + eidx + sy, n);
+                    for (int v = 0; v < 4; ++v) acc[v] = apply5(w, xc[v], l[v], r2[v], dn[v], n[v]);
+                } else {
+                    for (int v = 0; v < 4; ++v) acc[v] = diag * xc[v];
+                    ld4(X2s + eidx - Kp, n);
+                    for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wx, n[v], acc[v]);
+                    ld4(X2s + eidx + Kp, n);
+                    for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wx, n[v], acc[v]);
+                    ld4(X2s + eidx - sy, n);
+                    for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wy, n[v], acc[v]);
+                    ld4(X2s + eidx + sy, n);
+                    for (int v = 0; v < 4; ++v) acc[v] = fmaf(-g.wy, n[v], acc[v]);
+                }
                 ld4(Bs + ((ry + 2) * kRsX + rx + 2) * Kp + off, bv);
                 for (int v = 0; v < 4; ++v) r[v] = bv[v] - fmaf(-d[v], xc[v], acc[v]);
                 st4(Rs + p * Kp + off, r);
@@ -585,7 +680,7 @@ __global__ void __launch_bounds__(kTmaThreads, kTmaMaxCtasPerSM)
 // is k_prolong_cheb_tma's and k_cheb_tma's arithmetic, operation for operation; points outside the grid
 // hold zero (Dirichlet).  Traffic per tile: x, ec, b in, xout out, against x, ec, b in and x1, d1 out,
 // then x1, d1, b in and xout out for the two-kernel form.
-template <int C>
+template <int C, bool VAR>
 __global__ void __launch_bounds__(kTmaThreads, kPost2CtasPerSM)
     k_post2_tma(const __grid_constant__ TmaMaps3 mp, TmaGeo g, float* __restrict__ xout, ChebStepT<float> cs0,
                 ChebStepT<float> cs1, const float* __restrict__ dsh, Red red) {
@@ -593,7 +688,7 @@ __global__ void __launch_bounds__(kTmaThreads, kPost2CtasPerSM)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char* smem = aligned_ring(smem_raw);
     const int Kp = C * 4;
-    const size_t sb = stage_bytes(TK_POST2, Kp);
+    const size_t sb = stage_bytes(VAR ? TK_POST2_V : TK_POST2, Kp);
     float* X1 = reinterpret_cast<float*>(smem + g.stages * sb);
     float* D1 = reinterpret_cast<float*>(smem + g.stages * sb + halo_bytes(Kp));
     const int off = threadIdx.x * 4;
@@ -606,7 +701,8 @@ __global__ void __launch_bounds__(kTmaThreads, kPost2CtasPerSM)
     }
     const size_t e_ofs = vec_bytes(kH2X * kH2Y, Kp);
     const size_t b_ofs = e_ofs + vec_bytes(kCp2X * kCp2Y, Kp);
-    const unsigned tx_bytes = (unsigned)((kH2X * kH2Y + kCp2X * kCp2Y + kHaloPts) * Kp * 4);
+    const size_t w_ofs = b_ofs + halo_bytes(Kp);
+    const unsigned tx_bytes = (unsigned)((kH2X * kH2Y + kCp2X * kCp2Y + kHaloPts) * Kp * 4 + (VAR ? kH2X * kH2Y * 16 : 0));
     const bool dot = red.op != RED_NONE;
     Accum<float> acc;
     tile_loop<true>(
@@ -618,11 +714,13 @@ __global__ void __launch_bounds__(kTmaThreads, kPost2CtasPerSM)
             tma_load_pt(st, &mp.m[0], g, x0 - 2, y0 - 2, bar);
             tma_load_pt(st + e_ofs, &mp.m[1], g, x0 / 2 - 2, y0 / 2 - 2, bar);
             tma_load_pt(st + b_ofs, &mp.m[2], g, x0 - 1, y0 - 1, bar);
+            if (VAR) tma_load_2d(st + w_ofs, &mp.w, (x0 - 2) * 2, y0 - 2, bar);
         },
         [&](unsigned char* st, int t) {
             int x0, y0;
             tile_origin(g, t, x0, y0);
             float* X = reinterpret_cast<float*>(st);
+            const float* Ws = reinterpret_cast<const float*>(st + w_ofs);
             const float* E = reinterpret_cast<const float*>(st + e_ofs);
             const float* B = reinterpret_cast<const float*>(st + b_ofs);
             // (1) xin = x + P ec on the two-point halo region, by 2 x 2 blocks of fine points: the block
@@ -695,17 +793,15 @@ __global__ void __launch_bounds__(kTmaThreads, kPost2CtasPerSM)
                     const float(&xd)[4] = j ? dn : m1;
                     float xo[4] = {0.f, 0.f, 0.f, 0.f};
                     if (in_x && fj >= 0 && fj < g.ny) {
-                        const float diag = g.wx + g.wx + g.wy + g.wy;
+                        const W5 w = VAR ? tile_weights<kH2X>(Ws, (hy + 1) * kH2X + hx + 1)
+                                         : W5{g.wx, g.wx, g.wy, g.wy, g.wx + g.wx + g.wy + g.wy};
                         float bv[4], dv[4];
                         ld4(B + (hy * (kTX + 2) + hx) * Kp + off, bv);
                         for (int v = 0; v < 4; ++v) {
-                            float a = diag * xc[v];
-                            a = fmaf(-g.wx, xl[v], a);
-                            a = fmaf(-g.wx, xr[v], a);
-                            a = fmaf(-g.wy, xu[v], a);
-                            a = fmaf(-g.wy, xd[v], a);
+                            const float a = apply5(w, xc[v], xl[v], xr[v], xu[v], xd[v]);
                             const float res = bv[v] - fmaf(-d[v], xc[v], a);
-                            const float gg = c20[v] * res;
+                            float gg = c20[v] * res;
+                            if (VAR) gg = jdiv(gg, w.dg - d[v]);
                             dv[v] = fmaf(0.f, 0.f, gg);
                             xo[v] = xc[v] + dv[v];
                         }
@@ -742,18 +838,16 @@ __global__ void __launch_bounds__(kTmaThreads, kPost2CtasPerSM)
                     const float(&xr)[4] = j ? r1 : r0;
                     const float(&xu)[4] = j ? m0 : up;
                     const float(&xd)[4] = j ? dn : m1;
-                    const float diag = g.wx + g.wx + g.wy + g.wy;
+                    const W5 w = VAR ? tile_weights<kH2X>(Ws, (ly0 + j + 2) * kH2X + lx + 2)
+                                     : W5{g.wx, g.wx, g.wy, g.wy, g.wx + g.wx + g.wy + g.wy};
                     float bv[4], dv[4], xo[4];
                     ld4(B + c0 + (1 + j) * sy, bv);
                     ld4(D1 + ((ly0 + j) * kTX + lx) * Kp + off, dv);
                     for (int v = 0; v < 4; ++v) {
-                        float a = diag * xc[v];
-                        a = fmaf(-g.wx, xl[v], a);
-                        a = fmaf(-g.wx, xr[v], a);
-                        a = fmaf(-g.wy, xu[v], a);
-                        a = fmaf(-g.wy, xd[v], a);
+                        const float a = apply5(w, xc[v], xl[v], xr[v], xu[v], xd[v]);
                         const float res = bv[v] - fmaf(-d[v], xc[v], a);
-                        const float gg = c21[v] * res;
+                        float gg = c21[v] * res;
+                        if (VAR) gg = jdiv(gg, w.dg - d[v]);
                         dv[v] = fmaf(c11[v], dv[v], gg);
                         xo[v] = xc[v] + dv[v];
                     }
@@ -839,17 +933,24 @@ cudaError_t prepare_c() {
         return e;
     if ((e = cudaFuncSetAttribute(k_pre2_tma<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) != cudaSuccess)
         return e;
-    if ((e = cudaFuncSetAttribute(k_pre2_restrict_tma<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) !=
+    if ((e = cudaFuncSetAttribute(k_pre2_restrict_tma<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) !=
         cudaSuccess)
+        return e;
+    if ((e = cudaFuncSetAttribute(k_pre2_restrict_tma<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) !=
+        cudaSuccess)
+        return e;
+    if ((e = cudaFuncSetAttribute(k_post2_tma<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) != cudaSuccess)
+        return e;
+    if ((e = cudaFuncSetAttribute(k_spmv_tma<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) != cudaSuccess)
         return e;
     if ((e = cudaFuncSetAttribute(k_prolong_cheb_tma<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) !=
         cudaSuccess)
         return e;
-    if ((e = cudaFuncSetAttribute(k_post2_tma<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(k_post2_tma<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) != cudaSuccess)
         return e;
     if ((e = cudaFuncSetAttribute(k_cg_update_tma<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) != cudaSuccess)
         return e;
-    return cudaFuncSetAttribute(k_spmv_tma<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+    return cudaFuncSetAttribute(k_spmv_tma<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
 }
 
 template <class K, class... Args>
@@ -947,6 +1048,28 @@ cudaError_t tma_encode(CUtensorMap* m, const float* base, int Kp, int nx, int ny
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+cudaError_t tma_pack_weights(const Lev& L, float* out, cudaStream_t s) {
+    const size_t n = (size_t)(L.nx + 1) * (L.ny + 1);
+    k_pack_weights<<<(unsigned)std::min<size_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(
+        (const float*)L.fx, (const float*)L.fy, (const float*)L.dg, L.nx, L.ny, reinterpret_cast<float4*>(out));
+    return cudaGetLastError();
+}
+
+cudaError_t tma_encode_weights(CUtensorMap* m, const void* base, int nx, int ny, int boxkind) {
+    int bx = 0, by = 0;
+    tma_box_dims(boxkind, &bx, &by);
+    const PFN_cuTensorMapEncodeTiled_v12000 encode = encode_fn();
+    if (!encode) return cudaErrorNotSupported;
+    const cuuint64_t dims[2] = {(cuuint64_t)(nx + 1) * 2, (cuuint64_t)(ny + 1)};
+    const cuuint64_t strides[1] = {(cuuint64_t)(nx + 1) * 16};
+    const cuuint32_t box[2] = {(cuuint32_t)(bx * 2), (cuuint32_t)by};
+    const cuuint32_t estr[2] = {1, 1};
+    const CUresult r = encode(m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<void*>(base), dims, strides, box, estr,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 cudaError_t tma_prepare(int Kp) {
     switch (Kp) {
         case 4: return prepare_c<1>();
@@ -960,7 +1083,7 @@ cudaError_t tma_prepare(int Kp) {
 // Ring depth of a launch: the requested depth, reduced until the ring fits one CTA (at least 1).
 int ring_stages(const TmaGeo& g, int kind) {
     int S = g.stages < 1 ? kTmaStages : (g.stages > kTmaMaxStages ? kTmaMaxStages : g.stages);
-    if (kind == TK_POST2 && kPost2Stages > 0) S = kPost2Stages;
+    if ((kind == TK_POST2 || kind == TK_POST2_V) && kPost2Stages > 0) S = kPost2Stages;
     while (S > 1 && dyn_smem(kind, g.Kp, S) + kRingSlack > kSmemPerCTA) --S;
     return S;
 }
@@ -970,9 +1093,11 @@ int ring_stages(const TmaGeo& g, int kind) {
 int tma_blocks(const TmaGeo& g, int Kp, int nsm, int kind, int S) {
     const size_t smem = dyn_smem(kind, Kp, S) + kRingSlack + kSmemReserved + 64;  // + static
     int per_sm = (int)(kSmemPerSM / smem);
-    const int cap = kind == TK_POST2 ? kPost2CtasPerSM : kTmaMaxCtasPerSM;  // the launch bounds' registers
+    const int cap = kind == TK_POST2 || kind == TK_POST2_V ? kPost2CtasPerSM
+                    : kind == TK_PRE2R_V                   ? 2
+                                                           : kTmaMaxCtasPerSM;  // the launch bounds' registers
     per_sm = per_sm < 1 ? 1 : (per_sm > cap ? cap : per_sm);
-    const int nt = kind == TK_PRE2R ? g.nctiles : g.ntiles;
+    const int nt = kind == TK_PRE2R || kind == TK_PRE2R_V ? g.nctiles : g.ntiles;
     return nt < nsm * per_sm ? nt : nsm * per_sm;
 }
 
@@ -1025,13 +1150,20 @@ cudaError_t tma_pre2(const TmaGeo& g, int nsm, const CUtensorMap& mb_halo, float
                                         none))
 }
 
-cudaError_t tma_pre2_restrict(const TmaGeo& g, int nsm, const CUtensorMap& mb_rsrc, float* x2out, float* bc,
-                              ChebStepT<float> cs0, ChebStepT<float> cs1, const float* dsh, const Red& none, cudaStream_t s) {
+cudaError_t tma_pre2_restrict(const TmaGeo& g, int nsm, const CUtensorMap& mb_rsrc, const CUtensorMap* mw, float* x2out,
+                              float* bc, ChebStepT<float> cs0, ChebStepT<float> cs1, const float* dsh, const Red& none,
+                              cudaStream_t s) {
     TmaMaps3 mp;
     mp.m[0] = mp.m[1] = mp.m[2] = mb_rsrc;
+    if (mw) {
+        mp.w = *mw;
+        const Shape sh = shape_of(g, nsm, TK_PRE2R_V);
+        BURA_TMA_C(g.Kp, return launch_tile(k_pre2_restrict_tma<C, true>, sh.blocks, sh.threads, C, sh.smem, s, mp, sh.g, x2out,
+                                            bc, cs0, cs1, dsh, none))
+    }
     const Shape sh = shape_of(g, nsm, TK_PRE2R);
-    BURA_TMA_C(g.Kp, return launch_tile(k_pre2_restrict_tma<C>, sh.blocks, sh.threads, C, sh.smem, s, mp, sh.g, x2out, bc, cs0,
-                                        cs1, dsh, none))
+    BURA_TMA_C(g.Kp, return launch_tile(k_pre2_restrict_tma<C, false>, sh.blocks, sh.threads, C, sh.smem, s, mp, sh.g, x2out, bc,
+                                        cs0, cs1, dsh, none))
 }
 
 cudaError_t tma_prolong_cheb(const TmaGeo& g, int nsm, const CUtensorMap& mx_halo, const CUtensorMap& mec_cpro,
@@ -1047,25 +1179,37 @@ cudaError_t tma_prolong_cheb(const TmaGeo& g, int nsm, const CUtensorMap& mx_hal
 }
 
 cudaError_t tma_post2(const TmaGeo& g, int nsm, const CUtensorMap& mx_halo2, const CUtensorMap& mec_cpro2,
-                      const CUtensorMap& mb_halo, float* xout, ChebStepT<float> cs0, ChebStepT<float> cs1,
-                      const float* dsh, const Red& red, cudaStream_t s) {
+                      const CUtensorMap& mb_halo, const CUtensorMap* mw, float* xout, ChebStepT<float> cs0,
+                      ChebStepT<float> cs1, const float* dsh, const Red& red, cudaStream_t s) {
     TmaMaps3 mp;
     mp.m[0] = mx_halo2;
     mp.m[1] = mec_cpro2;
     mp.m[2] = mb_halo;
+    if (mw) {
+        mp.w = *mw;
+        const Shape sh = shape_of(g, nsm, TK_POST2_V);
+        BURA_TMA_C(g.Kp, return launch_tile(k_post2_tma<C, true>, sh.blocks, sh.threads, C, sh.smem, s, mp, sh.g, xout, cs0,
+                                            cs1, dsh, red))
+    }
     const Shape sh = shape_of(g, nsm, TK_POST2);
-    BURA_TMA_C(g.Kp, return launch_tile(k_post2_tma<C>, sh.blocks, sh.threads, C, sh.smem, s, mp, sh.g, xout, cs0, cs1,
+    BURA_TMA_C(g.Kp, return launch_tile(k_post2_tma<C, false>, sh.blocks, sh.threads, C, sh.smem, s, mp, sh.g, xout, cs0, cs1,
                                         dsh, red))
 }
 
 cudaError_t tma_spmv_p(const TmaGeo& g, int nsm, const CUtensorMap& mz, const CUtensorMap& mpa,
-                       const CUtensorMap& mpb, float* pa, float* pb, float* q, const Red& red, cudaStream_t s) {
+                       const CUtensorMap& mpb, const CUtensorMap* mw, float* pa, float* pb, float* q, const Red& red,
+                       cudaStream_t s) {
     TmaMaps3 mp;
     mp.m[0] = mz;
     mp.m[1] = mpa;
     mp.m[2] = mpb;
+    if (mw) {
+        mp.w = *mw;
+        const Shape sh = shape_of(g, nsm, TK_SPMV_V);
+        BURA_TMA_C(g.Kp, return launch_tile(k_spmv_tma<C, true>, sh.blocks, sh.threads, C, sh.smem, s, mp, sh.g, pa, pb, q, red))
+    }
     const Shape sh = shape_of(g, nsm, TK_SPMV);
-    BURA_TMA_C(g.Kp, return launch_tile(k_spmv_tma<C>, sh.blocks, sh.threads, C, sh.smem, s, mp, sh.g, pa, pb, q, red))
+    BURA_TMA_C(g.Kp, return launch_tile(k_spmv_tma<C, false>, sh.blocks, sh.threads, C, sh.smem, s, mp, sh.g, pa, pb, q, red))
 }
 
 bool tma_cg_fits(int Kp) { return dyn_smem(TK_CG, Kp, 2) + kRingSlack <= kSmemPerCTA; }

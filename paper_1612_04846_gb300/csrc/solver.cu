@@ -126,6 +126,8 @@ struct Work {
         TmaGeo geo{};
         struct Ent { int box; const void* buf; CUtensorMap map; };
         std::vector<Ent> maps;
+        bool var = false;  // variable coefficients: the packed weights, boxed as each sweep's stencil input
+        CUtensorMap w_rsrc, w_halo2, w_halo;
         const CUtensorMap* find(int box, const void* buf) const {
             for (const auto& e : maps)
                 if (e.box == box && e.buf == buf) return &e.map;
@@ -541,18 +543,32 @@ int coarse_degree_auto(const HostLevel& h, double d0) {
     return std::max(2, std::min(m, 400));
 }
 
-// Tensor maps for the TMA-staged sweeps: FP32, 2-D, constant coefficients, levels that the grid
+// The packed weights of a 2-D variable-coefficient level for the TMA-staged sweeps (from the stored ones, on the device:
+// packing on the host made a 511^2 plan's setup 0.8 ms longer, an eighth of it), and their maps.
+int pack_weights2(bura_plan* p, const Lev& L, CUtensorMap& rsrc, CUtensorMap& halo2, CUtensorMap& halo) {
+    float* d = nullptr;
+    CA(dalloc(p, &d, (size_t)(L.nx + 1) * (L.ny + 1) * 4 * sizeof(float)));
+    CK(tma_pack_weights(L, d, nullptr));
+    CK(tma_encode_weights(&rsrc, d, L.nx, L.ny, TB_RSRC));
+    CK(tma_encode_weights(&halo2, d, L.nx, L.ny, TB_HALO2));
+    CK(tma_encode_weights(&halo, d, L.nx, L.ny, TB_HALO));
+    return BURA_OK;
+}
+
+// Tensor maps for the TMA-staged sweeps: FP32, 2-D, levels that the grid
 // kernels would run (not the coarse kernel's) with at least one tile per SM.
 template <class T>
 int build_tma(bura_plan* p, Work<T>& w) {
     const int nlev = (int)p->hl.size();
     w.tma.assign(nlev, typename Work<T>::TmaLev());
-    if (sizeof(T) != 4 || p->dim != 2 || p->var || p->opt.sweeps == BURA_SWEEP_GRID || !tma_supported(w.Kp))
-        return BURA_OK;
+    if (sizeof(T) != 4 || p->dim != 2 || p->opt.sweeps == BURA_SWEEP_GRID || !tma_supported(w.Kp)) return BURA_OK;
+    // variable coefficients: the fused sweeps only (degree 2, FP32 weights); other options keep the grid sweeps
+    if (p->var && (p->opt.smoother_degree != 2 || p->opt.post_smooth_split != 0 || p->opt.smoother_bf16)) return BURA_OK;
     bool any = false;
     for (int l = 0; l < nlev; ++l) {
         if (w.lc >= 0 && l >= w.lc) break;
         const bool has_coarse = l + 1 < nlev;
+        if (p->var && !has_coarse) break;
         TmaGeo g = tma_geo(w.L[l], has_coarse ? &w.L[l + 1] : nullptr, w.Kp);
         if (p->opt.tma_stages > 0) g.stages = p->opt.tma_stages;
         // every grid level: even with fewer tiles than SMs the fused 3-launch V-cycle step beats the
@@ -595,6 +611,8 @@ int build_tma(bura_plan* p, Work<T>& w) {
             t = typename Work<T>::TmaLev();
             break;
         }
+        if (p->var) CA(pack_weights2(p, w.L[l], t.w_rsrc, t.w_halo2, t.w_halo));
+        t.var = p->var;
         t.on = true;
         any = true;
     }
@@ -1329,8 +1347,8 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
     const CUtensorMap* m_xa = tl.on ? tl.find(TB_HALO, A) : nullptr;
     const CUtensorMap* m_bp = tl.on ? tl.find(TB_PLAIN, b) : nullptr;
     if (m_rsrc && m_ca && m_cb && m_xa && m_bp) {
-        traced(p, K_PRE2R, f32, fine, vbytes<T>(p, l, 2.0, false) + vbytes<T>(p, l + 1, 1.0, false), s, [&] {
-            (void)tma_pre2_restrict(tl.geo, p->nsm, *m_rsrc, reinterpret_cast<float*>(A),
+        traced(p, K_PRE2R, f32, fine, vbytes<T>(p, l, 2.0, tl.var) + vbytes<T>(p, l + 1, 1.0, false), s, [&] {
+            (void)tma_pre2_restrict(tl.geo, p->nsm, *m_rsrc, tl.var ? &tl.w_rsrc : nullptr, reinterpret_cast<float*>(A),
                                     reinterpret_cast<float*>(w.b[l + 1]), f32_step(step_of(w, l, 0)),
                                     f32_step(step_of(w, l, 1)), f32_ptr(w.dsh), none, s);
         });
@@ -1359,7 +1377,7 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
         if (pss == 0 && mec2 && m_xa2 && m_bh) {
             const Red& red = rz_fused ? beta : none;
             traced(p, K_POST2, f32, fine, vbytes<T>(p, l, 3.0, false) + vbytes<T>(p, l + 1, 1.0, false), s, [&] {
-                (void)tma_post2(tl.geo, p->nsm, *m_xa2, *mec2, *m_bh, reinterpret_cast<float*>(B),
+                (void)tma_post2(tl.geo, p->nsm, *m_xa2, *mec2, *m_bh, tl.var ? &tl.w_halo2 : nullptr, reinterpret_cast<float*>(B),
                                 f32_step(step_of(w, l, 0, false)), f32_step(step_of(w, l, 1)), f32_ptr(w.dsh), red, s);
             });
             if (rz_fused) red_finish(p, beta, w.Kp, f32, s);
@@ -1506,7 +1524,7 @@ int pcg_body(bura_plan* p, Work<T>& w, unsigned long long cond, cudaStream_t s) 
         const CUtensorMap* ma = tl.on ? tl.find(TB_HALO, w.pa) : nullptr;
         const CUtensorMap* mbb = tl.on ? tl.find(TB_HALO, w.pb) : nullptr;
         if (mz && ma && mbb)
-            (void)tma_spmv_p(tl.geo, p->nsm, *mz, *ma, *mbb, reinterpret_cast<float*>(w.pa),
+            (void)tma_spmv_p(tl.geo, p->nsm, *mz, *ma, *mbb, tl.var ? &tl.w_halo : nullptr, reinterpret_cast<float*>(w.pa),
                              reinterpret_cast<float*>(w.pb), reinterpret_cast<float*>(w.q), ralpha, s);
         else if (s3)
             (void)sweep3_spmv(s3l.geo, s3l.at(S3B_HALO, z), s3l.at(S3B_HALO, w.pa), s3l.at(S3B_HALO, w.pb),

@@ -175,6 +175,7 @@ __device__ __forceinline__ void tma_load_pt(void* dst, const CUtensorMap* map, c
 
 struct TmaMaps3 {
     CUtensorMap m[3];
+    CUtensorMap w;  // variable coefficients: the packed weights
 };
 
 struct TmaMaps5 {
@@ -188,6 +189,13 @@ TmaGeo tma_geo(const Lev& L, const Lev* Lc, int Kp);
 bool tma_flat(int Kp);
 // Tensor map of an [ny][nx][Kp] float vector with a box of kind TmaBox.
 cudaError_t tma_encode(CUtensorMap* m, const float* base, int Kp, int nx, int ny, int box);
+// Packs a variable-coefficient level's FP32 weights: a float4 per point of the grid extended by one point along each axis
+// (the faces below the point along x and y, its diagonal, 0; zeros where a face or a point does not exist).
+cudaError_t tma_pack_weights(const Lev& L, float* out, cudaStream_t s);
+// Map of the packed weights of a variable-coefficient level, [ny + 1][nx + 1] float4 (the faces below a point along x and
+// y, its diagonal, 0), with the box of `boxkind`.  The sweeps that take one (mw, null for constant coefficients) need it
+// with the box of their stencil's input: TB_RSRC, TB_HALO2, TB_HALO.
+cudaError_t tma_encode_weights(CUtensorMap* m, const void* base, int nx, int ny, int boxkind);
 cudaError_t tma_prepare(int Kp);
 cudaError_t tma_cheb_step(const TmaGeo& g, int nsm, const CUtensorMap& mx, const CUtensorMap* md, const CUtensorMap& mb,
                           float* xout, float* dout, ChebStepT<float> cs, const float* dsh, const Red& red, cudaStream_t s);
@@ -195,8 +203,9 @@ cudaError_t tma_pre2(const TmaGeo& g, int nsm, const CUtensorMap& mb_halo, float
                      ChebStepT<float> cs1, const float* dsh, const Red& none, cudaStream_t s);
 // pre2 fused with the residual restriction: x2 = two Chebyshev steps from zero (written to x2out) and
 // bc = R (b - (A - dI) x2) on the coarse level; one tile = kTXc x kTYc coarse points.
-cudaError_t tma_pre2_restrict(const TmaGeo& g, int nsm, const CUtensorMap& mb_rsrc, float* x2out, float* bc,
-                              ChebStepT<float> cs0, ChebStepT<float> cs1, const float* dsh, const Red& none, cudaStream_t s);
+cudaError_t tma_pre2_restrict(const TmaGeo& g, int nsm, const CUtensorMap& mb_rsrc, const CUtensorMap* mw, float* x2out,
+                              float* bc, ChebStepT<float> cs0, ChebStepT<float> cs1, const float* dsh, const Red& none,
+                              cudaStream_t s);
 // First post-smoothing step on x + P ec (prolongation fused): xout = xin + dnew, dout = dnew with
 // dnew = c2 Dinv (b - (A - dI) xin), xin = x + P ec never stored.
 cudaError_t tma_prolong_cheb(const TmaGeo& g, int nsm, const CUtensorMap& mx_halo, const CUtensorMap& mec_cpro,
@@ -208,8 +217,8 @@ cudaError_t tma_prolong_cheb(const TmaGeo& g, int nsm, const CUtensorMap& mx_hal
 // xout is stored.  x is read through a TB_HALO2 map, ec through a TB_CPRO2 map of the coarse level, b
 // through a TB_HALO map.
 cudaError_t tma_post2(const TmaGeo& g, int nsm, const CUtensorMap& mx_halo2, const CUtensorMap& mec_cpro2,
-                      const CUtensorMap& mb_halo, float* xout, ChebStepT<float> cs0, ChebStepT<float> cs1,
-                      const float* dsh, const Red& red, cudaStream_t s);
+                      const CUtensorMap& mb_halo, const CUtensorMap* mw, float* xout, ChebStepT<float> cs0,
+                      ChebStepT<float> cs1, const float* dsh, const Red& red, cudaStream_t s);
 // CG update x += alpha p, r -= alpha q with r.r (RED_CONV) from TMA-staged tiles of x, r, p, q (pointwise);
 // the direction is pa or pb by the Scal parity, as in the grid kernel.  False from tma_cg_fits when the
 // ring of at least two stages does not fit.
@@ -218,7 +227,8 @@ cudaError_t tma_cg_update(const TmaGeo& g, int nsm, const CUtensorMap& mx, const
                           const CUtensorMap& mpa, const CUtensorMap& mpb, const CUtensorMap& mq, float* x, float* r,
                           const Red& red, cudaStream_t s);
 cudaError_t tma_spmv_p(const TmaGeo& g, int nsm, const CUtensorMap& mz, const CUtensorMap& mpa,
-                       const CUtensorMap& mpb, float* pa, float* pb, float* q, const Red& red, cudaStream_t s);
+                       const CUtensorMap& mpb, const CUtensorMap* mw, float* pa, float* pb, float* q, const Red& red,
+                       cudaStream_t s);
 
 // Tensor map of ny x nz rows of `row` eight-byte elements (a row a multiple of 16 bytes), box bx x by elements and rows
 // of one plane; zero fill outside.
