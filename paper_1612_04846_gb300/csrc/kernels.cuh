@@ -127,7 +127,9 @@ struct Red {
 // The final step of a deferred reduction: one CTA of kRedFinishThreads sums the producer's block
 // partials in block order and applies op; launched right after the producer on the same stream.
 constexpr int kRedFinishThreads = 256;
-void launch_red_finish(const Red& red, int Kp, cudaStream_t s);
+constexpr int kRedFinishThreads32 = 512;  // FP32 data, whose partials are pairs: all of 8 systems x 1280 blocks in flight
+constexpr int kRedFinBatch32 = 20;
+void launch_red_finish(const Red& red, int Kp, bool f32, cudaStream_t s);
 
 // One level of the single-CTA coarse V-cycle: its vectors live in the CTA's shared memory at the
 // given byte offsets.  c1/c2 hold deg rows of Kp Chebyshev coefficients (global memory).

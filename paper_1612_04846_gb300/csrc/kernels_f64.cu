@@ -173,31 +173,67 @@ void launch_norm2(long long N, const double* f, const Red& red, int nsm, cudaStr
 // Final step of a deferred grid reduction (Red::defer): the producer, the previous kernel on the
 // stream, has completed when griddepcontrol.wait returns, so its partials are visible without fences.
 // The CG state record is loaded into shared memory together with the partials (one L2 round trip for
-// both), updated there and written back whole; no other kernel touches it meanwhile.
-__global__ void __launch_bounds__(kRedFinishThreads) k_red_finish(Red red, int Kp) {
-    __shared__ double sm[kRedFinishThreads];
+// both), updated there and written back whole; no other kernel touches it meanwhile.  F32: the partials are pairs, summed
+// by one thread per (system, group of blocks), then one warp per system; 1216 partials of 8 systems in FP64 on one SM
+// were bound by its FP64 pipe.
+template <bool F32>
+__global__ void __launch_bounds__(F32 ? kRedFinishThreads32 : kRedFinishThreads) k_red_finish(Red red, int Kp) {
+    constexpr int kThreads = F32 ? kRedFinishThreads32 : kRedFinishThreads;
+    __shared__ double sm[kThreads];
     __shared__ Scal sc;
     constexpr int kWords = (int)(sizeof(Scal) / sizeof(unsigned));
-    static_assert(sizeof(Scal) % sizeof(unsigned) == 0 && kWords <= 2 * kRedFinishThreads, "Scal copy");
+    static_assert(sizeof(Scal) % sizeof(unsigned) == 0 && kWords <= 2 * kThreads, "Scal copy");
     pdl_trigger();  // the next kernel may start its prologue; it waits for this grid to complete
     pdl_wait();
     const int tid = threadIdx.x;
     const unsigned* gs = reinterpret_cast<const unsigned*>(red.scal);
     const unsigned w0 = tid < kWords ? __ldcg(gs + tid) : 0u;
-    const unsigned w1 = tid + kRedFinishThreads < kWords ? __ldcg(gs + tid + kRedFinishThreads) : 0u;
-    const double part = red_thread_sum(red.partial, (int)__ldcg(red.nblk), Kp);
+    const unsigned w1 = tid + kThreads < kWords ? __ldcg(gs + tid + kThreads) : 0u;
+    const int nblk = (int)__ldcg(red.nblk);
     unsigned* ss = reinterpret_cast<unsigned*>(&sc);
     if (tid < kWords) ss[tid] = w0;
-    if (tid + kRedFinishThreads < kWords) ss[tid + kRedFinishThreads] = w1;
-    red_apply(red, &sc, part, Kp, sm);  // its first barrier publishes the copy
+    if (tid + kThreads < kWords) ss[tid + kThreads] = w1;
+    if constexpr (F32) {
+        const int G = kThreads / Kp, s = tid % Kp, g = tid / Kp;
+        const float2* fin = reinterpret_cast<const float2*>(red.partial);
+        Df* sd = reinterpret_cast<Df*>(sm);
+        if (g < G) {
+            DfSum part;
+            for (int b0 = g; b0 < nblk; b0 += kRedFinBatch32 * G) {
+                float2 v[kRedFinBatch32];
+#pragma unroll
+                for (int j = 0; j < kRedFinBatch32; ++j) {
+                    const int b = b0 + j * G;
+                    v[j] = b < nblk ? __ldcg(fin + (size_t)b * Kp + s) : make_float2(0.f, 0.f);
+                }
+#pragma unroll
+                for (int j = 0; j < kRedFinBatch32; ++j) part.add(Df{v[j].x, v[j].y});
+            }
+            sd[tid] = part.get();
+        }
+        __syncthreads();
+        __shared__ Df total[KMAXP];
+        const int lane = tid & 31;
+        for (int q = tid >> 5; q < Kp; q += kThreads / 32) {
+            Df t = {0.f, 0.f};
+            for (int h = lane; h < G; h += 32) t = df_add(t, sd[h * Kp + q]);
+            for (int o = 16; o; o >>= 1) t = df_add(t, df_shfl_xor(t, o));
+            if (lane == 0) total[q] = t;
+        }
+        __syncthreads();
+        if (tid < 32) red_ops(red, &sc, tid, tid < Kp ? (double)total[tid].h + (double)total[tid].l : 0.0, Kp);
+    } else {
+        red_apply(red, &sc, red_thread_sum(red.partial, nblk, Kp), Kp, sm);  // its first barrier publishes the copy
+    }
     __syncthreads();
     unsigned* gd = reinterpret_cast<unsigned*>(red.scal);
     if (tid < kWords) gd[tid] = ss[tid];
-    if (tid + kRedFinishThreads < kWords) gd[tid + kRedFinishThreads] = ss[tid + kRedFinishThreads];
+    if (tid + kThreads < kWords) gd[tid + kThreads] = ss[tid + kThreads];
 }
 
-void launch_red_finish(const Red& red, int Kp, cudaStream_t s) {
-    launch_pdl(k_red_finish, dim3(1), dim3(kRedFinishThreads), 0, s, red, Kp);
+void launch_red_finish(const Red& red, int Kp, bool f32, cudaStream_t s) {
+    if (f32) launch_pdl(k_red_finish<true>, dim3(1), dim3(kRedFinishThreads32), 0, s, red, Kp);
+    else launch_pdl(k_red_finish<false>, dim3(1), dim3(kRedFinishThreads), 0, s, red, Kp);
 }
 
 // r32 = f * invscale_j for every active system (the residual of the zero initial guess); x32 = p32 = 0.

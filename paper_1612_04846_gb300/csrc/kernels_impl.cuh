@@ -38,30 +38,69 @@ __device__ __forceinline__ void vst(T* p, const T (&o)[VecT<T>::W]) {
     *reinterpret_cast<typename VecT<T>::V*>(p) = v;
 }
 
-// Per-thread partial sums: FP64 for double data; for float data FP32 over at most 8 grid-stride
-// steps, then folded into FP64.
+// An unevaluated sum h + l of two FP32 values (about 48 bits).  GB300's FP64 pipe takes a warp instruction in 16 SM
+// clocks, so FP64 steps that all warps of a kernel execute cost more than the FP32 arithmetic they finish: sums of FP32
+// products are kept in pairs.
+struct Df {
+    float h, l;
+};
+__device__ __forceinline__ Df df_add(Df a, Df b) {
+    const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
+    const float e = __fadd_rn(__fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t)), __fadd_rn(a.l, b.l));
+    const float h = __fadd_rn(s, e);
+    return {h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ Df df_add(Df a, float b) { return df_add(a, Df{b, 0.f}); }
+__device__ __forceinline__ Df df_shfl_xor(Df v, int o) {
+    return {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
+}
+// A running pair sum whose rounding errors add up on the side: one FP32 addition on the chain from term to term.
+struct DfSum {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float h) {
+        const float t = __fadd_rn(s, h), b = __fsub_rn(t, s);
+        c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(h, b)));
+        s = t;
+    }
+    __device__ __forceinline__ void add(Df a) {
+        add(a.h);
+        c = __fadd_rn(c, a.l);
+    }
+    __device__ __forceinline__ Df get() const {
+        const float h = __fadd_rn(s, c);
+        return {h, __fsub_rn(c, __fsub_rn(h, s))};
+    }
+};
+
+// Per-thread partial sums: FP64 for double data; for float data FP32 over at most 8 grid-stride steps, then folded into a
+// pair sum (a conversion and an FP64 addition per fold occupied the FP64 pipe for about 4 us of a 1023^2, 8-system dot).
 template <class T>
 struct Accum {
     static constexpr int W = VecT<T>::W;
     double tot[W];
+    __device__ Accum() {
+        for (int v = 0; v < W; ++v) tot[v] = 0.0;
+    }
+    __device__ __forceinline__ void add(const T (&a)[W], const T (&b)[W]) {
+        for (int v = 0; v < W; ++v) tot[v] = fma((double)a[v], (double)b[v], tot[v]);
+    }
+};
+template <>
+struct Accum<float> {
+    static constexpr int W = VecT<float>::W;
+    DfSum tot[W];
     float part[W];
     int n;
     __device__ Accum() : n(0) {
-        for (int v = 0; v < W; ++v) { tot[v] = 0.0; part[v] = 0.f; }
+        for (int v = 0; v < W; ++v) part[v] = 0.f;
     }
-    __device__ __forceinline__ void add(const T (&a)[W], const T (&b)[W]) {
-        if constexpr (sizeof(T) == 8) {
-            for (int v = 0; v < W; ++v) tot[v] = fma((double)a[v], (double)b[v], tot[v]);
-        } else {
-            for (int v = 0; v < W; ++v) part[v] = fmaf(a[v], b[v], part[v]);
-            if (++n == 8) flush();
-        }
+    __device__ __forceinline__ void add(const float (&a)[W], const float (&b)[W]) {
+        for (int v = 0; v < W; ++v) part[v] = fmaf(a[v], b[v], part[v]);
+        if (++n == 8) flush();
     }
     __device__ __forceinline__ void flush() {
-        if constexpr (sizeof(T) == 4) {
-            for (int v = 0; v < W; ++v) { tot[v] += (double)part[v]; part[v] = 0.f; }
-            n = 0;
-        }
+        for (int v = 0; v < W; ++v) { tot[v].add(part[v]); part[v] = 0.f; }
+        n = 0;
     }
 };
 
@@ -466,21 +505,14 @@ __device__ __forceinline__ double red_thread_sum(const double* fin, int nfin, in
     return part;
 }
 
-__device__ __forceinline__ void red_apply(const Red& red, Scal* S, double part, int Kp, double* sm) {
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int G = (int)(blockDim.x * blockDim.y) / Kp;
-    __syncthreads();
-    if (tid < Kp * G) sm[tid] = part;
-    __syncthreads();
-    if (tid < Kp) {
-        double tot = 0.0;
-        for (int g = 0; g < G; ++g) tot += sm[g * Kp + tid];
-        finish_one(red, S, tid, tot);
-    }
-    __syncthreads();
-    if (tid == 0 && red.op == RED_CONV) {
-        int na = 0;
-        for (int s = 0; s < Kp; ++s) na += S->active[s] ? 1 : 0;
+// op with the total of system tid < Kp, by the block's first warp
+__device__ __forceinline__ void red_ops(const Red& red, Scal* S, int tid, double tot, int Kp) {
+    if (tid < Kp) finish_one(red, S, tid, tot);
+    if (red.op != RED_CONV) return;
+    __syncwarp();
+    const unsigned live = __ballot_sync(0xffffffffu, tid < Kp && S->active[tid] != 0);
+    if (tid == 0) {
+        const int na = __popc(live);
         S->nactive = na;
         S->it += 1;
         S->parity ^= 1;
@@ -491,6 +523,18 @@ __device__ __forceinline__ void red_apply(const Red& red, Scal* S, double part, 
         }
     }
 }
+__device__ __forceinline__ void red_apply(const Red& red, Scal* S, double part, int Kp, double* sm) {
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    const int G = (int)(blockDim.x * blockDim.y) / Kp;
+    __syncthreads();
+    if (tid < Kp * G) sm[tid] = part;
+    __syncthreads();
+    if (tid >= 32) return;
+    double tot = 0.0;
+    if (tid < Kp)
+        for (int g = 0; g < G; ++g) tot += sm[g * Kp + tid];
+    red_ops(red, S, tid, tot, Kp);
+}
 
 // Block reduction of per-thread partials (W systems per thread, chunk = threadIdx.x) followed by
 // the grid reduction in the last block, or, for a deferred reduction, by k_red_finish.  Every thread
@@ -500,27 +544,50 @@ __device__ void reduce_finish(Accum<T>& acc, const Red& red, int Kp) {
     constexpr int W = VecT<T>::W;
     extern __shared__ double sm[];
     __shared__ int am_last;
-    acc.flush();
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     const int nthr = blockDim.x * blockDim.y;
-    for (int v = 0; v < W; ++v) sm[tid * W + v] = acc.tot[v];  // = sm[point * Kp + system]
-    __syncthreads();
     const int G = nthr / Kp;
-    double part = 0.0;
-    if (tid < Kp * G) {
-        const int s = tid % Kp, g = tid / Kp;
-        for (int p = g; p < (int)blockDim.y; p += G) part += sm[p * Kp + s];
-    }
-    __syncthreads();
-    if (tid < Kp * G) sm[tid] = part;
-    __syncthreads();
     const int nblk = (int)gridDim.x;
+    double tot = 0.0;  // the block's sum of system tid < Kp; FP32 data: Df until here
+    Df td = {0.f, 0.f};
+    if constexpr (sizeof(T) == 4) {
+        Df* sd = reinterpret_cast<Df*>(sm);
+        acc.flush();
+        for (int v = 0; v < W; ++v) sd[tid * W + v] = acc.tot[v].get();  // = sd[point * Kp + system]
+        __syncthreads();
+        DfSum part;
+        if (tid < Kp * G) {
+            const int s = tid % Kp, g = tid / Kp;
+            for (int p = g; p < (int)blockDim.y; p += G) part.add(sd[p * Kp + s]);
+        }
+        __syncthreads();
+        if (tid < Kp * G) sd[tid] = part.get();
+        __syncthreads();
+        if (tid < Kp) {
+            DfSum t;
+            for (int g = 0; g < G; ++g) t.add(sd[g * Kp + tid]);
+            td = t.get();
+            tot = (double)td.h + (double)td.l;
+        }
+    } else {
+        for (int v = 0; v < W; ++v) sm[tid * W + v] = acc.tot[v];
+        __syncthreads();
+        double part = 0.0;
+        if (tid < Kp * G) {
+            const int s = tid % Kp, g = tid / Kp;
+            for (int p = g; p < (int)blockDim.y; p += G) part += sm[p * Kp + s];
+        }
+        __syncthreads();
+        if (tid < Kp * G) sm[tid] = part;
+        __syncthreads();
+        if (tid < Kp)
+            for (int g = 0; g < G; ++g) tot += sm[g * Kp + tid];
+    }
     if (red.defer) {
         // visible to k_red_finish, which waits for this grid to complete
         if (tid < Kp) {
-            double tot = 0.0;
-            for (int g = 0; g < G; ++g) tot += sm[g * Kp + tid];
-            red.partial[(size_t)blockIdx.x * Kp + tid] = tot;
+            if constexpr (sizeof(T) == 4) reinterpret_cast<Df*>(red.partial)[(size_t)blockIdx.x * Kp + tid] = td;
+            else red.partial[(size_t)blockIdx.x * Kp + tid] = tot;
         }
         if (tid == 0 && blockIdx.x == 0) *red.nblk = (unsigned)nblk;
         return;
@@ -533,8 +600,6 @@ __device__ void reduce_finish(Accum<T>& acc, const Red& red, int Kp) {
     const int gsize = one_level ? nblk : min(kRedGroup, nblk - group * kRedGroup);
     double* part2 = red.partial + (size_t)nblk * Kp;
     if (tid < Kp) {
-        double tot = 0.0;
-        for (int g = 0; g < G; ++g) tot += sm[g * Kp + tid];
         red.partial[(size_t)blockIdx.x * Kp + tid] = tot;
         __threadfence();  // only the writers of the partials need their stores visible before the ticket
     }

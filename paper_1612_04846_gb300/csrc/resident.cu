@@ -63,27 +63,13 @@ constexpr int kHR = 3, kHX = 2, kHY = 1, kHD = 2, kHP = 1;  // halo rows of R, X
 constexpr int kSP = 64;                                     // leading dimension of the sine bases
 constexpr int kStrip = 4;                                   // most rows a thread takes at a time
 
-// An unevaluated sum h + l of two FP32 values (about 48 bits).  GB300's FP64 pipe takes a warp instruction in
-// 16 SM clocks, so a scalar FP64 step that all 16 warps execute costs 256: the CG's sums and scalars run on the
-// FP32 pipe in pairs instead (a reduction over 16 CTAs of 512 threads: 3700 -> 2000 clocks).
-struct Df {
-    float h, l;
-};
-__device__ __forceinline__ Df df_add(Df a, Df b) {
-    const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
-    const float e = __fadd_rn(__fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t)), __fadd_rn(a.l, b.l));
-    const float h = __fadd_rn(s, e);
-    return {h, __fsub_rn(e, __fsub_rn(h, s))};
-}
-__device__ __forceinline__ Df df_add(Df a, float b) { return df_add(a, Df{b, 0.f}); }
+// The CG's sums and scalars are pairs: a scalar FP64 step that all 16 warps execute costs 256 SM clocks (a reduction over
+// 16 CTAs of 512 threads: 3700 -> 2000 clocks).
 // a / b rounded to FP32 from a pair quotient (about 45 bits)
 __device__ __forceinline__ float df_div(Df a, Df b) {
     const float q = __fdiv_rn(a.h, b.h);
     const float r = __fadd_rn(__fmaf_rn(-q, b.h, a.h), __fmaf_rn(-q, b.l, a.l));
     return __fadd_rn(q, __fdiv_rn(r, b.h));
-}
-__device__ __forceinline__ Df df_shfl_xor(Df v, int o) {
-    return {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
 }
 
 __device__ __forceinline__ unsigned map_rank(const void* p, int rank) {

@@ -306,7 +306,7 @@ Red deferred(const bura_plan* p, Red r) {
 }
 
 void red_finish(bura_plan* p, const Red& r, int Kp, bool is_f32, cudaStream_t s) {
-    traced(p, K_REDFIN, is_f32, true, 0.0, s, [&] { launch_red_finish(r, Kp, s); });
+    traced(p, K_REDFIN, is_f32, true, 0.0, s, [&] { launch_red_finish(r, Kp, is_f32, s); });
 }
 
 // Fold the timed launches of the finished solve into the per-kernel totals (stream must be idle).
