@@ -376,6 +376,22 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// FP64 sweeps of 2-D constant-coefficient levels with degree-2 smoothing (sweep64.cu).
+void sweep64_pre2(const Lev& L, int Kp, int nsm, const double* b, double* x, ChebStepT<double> c0, ChebStepT<double> c1,
+                  const double* dsh, const Red& none, cudaStream_t s);
+void sweep64_residual(const Lev& L, int Kp, int nsm, const double* x, const double* b, double* r, const double* dsh,
+                      const Red& none, cudaStream_t s);
+void sweep64_restrict(const Lev& Lf, const Lev& Lc, int Kp, int nsm, const double* x, const double* b, double* bc,
+                      const double* dsh, cudaStream_t s);
+void sweep64_prolong(const Lev& Lf, const Lev& Lc, int Kp, int nsm, const double* ec, double* x, cudaStream_t s);
+// The post-smoothing steps: x1 = the first one's iterate; the second one's in x, with b . x when red asks for it.
+void sweep64_post1(const Lev& L, int Kp, int nsm, const double* x, double* x1, const double* b, ChebStepT<double> c0,
+                   const double* dsh, const Red& none, cudaStream_t s);
+void sweep64_post2(const Lev& L, int Kp, int nsm, double* x, const double* x1, const double* b, ChebStepT<double> c1,
+                   const double* dsh, const Red& red, cudaStream_t s);
+// q = (A - d_j I) p and p . q for the direction buffer the parity selects, as k_spmv_q.
+void sweep64_spmv(const Lev& L, int Kp, int nsm, const double* pa, const double* pb, double* q, const Red& red, cudaStream_t s);
+
 // FP64 refinement and output kernels.
 // fp (optional): the address of a device pointer to the right-hand side, read by the kernel instead of f
 // (a captured solve whose right-hand side changes from launch to launch)

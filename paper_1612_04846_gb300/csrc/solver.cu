@@ -1165,6 +1165,17 @@ ChebStepT<T> step_of(const Work<T>& w, int l, int m, bool with_c1 = true) {
 // fused kernels do) costs more there than the extra vector pass.
 bool split_sweeps(const bura_plan* p) { return p->dim != 2 || p->var; }
 
+// Whether level l of the FP64 work takes the sweeps of sweep64.cu: any 2-D constant-coefficient level above the coarse
+// solver with degree-2 smoothing (511^2, k = 7: the whole solve 4.02 -> 2.22 ms).  Levels of at
+// least kLean64Stored values store the residual and restrict it (255^2, k = 7: 18 us of kernels against 22 for the single
+// sweep, 511^2: 45 against 54); smaller ones save a launch (127^2: 10 us against 17).
+constexpr long long kLean64Stored = 300000;
+template <class T>
+bool lean64(const bura_plan* p, const Work<T>& w, int l) {
+    return sizeof(T) == 8 && p->dim == 2 && !p->var && w.deg[l] == 2 && l + 1 < (int)p->hl.size() &&
+           p->opt.sweeps == BURA_SWEEP_AUTO;
+}
+
 // Launch the shared-memory V-cycle over levels w.lc..nlev-1 for the right-hand side b (global), one
 // CTA per 16-byte chunk of systems; the result of level lc is written to w.xa[lc].  Inside a CTA every
 // level has b, xa, xb, dd of its chunk in shared memory; a level's pre-smoothing (zero step + deg-1
@@ -1338,6 +1349,33 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
         else
             Ops<T>::cheb_step(g, L, dim, var, xin, din, b, xout, dout, cs, w.dsh, red, s);
     };
+    if constexpr (sizeof(T) == 8) {
+        if (lean64(p, w, l)) {
+            const Lev& Lc = w.L[l + 1];
+            traced(p, K_PRE2, f32, fine, vbytes<T>(p, l, 2.0, false), s,
+                   [&] { sweep64_pre2(L, w.Kp, p->nsm, b, A, step_of(w, l, 0), step_of(w, l, 1), w.dsh, none, s); });
+            if ((long long)w.Kp * L.N >= kLean64Stored) {
+                traced(p, K_RESID, f32, fine, vbytes<T>(p, l, 3.0, false), s,
+                       [&] { sweep64_residual(L, w.Kp, p->nsm, A, b, D, w.dsh, none, s); });
+                traced(p, K_RESTRICT, f32, fine, vbytes<T>(p, l, 1.0, false) + vbytes<T>(p, l + 1, 1.0, false), s,
+                       [&] { Ops<T>::restrict_r(w.g[l + 1], L, Lc, dim, D, w.b[l + 1], s); });
+            } else {
+                traced(p, K_RESTRICT, f32, fine, vbytes<T>(p, l, 2.0, false) + vbytes<T>(p, l + 1, 1.0, false), s,
+                       [&] { sweep64_restrict(L, Lc, w.Kp, p->nsm, A, b, w.b[l + 1], w.dsh, s); });
+            }
+            const T* ec = vcycle<T>(p, w, l + 1, w.b[l + 1], false, s);
+            traced(p, K_PROLONG, f32, fine, vbytes<T>(p, l, 2.0, false) + vbytes<T>(p, l + 1, 1.0, false), s,
+                   [&] { sweep64_prolong(L, Lc, w.Kp, p->nsm, ec, A, s); });
+            traced(p, K_CHEB, f32, fine, vbytes<T>(p, l, 3.0, false), s, [&] {
+                sweep64_post1(L, w.Kp, p->nsm, A, B, b, step_of(w, l, 0), w.dsh, none, s);
+            });
+            traced(p, K_CHEB, f32, fine, vbytes<T>(p, l, 4.0, false), s, [&] {
+                sweep64_post2(L, w.Kp, p->nsm, A, B, b, step_of(w, l, 1), w.dsh, rz_fused ? beta : none, s);
+            });
+            if (rz_fused) red_finish(p, beta, w.Kp, f32, s);
+            return A;
+        }
+    }
     // TMA-staged level with degree-2 smoothing: pre-smoothing fused with the restriction of its
     // residual, the coarse levels, the first post-smoothing step fused with the prolongation, the last
     // post-smoothing step (with r.z and beta at the finest level)
@@ -1516,10 +1554,15 @@ int pcg_body(bura_plan* p, Work<T>& w, unsigned long long cond, cudaStream_t s) 
     const auto& tl = w.tma[0];
     const auto& s3l = w.s3[0];
     const bool s3 = s3l.on;
-    if (!tl.on && split_sweeps(p) && !s3)  // p = z + beta p as its own pointwise sweep
+    const bool lean = lean64(p, w, 0) && w.lc != 0;
+    const bool split = !tl.on && !s3 && (split_sweeps(p) || lean);
+    if (split)  // p = z + beta p as its own pointwise sweep
         traced(p, K_PUPD, f32, true, vbytes<T>(p, 0, 3.0, false), s,
                [&] { Ops<T>::pupdate(g, L.N, z, w.pa, w.pb, ralpha, s); });
-    traced(p, K_SPMV, f32, true, vbytes<T>(p, 0, !tl.on && split_sweeps(p) && !s3 ? 2.0 : 4.0, true), s, [&] {
+    traced(p, K_SPMV, f32, true, vbytes<T>(p, 0, split ? 2.0 : 4.0, true), s, [&] {
+        if constexpr (sizeof(T) == 8) {
+            if (lean) return sweep64_spmv(L, w.Kp, p->nsm, w.pa, w.pb, w.q, ralpha, s);
+        }
         const CUtensorMap* mz = tl.on ? tl.find(TB_HALO, z) : nullptr;
         const CUtensorMap* ma = tl.on ? tl.find(TB_HALO, w.pa) : nullptr;
         const CUtensorMap* mbb = tl.on ? tl.find(TB_HALO, w.pb) : nullptr;
