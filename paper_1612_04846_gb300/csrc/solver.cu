@@ -1331,6 +1331,7 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
     T* D = w.dd[l];
     T* cur = A;
     T* oth = B;
+    bool rz_done = false;
     const auto& tl = w.tma[l];
     const auto& s3l = w.s3[l];
     const bool s3 = s3l.on;
@@ -1466,8 +1467,11 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
         std::swap(cur, oth);
         for (int m = 2; m < deg; ++m) {
             T* dout = m < deg - 1 ? D : nullptr;
+            // a single level's last step also forms r.z
+            const bool dot = rz_fused && m == deg - 1 && l == (int)p->hl.size() - 1;
             traced(p, K_CHEB, f32, fine, vbytes<T>(p, l, 4.0 + (dout ? 1.0 : 0.0), true), s,
-                   [&] { cheb(cur, D, oth, dout, step_of(w, l, m), none); });
+                   [&] { cheb(cur, D, oth, dout, step_of(w, l, m), dot ? beta : none); });
+            rz_done |= dot;
             std::swap(cur, oth);
         }
     } else {
@@ -1490,7 +1494,8 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
     }
     if (l == (int)p->hl.size() - 1) {  // coarsest level on the grid kernels: the Chebyshev solve above
         if (rz_fused) {
-            traced(p, K_DOT, f32, fine, vbytes<T>(p, l, 2.0, false), s, [&] { Ops<T>::dot(g, L.N, b, cur, beta, s); });
+            if (!rz_done)
+                traced(p, K_DOT, f32, fine, vbytes<T>(p, l, 2.0, false), s, [&] { Ops<T>::dot(g, L.N, b, cur, beta, s); });
             red_finish(p, beta, w.Kp, f32, s);
         }
         return cur;
