@@ -285,6 +285,7 @@ struct ResArgs {
     int re, ce;                                  // rows and columns of it per CTA
     int G, threads;                              // CTAs per system, threads per CTA
     int Kp;
+    int blk_pq, blk_rz;                          // CTAs of the TMA-staged A p and post-smoothing of level 0
     size_t N;
     double wx, wy;                               // level-0 weights in FP64
     ResLevel lev[kResMaxLevels], tail[kResMaxLevels];  // in slabs; the tail's whole levels (le .. ld)

@@ -1101,6 +1101,11 @@ int tma_blocks(const TmaGeo& g, int Kp, int nsm, int kind, int S) {
     return nt < nsm * per_sm ? nt : nsm * per_sm;
 }
 
+void tma_dot_blocks(const TmaGeo& g, int nsm, int* spmv, int* post2) {
+    *spmv = tma_blocks(g, g.Kp, nsm, TK_SPMV, ring_stages(g, TK_SPMV));
+    *post2 = tma_blocks(g, g.Kp, nsm, TK_POST2, ring_stages(g, TK_POST2));
+}
+
 // Launch geometry of one kind: g with its ring depth, CTAs, dynamic shared memory.
 struct Shape {
     TmaGeo g;

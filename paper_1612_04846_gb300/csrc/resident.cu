@@ -4,7 +4,8 @@
 // The shifted systems never exchange values, so each system gets a thread-block cluster of G CTAs of its own
 // that runs the refinement loop, the multigrid-preconditioned CG inside it and all their decisions: the
 // formulas are those of the grid kernels (kernels_tma.cu, fdiag.cu), of the reductions (kernels_impl.cuh) and
-// of the controller (outer.cu), point by point; only the grouping of the dot products' sums differs.
+// of the controller (outer.cu), point by point; only the grouping of the dot products' sums differs (except in the first
+// iteration: see grid_dot).
 //
 // Why: on grids of up to about 10^5 points the graph of grid kernels is bound by its own launches.  A 383 x 255,
 // k = 8 solve is 108 launches in 812 us, 7.5 us each, for about 1 us of work each.  Here a vector is read from
@@ -30,7 +31,7 @@
 // The exact solve of level le is fdiag.cu's fast diagonalization, every sum in the same order.
 //
 // Measured (GB300, one solve, tol 1e-6, graph of kernels -> here): 63^2, k = 5: 168 -> 45 us; 127^2, k = 6: 372 -> 100;
-// 255^2, k = 7: 550 -> 201; 383 x 255, k = 8: 812 -> 280.  What is left is latency: a 127^2 iteration is 9.5 us, of
+// 255^2, k = 7: 550 -> 201; 383 x 255, k = 8: 812 -> 330.  What is left is latency: a 127^2 iteration is 9.5 us, of
 // which the exact solve's four products and three exchanges take 3.6.
 //
 // Variable coefficients: every level's face and diagonal weights stay in the owner's shared memory too (three floats a
@@ -366,6 +367,84 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) t = df_add(t, df_shfl_xor(t, o));
         flip ^= 1;
+        return t;
+    };
+    // This thread's share of a . b (level 0) in the groups that the graph's kernels sum in FP32.  A system that ends after
+    // one iteration returns alpha p, so another grouping, which may round alpha the other way, would show in the result's
+    // eighth digit (small powers, whose largest shifts converge at once: one plan of 32 in ten batches).  Taken in the first
+    // iteration only, later ones correct such a difference (the cost: 63^2 47 -> 48 us, 383 x 255, k = 8, 282 -> 330, 32
+    // mixed problems 2.51 -> 2.81 ms).  A group's values are read from the CTAs
+    // that own their rows, behind a reduction used as a barrier: unlike a cluster barrier it is bounded, and a CTA that gave
+    // up keeps its shared memory until all are done.
+    //   one exact solve, or variable coefficients: points P and P + 64, P in the even runs of 64 (the grid sweeps)
+    //   else: the points of a thread of k_spmv_tma, or, with rz, of k_post2_tma, up to eight at a time
+    auto grid_dot = [&](int oa, int Ha, int ob, int Hb, bool rz) {
+        const Slab s = range(0);
+        const int nx = s.nx, ny = s.ny, N = nx * ny;
+        asm volatile("fence.acq_rel.cluster;" ::: "memory");
+        (void)all_sum(Df{0.f, 0.f});
+        asm volatile("fence.acq_rel.cluster;" ::: "memory");
+        Df t{0.f, 0.f};
+        float v = 0.f;
+        int n = 0;
+        auto flush = [&]() {
+            t = df_add(t, v);
+            v = 0.f;
+            n = 0;
+        };
+        // up to four terms in order, all their values loaded first; where(i, y, x) says whether term i exists
+        auto four = [&](auto&& where) {
+            float av[4], bv[4];
+            bool on[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                int y = 0, x = 0;
+                on[i] = where(i, y, x);
+                if (on[i]) {
+                    const int rank = min(y >> le, a.ne - 1) / a.re;
+                    const int k = (y - ((rank * a.re) << le)) * s.ld + 2 + x;
+                    const float *pa = sm + oa + Ha * s.ld + k, *pb = sm + ob + Hb * s.ld + k;
+                    av[i] = rank == g ? *pa : *cl.map_shared_rank(pa, rank);
+                    bv[i] = rank == g ? *pb : *cl.map_shared_rank(pb, rank);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (on[i]) {
+                    v = fmaf(av[i], bv[i], v);
+                    if (++n == 8) flush();
+                }
+        };
+        // a CTA takes the groups that start in its own rows (another CTA's shared memory is some 50 clocks a warp's load)
+        if (VAR || le == 0) {
+            for (int c = s.y0 * nx + tid; c < s.y1 * nx; c += kResThreads) {
+                if (c & 64) continue;
+                four([&](int i, int& y, int& x) {
+                    const int P = c + 64 * i;
+                    y = P / nx;
+                    x = P - y * nx;
+                    return i < 2 && P < N;
+                });
+                flush();
+            }
+        } else {
+            const int R = 256 / (a.Kp / 4), blocks = rz ? a.blk_rz : a.blk_pq;  // thread rows a CTA, CTAs
+            const int ntx = (nx + kTX - 1) / kTX, tiles = ntx * ((ny + kTY - 1) / kTY);
+            const int lo = (s.y0 + kTY - 1) / kTY * ntx, hi = min((s.y1 + kTY - 1) / kTY * ntx, blocks);
+            for (int c = tid; c < (hi - lo) * R; c += kResThreads) {
+                const int c0 = c / R, row = c - c0 * R;
+                for (int tile = lo + c0; tile < tiles; tile += blocks) {
+                    const int ty = tile / ntx, x0 = (tile - ty * ntx) * kTX, y0 = ty * kTY;
+                    four([&](int i, int& y, int& x) {
+                        const int p = row + (rz ? i / 2 : i) * R;
+                        x = x0 + p % kTX;
+                        y = y0 + (rz ? p / kTX * 2 + (i & 1) : p / kTX);
+                        return p < (rz ? kTX * kTY / 2 : kTX * kTY) && x < nx && y < ny;
+                    });
+                }
+                flush();
+            }
+        }
         return t;
     };
     // the same in FP64 (norms of the refinement): warp 0 adds the partials; the sum is returned in warp 0 only.
@@ -851,6 +930,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
             // z = M r into D
             Df t;
             t = cycle();
+            if (siters == 0) t = grid_dot(L0.oR, kHR, L0.oD, kHD, true);
             const Df rzn = all_sum(t);
             if (!isfinite(rzn.h)) breakdown = 1;
             const float beta = df_div(rzn, rz);
@@ -886,6 +966,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
                     t = df_add(t, p2.x + p2.y);
                 });
             }
+            if (siters == 0) t = grid_dot(a.o_p, kHP, L0.oY, kHY, false);
             const Df pq = all_sum(t);
             float af = 0.f;
             if (!(pq.h > 0.f) || !isfinite(pq.h)) breakdown = 1;

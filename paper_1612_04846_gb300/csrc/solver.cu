@@ -923,6 +923,7 @@ int build_resident(bura_plan* p) {
     ResArgs& a = p->res;
     CA(resident_args(p, w, 0, false, a, &p->res_on));
     if (!p->res_on) return BURA_OK;
+    if (a.le > 0 && !p->var) tma_dot_blocks(tma_geo(w.L[0], &w.L[1], w.Kp), p->nsm, &a.blk_pq, &a.blk_rz);
     CA(dalloc(p, &a.out, (size_t)p->K * sizeof(ResOut)));
     a.cfg = p->ocfg;
     a.x = nullptr;

@@ -185,6 +185,8 @@ struct TmaMaps5 {
 // Host side.  Every launcher returns the launch status; the kernels take the fault flag from red.scal.
 bool tma_supported(int Kp);
 TmaGeo tma_geo(const Lev& L, const Lev* Lc, int Kp);
+// CTAs that tma_spmv_p and tma_post2 launch for a level (constant coefficients).
+void tma_dot_blocks(const TmaGeo& g, int nsm, int* spmv, int* post2);
 // Whether the maps of a level with Kp floats per point are flat (2-D over 8-byte elements).
 bool tma_flat(int Kp);
 // Tensor map of an [ny][nx][Kp] float vector with a box of kind TmaBox.
