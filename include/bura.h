@@ -66,7 +66,7 @@ typedef struct {
 
 /* How the small levels of the multigrid V-cycle are run. */
 typedef enum {
-    BURA_COARSE_AUTO = 0,    /* FDIAG for 2-D constant coefficients, else CTA (faster than CLUSTER on GB300) */
+    BURA_COARSE_AUTO = 0,    /* 2-D: one resident launch where it fits, else FDIAG (constant) or CTA; 3-D: CTA */
     BURA_COARSE_CLUSTER = 1, /* levels with <= 16384 points in one thread-block cluster (vectors in L2);
                                 bura_setup returns BURA_EINVAL on a device without cluster launch */
     BURA_COARSE_CTA = 2,     /* the levels that fit 200 KB of shared memory in a single CTA */
@@ -81,7 +81,7 @@ typedef enum {
 
 /* How the level sweeps of the large levels are run. */
 typedef enum {
-    BURA_SWEEP_AUTO = 0, /* TMA-staged tiles (FP32, 2-D, constant coefficients, >= 1 tile per SM), else GRID */
+    BURA_SWEEP_AUTO = 0, /* TMA-staged sweeps (FP32, 2-D and large 3-D levels), small 2-D solves as one launch, else GRID */
     BURA_SWEEP_GRID = 1  /* grid-stride kernels with direct global loads everywhere */
 } bura_sweep_kind;
 
