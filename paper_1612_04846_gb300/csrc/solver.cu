@@ -704,7 +704,7 @@ int upload_tables(bura_plan* p, Work<T>& w) {
     if (w.minv) {
         std::vector<double> inv;
         dense_inverses(p->hl[w.le], p->dim, p->var, p->d, p->K, w.Kp, inv);
-        const std::vector<T> tv(inv.begin(), inv.end());  // (w.le: its level)
+        const std::vector<T> tv(inv.begin(), inv.end());
         CK(cudaMemcpy(w.minv, tv.data(), tv.size() * sizeof(T), cudaMemcpyHostToDevice));
     }
     return BURA_OK;
@@ -1110,6 +1110,7 @@ int build_work(bura_plan* p, Work<T>& w, bool full = true) {
     }
     if (w.lc < 0 || w.coarse_kind == BURA_COARSE_FDIAG || (w.coarse_kind == kCoarseResident && !p->var))
         w.le = -1;  // no dense solve
+    if (w.le < 0) w.minv = nullptr;
     if (w.le >= 0 && !w.minv) {  // [row][col][Kp] dense inverses of the exact level, filled by upload_tables
         const size_t n = (size_t)p->hl[w.le].N;
         CA(dalloc(p, &w.minv, n * n * w.Kp * sizeof(T)));
