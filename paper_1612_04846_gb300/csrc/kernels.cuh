@@ -78,7 +78,7 @@ struct OuterCfg {
     double c[KMAXP], d[KMAXP];  // weights and shifts
     double lambda_lo;           // lower bound on lambda_min(A); 0: relative residual thresholds
     double inner_rtol;          // largest residual reduction asked of one FP32 inner solve
-    double rtol_slack;          // inner_rtol^1e-9 (the margin of the refinement plan's step count)
+    double rtol_slack, log_rtol;  // inner_rtol^1e-9 and log(inner_rtol), for the refinement plan's step count
     long long wait_cycles;      // TMA ring wait budget of the inner solves (0: default)
     int K, max_outer, max_iters;
 };

@@ -51,6 +51,7 @@
 #include <mutex>
 
 #include "kernels_impl.cuh"
+#include "refine_plan.h"
 #include "tma.cuh"
 
 namespace cg = cooperative_groups;
@@ -844,16 +845,13 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
     const size_t gofs = (size_t)s0.y0 * s0.nx;
 
     if (cx.warp == kResWarps - 1) {
-        // this system's relative threshold need_j, reached in n_j = ceil(log need_j / log inner_rtol - 1e-9) steps of
-        // need_j^(1/n_j) each; n_j by comparing with the powers of inner_rtol (rtol_slack = inner_rtol^1e-9)
+        // this system's relative threshold need_j, reached in n_j steps of need_j^(1/n_j) each
         const OuterCfg& c = *a.cfg;
         const double t = c.lambda_lo > 0 ? tol * (c.lambda_lo - c.d[sys]) / (c.K * c.c[sys]) : tol;
         double st2 = 1.0;  // the square of a step's share
         if (t < 1.0) {
-            double r = c.inner_rtol;
-            int n = 1;
-            for (; t < r * c.rtol_slack && r > 0.0; ++n) r *= c.inner_rtol;
-            st2 = n == 1 ? t * t : n == 2 ? t : pow(t, 2.0 / n);
+            const double n = plan_steps(t, c.inner_rtol, c.rtol_slack, c.log_rtol);
+            st2 = n == 1.0 ? t * t : n == 2.0 ? t : pow(t, 2.0 / n);
         }
         if (cx.lane == 0) {
             bc[5] = t;

@@ -2030,6 +2030,7 @@ int upload_outer(bura_plan* p) {
         oc.lambda_lo = p->lambda_lo;
         oc.inner_rtol = p->opt.inner_rtol;
         oc.rtol_slack = std::pow(p->opt.inner_rtol, 1e-9);
+        oc.log_rtol = std::log(p->opt.inner_rtol);
         oc.wait_cycles = p->wait_cycles;
         oc.K = p->K;
         oc.max_outer = p->opt.max_outer;
