@@ -406,7 +406,9 @@ int bura_solve_sum(bura_plan* const* plans, int n, const double* f, double* u, d
  * of their waits on the shared-memory ring for the later solves of this plan.  A budget shorter than a
  * copy's latency makes the first waits give up: the kernel drains its copies in flight under the default
  * budget, records the fault in the plan's CG state, and the solve returns BURA_ETIMEOUT; the plan stays
- * usable.  Errors: BURA_EINVAL (null plan, cycles < 0).
+ * usable.  The one-launch solve of a small 2-D plan holds its waits for the other CTAs of a cluster to the same
+ * budget: it reports a wait that took longer, and waits on under the default one.
+ * Errors: BURA_EINVAL (null plan, cycles < 0).
  */
 int bura_set_tma_wait_cycles(bura_plan* plan, long long cycles);
 

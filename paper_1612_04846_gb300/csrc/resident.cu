@@ -26,7 +26,8 @@
 // with 16 CTAs of 512 threads).  Every (buffer, level) has an mbarrier of its own, used once per CG iteration;
 // the reductions alternate between two.  A sender is never two uses ahead of a receiver: between two uses of a
 // barrier lies a reduction, which needs every CTA's contribution.  For the same reason a halo row is only
-// written when its last readers are done.  Every wait is bounded.
+// written when its last readers are done.  Every wait is bounded, and a wait that ran out is looked at before the sum it
+// was for is used and once more at the end: the outcome is then BURA_ETIMEOUT.
 //
 // The exact solve of level le is fdiag.cu's fast diagonalization, every sum in the same order.
 //
@@ -91,8 +92,10 @@ __device__ __forceinline__ void put2(void* p, int rank, uint64_t* bar, float v0,
                  "f"(v0), "f"(v1), "r"(map_rank(bar, rank))
                  : "memory");
 }
-// Wait for a phase whose bytes other CTAs of the cluster store; false after the default budget.
-__device__ __forceinline__ bool wait_bytes(uint64_t* bar, unsigned parity) {
+// Wait for a phase whose bytes other CTAs of the cluster store; false if they have not come within the larger of the default
+// budget and `budget`, the caller's (0: none).  A phase that takes longer than the caller's sets `late`: it is waited for all
+// the same, so that no store is in flight into a buffer that is in use again, and the CTAs of a cluster stay together.
+__device__ __forceinline__ bool wait_bytes(uint64_t* bar, unsigned parity, long long budget, bool& late) {
     const long long t0 = clock64();
     for (;;) {
         unsigned ok;
@@ -105,8 +108,11 @@ __device__ __forceinline__ bool wait_bytes(uint64_t* bar, unsigned parity) {
             : "=r"(ok)
             : "r"(smem_u32(bar)), "r"(parity)
             : "memory");
+        if (ok && budget == 0) return true;
+        const long long t = clock64() - t0;
+        if (budget > 0 && t > budget) late = true;
         if (ok) return true;
-        if (clock64() - t0 > kTmaWaitCycles) return false;
+        if (t > max(budget, kTmaWaitCycles)) return false;
     }
 }
 // One float from global to shared memory, asynchronously; copies_done() waits for this thread's.
@@ -223,7 +229,8 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
     Ctx<kResWarps> cx{&a, sm, g, G, tid >> 5, tid & 31};
     const int le = a.le;
     const float d = a.dsh[sys];
-    bool late = false;
+    const long long budget = a.cfg->wait_cycles;  // the caller's, 0: the default
+    bool late = false;  // a wait of this thread outlasted the caller's budget
     if (tid == 0) {
         mbar_init(&bimg, 1);
         for (int l = 0; l <= le; ++l) {
@@ -237,13 +244,12 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         mbar_init(&bS[1], 1);
         mbar_fence_init();
         if (!VAR) {
-            const long long w = a.cfg->wait_cycles;
             mbar_expect_tx(&bimg, a.img_bytes);
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                          ::"r"(smem_u32(sm + a.o_sx)), "l"(a.img), "r"(a.img_bytes), "r"(smem_u32(&bimg))
                          : "memory");
             // a wait budget of the caller's starts at the copy's issue; the default one after the buffers are cleared
-            if (w > 0) late = !mbar_wait_bounded(&bimg, 0, w);
+            if (budget > 0) late = !mbar_wait_bounded(&bimg, 0, budget);
         }
     }
     __syncthreads();
@@ -278,7 +284,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
     // everything but the bases starts at zero: the zero columns and the rows outside the grid stay zero
     for (int i = a.o_zero / 4 + tid; i < a.floats / 4; i += kResThreads)
         reinterpret_cast<float4*>(sm)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (!VAR && !mbar_wait_bounded(&bimg, 0, kTmaWaitCycles)) late = true;  // (a late copy lands before the kernel goes on)
+    if (!VAR && !mbar_wait_bounded(&bimg, 0, max(budget, kTmaWaitCycles))) late = true;  // (it lands before the kernel goes on)
     int faulted = __syncthreads_or(late);
     if constexpr (VAR) {
         // the weights (faces negated) of the own rows and three halo rows, the tail's whole levels and its dense inverse in
@@ -326,14 +332,14 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
     cl.sync();  // every CTA runs and has cleared its buffers and barriers before the first remote store
 
     unsigned uR = 0, uD = 0, uC = 0, uB = 0, uV = 0, uS = 0;  // the parity of each barrier's next phase
-    bool lost = false;  // a wait of this thread ran out
+    bool lost = false;  // what a wait of this thread was for did not come
     int gone = 0;       // ... of this CTA, as of its last reduction
     // arm (thread 0) and await one phase; local values of the phase are published by the caller's barrier
     auto arm = [&](uint64_t* bar, unsigned bytes) {
         if (tid == 0) mbar_expect_tx(bar, bytes);
     };
     auto await = [&](uint64_t* bar, unsigned& bits, int at) {
-        if (!lost && !wait_bytes(bar, (bits >> at) & 1u)) lost = true;
+        if (!lost && !wait_bytes(bar, (bits >> at) & 1u, budget, late)) lost = true;
         bits ^= 1u << at;
     };
     auto range = [&](int l) {
@@ -824,7 +830,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         if (s.some())
             for (int y = s.y0 + cx.warp; y < s.y1; y += kResWarps)
                 for (int x = cx.lane; x < s.nx; x += 32) a.vx[((size_t)y * s.nx + x) * a.Kp + sys] = D[y * s.ld + x];
-        if (lost || faulted) atomicExch(&a.scal->fault, 1);
+        if (lost || late || faulted) atomicExch(&a.scal->fault, 1);
         pdl_trigger();
         cl.sync();  // no CTA leaves while another may still store into its shared memory
         return;
@@ -871,7 +877,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         bc[0] = sum_f;
         bc[1] = bc[5] * bc[5] * sum_f;
     }
-    __syncthreads();
+    if (__syncthreads_or(lost)) faulted = gone = 1;
     const double fn2 = bc[0], thr64 = bc[1];
     const int max_outer = a.cfg->max_outer, max_iters = a.cfg->max_iters;
 
@@ -1043,7 +1049,8 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         }
         t = all_sum64(t, 0u);
         if (tid == 0) bc[0] = t;
-        __syncthreads();
+        gone = __syncthreads_or(lost);
+        if (gone) { status = -6; break; }  // (the sum lacks what did not come)
         rr64 = bc[0];
     }
     if (outer == 0)
@@ -1055,6 +1062,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         out.siters = siters;
     }
     if (tid == 0 && g == 0) out.status = status;
+    gone = __syncthreads_or(lost || late);
     cl.sync();  // no CTA leaves while another may still store into its shared memory
     if (tid == 0 && gone) out.status = -6;
 }
