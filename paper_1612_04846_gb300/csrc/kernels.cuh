@@ -10,8 +10,8 @@
 // Reductions (per system dot products) are deterministic: per-thread partials, a fixed-order
 // block reduction in shared memory, per-block partials in global scratch and a fixed-order
 // reduction by the last block to finish (threadfence + atomic ticket), which also applies the
-// CG scalar updates for every system.  Accumulation is FP64 from the block level up; a thread's
-// own partial is FP32 for FP32 data (at most a few tens of products) and FP64 for FP64 data.
+// CG scalar updates for every system.  FP64 data: FP64 throughout.  FP32 data: FP32 over at most eight products, then sums
+// of three FP32 words (sum3.h), whose error is below that of FP64 sums, and FP64 for the totals and the scalar updates.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -127,8 +127,8 @@ struct Red {
 // The final step of a deferred reduction: one CTA of kRedFinishThreads sums the producer's block
 // partials in block order and applies op; launched right after the producer on the same stream.
 constexpr int kRedFinishThreads = 256;
-constexpr int kRedFinishThreads32 = 512;  // FP32 data, whose partials are pairs: all of 8 systems x 1280 blocks in flight
-constexpr int kRedFinBatch32 = 20;
+constexpr int kRedFinishThreads32 = 512;  // FP32 data, whose partials are three words: all of 8 systems x 1280 blocks in flight
+constexpr int kRedFinBatch32 = 10, kRedFinBatchFew = 4;  // blocks loaded at once per thread; ... of a small grid
 void launch_red_finish(const Red& red, int Kp, bool f32, cudaStream_t s);
 
 // One level of the single-CTA coarse V-cycle: its vectors live in the CTA's shared memory at the

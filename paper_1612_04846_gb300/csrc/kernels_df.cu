@@ -241,7 +241,7 @@ void launch_update_residual_df(const Launch& g, const Lev& L, int dim, bool var,
     op.fyh = h.fh[1]; op.fyl = h.fl[1];
     op.fzh = h.fh[2]; op.fzl = h.fl[2];
     const float inv_sf = 1.0f / sf;
-    const size_t sh = (size_t)g.C * g.PPB * 4 * sizeof(double);
+    const size_t sh = (size_t)g.C * g.PPB * 4 * kRedBytes;
     if (dim == 2 && !var)
         launch_pdl(k_update_residual_df<2, false>, dim3(g.blocks), dim3(g.C, g.PPB), sh, s, L, g.Kp, op, fh, fl, vhin,
                    vlin, x, vhout, vlout, r32, sf, inv_sf, red);

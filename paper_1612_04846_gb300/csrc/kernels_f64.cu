@@ -1,5 +1,6 @@
 // FP64 instantiation of the multi-shift MG-PCG kernels, plus the FP64 refinement, cast and output
 // kernels shared by both precision paths.
+#include <type_traits>
 #include <cstddef>
 
 #include "kernels_impl.cuh"
@@ -173,13 +174,14 @@ void launch_norm2(long long N, const double* f, const Red& red, int nsm, cudaStr
 // Final step of a deferred grid reduction (Red::defer): the producer, the previous kernel on the
 // stream, has completed when griddepcontrol.wait returns, so its partials are visible without fences.
 // The CG state record is loaded into shared memory together with the partials (one L2 round trip for
-// both), updated there and written back whole; no other kernel touches it meanwhile.  F32: the partials are pairs, summed
-// by one thread per (system, group of blocks), then one warp per system; 1216 partials of 8 systems in FP64 on one SM
-// were bound by its FP64 pipe.
+// both), updated there and written back whole; no other kernel touches it meanwhile.  F32: the partials are three-word sums
+// (all first words, all second, all third), added by one thread per (pair of systems, group of blocks), then one warp per system;
+// 1216 partials of 8 systems in FP64 on one SM were bound by its FP64 pipe.
 template <bool F32>
 __global__ void __launch_bounds__(F32 ? kRedFinishThreads32 : kRedFinishThreads) k_red_finish(Red red, int Kp) {
     constexpr int kThreads = F32 ? kRedFinishThreads32 : kRedFinishThreads;
-    __shared__ double sm[kThreads];
+    __shared__ double sm[F32 ? 1 : kThreads];
+    __shared__ Sum3 sd[F32 ? 2 * kThreads : 1];
     __shared__ Scal sc;
     constexpr int kWords = (int)(sizeof(Scal) / sizeof(unsigned));
     static_assert(sizeof(Scal) % sizeof(unsigned) == 0 && kWords <= 2 * kThreads, "Scal copy");
@@ -194,34 +196,43 @@ __global__ void __launch_bounds__(F32 ? kRedFinishThreads32 : kRedFinishThreads)
     if (tid < kWords) ss[tid] = w0;
     if (tid + kThreads < kWords) ss[tid + kThreads] = w1;
     if constexpr (F32) {
-        const int G = kThreads / Kp, s = tid % Kp, g = tid / Kp;
+        const int Q = Kp / 2, G = kThreads / Q, q = tid % Q, g = tid / Q;  // a thread takes a pair of systems
         const float2* fin = reinterpret_cast<const float2*>(red.partial);
-        Df* sd = reinterpret_cast<Df*>(sm);
+        const size_t n = (size_t)nblk * Q;
         if (g < G) {
-            DfSum part;
-            for (int b0 = g; b0 < nblk; b0 += kRedFinBatch32 * G) {
-                float2 v[kRedFinBatch32];
+            Sum3x2 part{};
+            auto some = [&](auto count, int b0) {  // blocks b0, b0 + G, ..., all loads before the first addition
+                constexpr int B = decltype(count)::value;
+                float2 v[3][B];
 #pragma unroll
-                for (int j = 0; j < kRedFinBatch32; ++j) {
-                    const int b = b0 + j * G;
-                    v[j] = b < nblk ? __ldcg(fin + (size_t)b * Kp + s) : make_float2(0.f, 0.f);
-                }
+                for (int w = 0; w < 3; ++w)
 #pragma unroll
-                for (int j = 0; j < kRedFinBatch32; ++j) part.add(Df{v[j].x, v[j].y});
-            }
-            sd[tid] = part.get();
+                    for (int j = 0; j < B; ++j) {
+                        const int b = b0 + j * G;
+                        v[w][j] = b < nblk ? __ldcg(fin + w * n + (size_t)b * Q + q) : make_float2(0.f, 0.f);
+                    }
+#pragma unroll
+                for (int j = 0; j < B; ++j) part.add(Sum3x2{v[0][j], v[1][j], v[2][j]});
+            };
+            if (nblk <= kRedFinBatchFew * G)
+                some(std::integral_constant<int, kRedFinBatchFew>(), g);
+            else
+                for (int b0 = g; b0 < nblk; b0 += kRedFinBatch32 * G) some(std::integral_constant<int, kRedFinBatch32>(), b0);
+            sd[2 * tid] = part.lo();
+            sd[2 * tid + 1] = part.hi();
         }
         __syncthreads();
-        __shared__ Df total[KMAXP];
+        __shared__ double total[KMAXP];
         const int lane = tid & 31;
-        for (int q = tid >> 5; q < Kp; q += kThreads / 32) {
-            Df t = {0.f, 0.f};
-            for (int h = lane; h < G; h += 32) t = df_add(t, sd[h * Kp + q]);
-            for (int o = 16; o; o >>= 1) t = df_add(t, df_shfl_xor(t, o));
-            if (lane == 0) total[q] = t;
+        for (int q = tid >> 5; q < Kp; q += kThreads / 32) {  // (sd[group * Kp + system])
+            Sum3 t{};
+            for (int h = lane; h < G; h += 32) t.add(sd[h * Kp + q]);
+#pragma unroll
+            for (int o = 16; o; o >>= 1) t.add(sum3_shfl_xor(t, o));
+            if (lane == 0) total[q] = t.value();
         }
         __syncthreads();
-        if (tid < 32) red_ops(red, &sc, tid, tid < Kp ? (double)total[tid].h + (double)total[tid].l : 0.0, Kp);
+        if (tid < 32) red_ops(red, &sc, tid, tid < Kp ? total[tid] : 0.0, Kp);
     } else {
         red_apply(red, &sc, red_thread_sum(red.partial, nblk, Kp), Kp, sm);  // its first barrier publishes the copy
     }

@@ -12,6 +12,7 @@
 #include <mutex>
 
 #include "kernels.cuh"
+#include "sum3.h"
 
 namespace cg = cooperative_groups;
 
@@ -39,42 +40,35 @@ __device__ __forceinline__ void vst(T* p, const T (&o)[VecT<T>::W]) {
     *reinterpret_cast<typename VecT<T>::V*>(p) = v;
 }
 
-// An unevaluated sum h + l of two FP32 values (about 48 bits).  GB300's FP64 pipe takes a warp instruction in 16 SM
-// clocks, so FP64 steps that all warps of a kernel execute cost more than the FP32 arithmetic they finish: sums of FP32
-// products are kept in pairs.
-struct Df {
-    float h, l;
-};
-__device__ __forceinline__ Df df_add(Df a, Df b) {
-    const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
-    const float e = __fadd_rn(__fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t)), __fadd_rn(a.l, b.l));
-    const float h = __fadd_rn(s, e);
-    return {h, __fsub_rn(e, __fsub_rn(h, s))};
+__device__ __forceinline__ Sum3 sum3_shfl_xor(const Sum3& v, int o) {
+    return {__shfl_xor_sync(0xffffffffu, v.s, o), __shfl_xor_sync(0xffffffffu, v.c, o), __shfl_xor_sync(0xffffffffu, v.e, o)};
 }
-__device__ __forceinline__ Df df_add(Df a, float b) { return df_add(a, Df{b, 0.f}); }
-__device__ __forceinline__ Df df_shfl_xor(Df v, int o) {
-    return {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
-}
-// A running pair sum whose rounding errors add up on the side: one FP32 addition on the chain from term to term.
-struct DfSum {
-    float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float h) {
-        const float t = __fadd_rn(s, h), b = __fsub_rn(t, s);
-        c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(h, b)));
+
+// Two such sums side by side, with packed FP32 instructions (the same operations on each).
+struct Sum3x2 {
+    float2 s, c, e;
+    __device__ __forceinline__ static float2 two_sum_err2(float2 a, float2 b, float2& s) {
+        const float2 m = make_float2(-1.f, -1.f);
+        const float2 t = __fadd2_rn(a, b), v = __ffma2_rn(a, m, t);
         s = t;
+        return __fadd2_rn(__ffma2_rn(__ffma2_rn(v, m, t), m, a), __ffma2_rn(v, m, b));
     }
-    __device__ __forceinline__ void add(Df a) {
-        add(a.h);
-        c = __fadd_rn(c, a.l);
+    __device__ __forceinline__ void add(float2 x) {
+        const float2 r = two_sum_err2(s, x, s);
+        e = __fadd2_rn(e, two_sum_err2(c, r, c));
     }
-    __device__ __forceinline__ Df get() const {
-        const float h = __fadd_rn(s, c);
-        return {h, __fsub_rn(c, __fsub_rn(h, s))};
+    __device__ __forceinline__ void add(const Sum3x2& o) {
+        const float2 r = two_sum_err2(s, o.s, s);
+        const float2 q = two_sum_err2(c, o.c, c);
+        e = __fadd2_rn(__fadd2_rn(e, o.e), __fadd2_rn(q, two_sum_err2(c, r, c)));
     }
+    __device__ __forceinline__ Sum3 lo() const { return {s.x, c.x, e.x}; }
+    __device__ __forceinline__ Sum3 hi() const { return {s.y, c.y, e.y}; }
 };
+constexpr size_t kRedBytes = 3 * sizeof(float);  // shared memory that a reduction of FP32 data takes per system and thread row
 
 // Per-thread partial sums: FP64 for double data; for float data FP32 over at most 8 grid-stride steps, then folded into a
-// pair sum (a conversion and an FP64 addition per fold occupied the FP64 pipe for about 4 us of a 1023^2, 8-system dot).
+// three-word sum (a conversion and an FP64 addition per fold occupied the FP64 pipe for about 4 us of a 1023^2, 8-system dot).
 template <class T>
 struct Accum {
     static constexpr int W = VecT<T>::W;
@@ -89,11 +83,12 @@ struct Accum {
 template <>
 struct Accum<float> {
     static constexpr int W = VecT<float>::W;
-    DfSum tot[W];
+    Sum3 tot[W];
     float part[W];
-    int n;
-    __device__ Accum() : n(0) {
-        for (int v = 0; v < W; ++v) part[v] = 0.f;
+    int n;        // products since the last fold
+    bool folded;
+    __device__ Accum() : n(0), folded(false) {
+        for (int v = 0; v < W; ++v) { tot[v] = Sum3{}; part[v] = 0.f; }
     }
     __device__ __forceinline__ void add(const float (&a)[W], const float (&b)[W]) {
         for (int v = 0; v < W; ++v) part[v] = fmaf(a[v], b[v], part[v]);
@@ -102,6 +97,12 @@ struct Accum<float> {
     __device__ __forceinline__ void flush() {
         for (int v = 0; v < W; ++v) { tot[v].add(part[v]); part[v] = 0.f; }
         n = 0;
+        folded = true;
+    }
+    // the last fold; a thread that never folded holds one FP32 value
+    __device__ __forceinline__ void close() {
+        if (folded) flush();
+        else for (int v = 0; v < W; ++v) tot[v].s = part[v];
     }
 };
 
@@ -543,32 +544,75 @@ __device__ __forceinline__ void red_apply(const Red& red, Scal* S, double part, 
 template <class T>
 __device__ void reduce_finish(Accum<T>& acc, const Red& red, int Kp) {
     constexpr int W = VecT<T>::W;
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) double sm[];
     __shared__ int am_last;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     const int nthr = blockDim.x * blockDim.y;
     const int G = nthr / Kp;
     const int nblk = (int)gridDim.x;
-    double tot = 0.0;  // the block's sum of system tid < Kp; FP32 data: Df until here
-    Df td = {0.f, 0.f};
+    double tot = 0.0;  // the block's sum of system tid < Kp; FP32 data: three words until here
+    Sum3 td{};
     if constexpr (sizeof(T) == 4) {
-        Df* sd = reinterpret_cast<Df*>(sm);
-        acc.flush();
-        for (int v = 0; v < W; ++v) sd[tid * W + v] = acc.tot[v].get();  // = sd[point * Kp + system]
-        __syncthreads();
-        DfSum part;
-        if (tid < Kp * G) {
-            const int s = tid % Kp, g = tid / Kp;
-            for (int p = g; p < (int)blockDim.y; p += G) part.add(sd[p * Kp + s]);
+        // The three words of the sums in a plane each, [thread row][system]; a thread adds a pair of systems (packed) of up to
+        // four rows at a time into the first of them, until one row is left.  Eight CTAs an SM do this at the same time at the
+        // end of a light sweep, so its instructions count: where no thread has folded (at most seven products each), the first
+        // step adds plain FP32 values.
+        const int plane = (int)blockDim.y * Kp, Q = Kp / 2;
+        float* sw = reinterpret_cast<float*>(sm);
+        float2* pw = reinterpret_cast<float2*>(sm);
+        float4* own = reinterpret_cast<float4*>(sw + tid * W);
+        const bool wide = __syncthreads_or(acc.folded);
+        acc.close();
+        own[0] = make_float4(acc.tot[0].s, acc.tot[1].s, acc.tot[2].s, acc.tot[3].s);
+        if (wide) {
+            own[plane / 4] = make_float4(acc.tot[0].c, acc.tot[1].c, acc.tot[2].c, acc.tot[3].c);
+            own[plane / 2] = make_float4(acc.tot[0].e, acc.tot[1].e, acc.tot[2].e, acc.tot[3].e);
         }
+        auto step = [&](int rows, auto&& at, auto&& plus) {
+            const int m = (rows + 3) / 4;
+            __syncthreads();
+            for (int i = tid; i < m * Q; i += nthr) {
+                Sum3x2 t = at(i);
+#pragma unroll
+                for (int j = 1; j < 4; ++j)
+                    if (i + j * m * Q < rows * Q) plus(t, i + j * m * Q);
+                pw[i] = t.s;
+                pw[i + plane / 2] = t.c;
+                pw[i + plane] = t.e;
+            }
+            return m;
+        };
+        int rows = (int)blockDim.y;
+        auto all3 = [&](int k) { return Sum3x2{pw[k], pw[k + plane / 2], pw[k + plane]}; };
+        if (!wide)
+            rows = step(rows, [&](int k) { return Sum3x2{pw[k], make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; },
+                        [&](Sum3x2& t, int k) { t.add(pw[k]); });
+        // down to one row, or to 32, which the first warp adds: a lane every m-th row, then a tree over m rows
+        auto plus3 = [&](Sum3x2& t, int k) { t.add(all3(k)); };
+        while (rows > (nthr < 32 ? 1 : 32)) rows = step(rows, all3, plus3);
         __syncthreads();
-        if (tid < Kp * G) sd[tid] = part.get();
-        __syncthreads();
-        if (tid < Kp) {
-            DfSum t;
-            for (int g = 0; g < G; ++g) t.add(sd[g * Kp + tid]);
-            td = t.get();
-            tot = (double)td.h + (double)td.l;
+        if (tid < 32 && rows > 1) {
+            const int m = Q <= 2 ? 16 : Q <= 4 ? 8 : 4;
+            Sum3x2 t{};
+            if (tid < m * Q) {
+                if (tid < rows * Q) t = all3(tid);
+                for (int k = tid + m * Q; k < rows * Q; k += m * Q) plus3(t, k);
+            }
+            for (int o = m / 2 * Q; o >= Q; o >>= 1) {
+                const int from = tid + o < m * Q ? tid + o : tid;
+                auto other = [&](float2 v) { return make_float2(__shfl_sync(0xffffffffu, v.x, from), __shfl_sync(0xffffffffu, v.y, from)); };
+                t.add(Sum3x2{other(t.s), other(t.c), other(t.e)});
+            }
+            if (tid < Q) {  // (the rows were read by this warp alone)
+                pw[tid] = t.s;
+                pw[tid + plane / 2] = t.c;
+                pw[tid + plane] = t.e;
+            }
+            __syncwarp();
+        }
+        if (tid < Kp) {  // (the first warp; a smaller block has passed the barrier above)
+            td = Sum3{sw[tid], sw[tid + plane], sw[tid + 2 * plane]};
+            if (!red.defer) tot = td.value();
         }
     } else {
         for (int v = 0; v < W; ++v) sm[tid * W + v] = acc.tot[v];
@@ -587,8 +631,16 @@ __device__ void reduce_finish(Accum<T>& acc, const Red& red, int Kp) {
     if (red.defer) {
         // visible to k_red_finish, which waits for this grid to complete
         if (tid < Kp) {
-            if constexpr (sizeof(T) == 4) reinterpret_cast<Df*>(red.partial)[(size_t)blockIdx.x * Kp + tid] = td;
-            else red.partial[(size_t)blockIdx.x * Kp + tid] = tot;
+            const size_t i = (size_t)blockIdx.x * Kp + tid;
+            if constexpr (sizeof(T) == 4) {  // all first words, all second ones, all third ones
+                const size_t n = (size_t)nblk * Kp;
+                float* out = reinterpret_cast<float*>(red.partial) + i;
+                out[0] = td.s;
+                out[n] = td.c;
+                out[2 * n] = td.e;
+            } else {
+                red.partial[i] = tot;
+            }
         }
         if (tid == 0 && blockIdx.x == 0) *red.nblk = (unsigned)nblk;
         return;
@@ -1561,7 +1613,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_coarse_cluster(ClusterAr
 
 // ------------------------------------------------------------------ host launchers
 inline dim3 blk(const Launch& g) { return dim3(g.C, g.PPB); }
-inline size_t shm(const Launch& g, int W) { return (size_t)g.C * g.PPB * W * sizeof(double); }
+inline size_t shm(const Launch& g, int W) { return (size_t)g.C * g.PPB * W * (W == 4 ? kRedBytes : sizeof(double)); }
 
 #define BURA_DISPATCH(dim, var, KERNEL, ...)                                        \
     do {                                                                            \
@@ -1589,6 +1641,8 @@ inline size_t shm(const Launch& g, int W) { return (size_t)g.C * g.PPB * W * siz
 // Launch shape of the sparse sweeps: a row per thread and chunk; with a reduction one round of resident CTAs at most (and
 // no more than the buffer of block partials is sized for).
 inline dim3 csr_block(const Launch& g) { return dim3((unsigned)g.C, (unsigned)(kCsrThreads / g.C)); }
+template <class T>
+size_t csr_shm(dim3 b) { return (size_t)b.x * b.y * VecT<T>::W * (sizeof(T) == 4 ? kRedBytes : sizeof(double)); }
 inline unsigned csr_blocks(const Launch& g, const Lev& L, dim3 b, bool dot) {
     const long long tiles = (L.N + b.y - 1) / b.y;
     return (unsigned)(dot ? std::min<long long>(tiles, std::min(g.blocks, 152 * kCsrCtasDot)) : tiles);
@@ -1616,7 +1670,7 @@ void Ops<T>::spmv_q(const Launch& g, const Lev& L, int dim, bool var, const T* p
                     cudaStream_t s) {
     if (dim == 0) {
         const dim3 b = csr_block(g);
-        launch_pdl(k_csr_spmv<T>, dim3(csr_blocks(g, L, b, true)), b, (size_t)b.x * b.y * VecT<T>::W * sizeof(double), s, L, g.Kp, pa, pb,
+        launch_pdl(k_csr_spmv<T>, dim3(csr_blocks(g, L, b, true)), b, csr_shm<T>(b), s, L, g.Kp, pa, pb,
                    q, red);
         return;
     }
@@ -1643,7 +1697,7 @@ void Ops<T>::cheb_step(const Launch& g, const Lev& L, int dim, bool var, const T
         const dim3 b2 = csr_block(g);
         const bool dot = red.op != RED_NONE;
         launch_pdl(dot ? k_csr_step<T, true> : k_csr_step<T, false>, dim3(csr_blocks(g, L, b2, dot)), b2,
-                   dot ? (size_t)b2.x * b2.y * VecT<T>::W * sizeof(double) : 0, s, L, g.Kp, xin, din, b, xout, dout, cs, dsh, red);
+                   dot ? csr_shm<T>(b2) : 0, s, L, g.Kp, xin, din, b, xout, dout, cs, dsh, red);
         return;
     }
     BURA_DISPATCH_PDL(dim, var, k_cheb_step, dim3(g.blocks), blk(g), sh, s, L, g.Kp, xin, din, b, xout, dout, cs, dsh,

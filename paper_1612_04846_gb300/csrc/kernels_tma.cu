@@ -1091,7 +1091,7 @@ int ring_stages(const TmaGeo& g, int kind) {
 // Persistent grid: as many CTAs per SM as their rings fit in shared memory (at most kTmaMaxCtasPerSM, or
 // kPost2CtasPerSM for the fused post-smoothing, whose launch bounds allow more registers).
 int tma_blocks(const TmaGeo& g, int Kp, int nsm, int kind, int S) {
-    const size_t smem = dyn_smem(kind, Kp, S) + kRingSlack + kSmemReserved + 64;  // + static
+    const size_t smem = dyn_smem(kind, Kp, S) + kRingSlack + kSmemReserved + 320;  // + static
     int per_sm = (int)(kSmemPerSM / smem);
     const int cap = kind == TK_POST2 || kind == TK_POST2_V ? kPost2CtasPerSM
                     : kind == TK_PRE2R_V                   ? 2
@@ -1119,7 +1119,8 @@ Shape shape_of(const TmaGeo& g0, int nsm, int kind) {
     sh.g.stages = ring_stages(g0, kind);
     sh.blocks = tma_blocks(sh.g, g0.Kp, nsm, kind, sh.g.stages);
     sh.threads = kTmaThreads;
-    sh.smem = dyn_smem(kind, g0.Kp, sh.g.stages) + kRingSlack;
+    // (a ring of one stage of a few systems is smaller than what the reduction of a sum takes)
+    sh.smem = std::max(dyn_smem(kind, g0.Kp, sh.g.stages), kTmaThreads * 4 * kRedBytes) + kRingSlack;
     return sh;
 }
 

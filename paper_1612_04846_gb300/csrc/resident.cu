@@ -66,14 +66,7 @@ constexpr int kHR = 3, kHX = 2, kHY = 1, kHD = 2, kHP = 1;  // halo rows of R, X
 constexpr int kSP = 64;                                     // leading dimension of the sine bases
 constexpr int kStrip = 4;                                   // most rows a thread takes at a time
 
-// The CG's sums and scalars are pairs: a scalar FP64 step that all 16 warps execute costs 256 SM clocks (a reduction over
-// 16 CTAs of 512 threads: 3700 -> 2000 clocks).
-// a / b rounded to FP32 from a pair quotient (about 45 bits)
-__device__ __forceinline__ float df_div(Df a, Df b) {
-    const float q = __fdiv_rn(a.h, b.h);
-    const float r = __fadd_rn(__fmaf_rn(-q, b.h, a.h), __fmaf_rn(-q, b.l, a.l));
-    return __fadd_rn(q, __fdiv_rn(r, b.h));
-}
+// The CG's sums and scalars are three-word sums (sum3.h): a scalar FP64 step that all 16 warps execute costs 256 SM clocks.
 
 __device__ __forceinline__ unsigned map_rank(const void* p, int rank) {
     unsigned r;
@@ -92,10 +85,14 @@ __device__ __forceinline__ void put2(void* p, int rank, uint64_t* bar, float v0,
                  "f"(v0), "f"(v1), "r"(map_rank(bar, rank))
                  : "memory");
 }
-// Wait for a phase whose bytes other CTAs of the cluster store; false if they have not come within the larger of the default
-// budget and `budget`, the caller's (0: none).  A phase that takes longer than the caller's sets `late`: it is waited for all
-// the same, so that no store is in flight into a buffer that is in use again, and the CTAs of a cluster stay together.
-__device__ __forceinline__ bool wait_bytes(uint64_t* bar, unsigned parity, long long budget, bool& late) {
+__device__ __forceinline__ void put4(float4* p, int rank, uint64_t* bar, float v0, float v1, float v2) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
+                     map_rank(p, rank)),
+                 "f"(v0), "f"(v1), "f"(v2), "f"(0.f), "r"(map_rank(bar, rank))
+                 : "memory");
+}
+// Wait for a phase whose bytes other CTAs of the cluster store; false if they have not come within `budget`.
+__device__ __forceinline__ bool wait_bytes(uint64_t* bar, unsigned parity, long long budget) {
     const long long t0 = clock64();
     for (;;) {
         unsigned ok;
@@ -108,12 +105,18 @@ __device__ __forceinline__ bool wait_bytes(uint64_t* bar, unsigned parity, long 
             : "=r"(ok)
             : "r"(smem_u32(bar)), "r"(parity)
             : "memory");
-        if (ok && budget == 0) return true;
-        const long long t = clock64() - t0;
-        if (budget > 0 && t > budget) late = true;
         if (ok) return true;
-        if (t > max(budget, kTmaWaitCycles)) return false;
+        if (clock64() - t0 > budget) return false;
     }
+}
+// The same under a budget of the caller's: a phase that takes longer sets *late, and is waited for all the same, so that no
+// store is in flight into a buffer that is in use again and the CTAs of a cluster stay together.  (Not inlined: 127^2 113.2 ->
+// 112.6 us, with variable coefficients 268.7 -> 267.0.)
+__device__ __noinline__ bool wait_timed(uint64_t* bar, unsigned parity, long long budget, int* late) {
+    const long long t0 = clock64();
+    const bool come = wait_bytes(bar, parity, max(budget, kTmaWaitCycles));
+    if (clock64() - t0 > budget) *late = 1;
+    return come;
 }
 // One float from global to shared memory, asynchronously; copies_done() waits for this thread's.
 __device__ __forceinline__ void copy4(float* dst, const float* src) {
@@ -162,8 +165,9 @@ __device__ __forceinline__ float2 stencil2(float wx, float wy, float diag, float
 // rounds of items take the fewest row steps, for the own rows (kind 0) and with 1, 2 and 4 rows more (1, 2, 3).
 template <int kResWarps>
 struct Split {
-    int nch, q, m;  // column chunks; a warp's next item lies q rows of items and m chunks on
-    int h[4];
+    // (bytes: the static arrays take from the 227 KB of a CTA)
+    unsigned char nch, q, m;  // column chunks; a warp's next item lies q rows of items and m chunks on
+    unsigned char h[4];
     unsigned char s[kResWarps], ch[kResWarps];  // a warp's first item
 };
 
@@ -215,13 +219,18 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
     constexpr int kResWarps = kResThreads / 32;
     extern __shared__ __align__(16) float rsm[];
     float* const sm = rsm;
-    __shared__ double slots[2][16];      // a reduction's partial sums of every CTA (FP64, or Df pairs)
-    __shared__ double wsum[kResWarps];
+    __shared__ __align__(16) float4 slots[2][16];  // a reduction's partial sums of every CTA (a Sum3, or an FP64 value)
+    __shared__ union {
+        Limbs sum[kResWarps];            // a reduction's sums of the warps
+        int late_in[16];                 // before the first one: each CTA's copy timed out
+    } wb;
     __shared__ double bc[6];             // FP64 scalars that one warp computes for all
+    __shared__ Sum3 thr_s;               // the inner threshold
+    __shared__ float2 sum_r;             // a reduction's result
     __shared__ Split<kResWarps> split[kResMaxLevels], tsplit[VAR ? kResMaxLevels : 1];  // of the slabs; of the tail's levels
     __shared__ float coef[kResMaxLevels][3];  // c2 of the first Chebyshev step, c1 and c2 of the second
-    __shared__ int late_in[16];          // each CTA's copy timed out
     __shared__ __align__(8) uint64_t bimg, bR[kResMaxLevels], bD[kResMaxLevels], bC, bB, bV, bS[2];
+    __shared__ int late;                 // a wait outlasted the caller's budget
     cg::cluster_group cl = cg::this_cluster();
     const int tid = threadIdx.x;
     const int G = (int)cl.num_blocks(), g = (int)cl.block_rank();
@@ -229,8 +238,8 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
     Ctx<kResWarps> cx{&a, sm, g, G, tid >> 5, tid & 31};
     const int le = a.le;
     const float d = a.dsh[sys];
-    const long long budget = a.cfg->wait_cycles;  // the caller's, 0: the default
-    bool late = false;  // a wait of this thread outlasted the caller's budget
+    const long long* const budget = &a.cfg->wait_cycles;  // the caller's, 0: the default
+    const bool timed = *budget > 0;
     if (tid == 0) {
         mbar_init(&bimg, 1);
         for (int l = 0; l <= le; ++l) {
@@ -243,13 +252,15 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         mbar_init(&bS[0], 1);
         mbar_init(&bS[1], 1);
         mbar_fence_init();
-        if (!VAR) {
+        if (VAR) {
+            late = 0;
+        } else {
             mbar_expect_tx(&bimg, a.img_bytes);
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                          ::"r"(smem_u32(sm + a.o_sx)), "l"(a.img), "r"(a.img_bytes), "r"(smem_u32(&bimg))
                          : "memory");
             // a wait budget of the caller's starts at the copy's issue; the default one after the buffers are cleared
-            if (budget > 0) late = !mbar_wait_bounded(&bimg, 0, budget);
+            late = timed && !mbar_wait_bounded(&bimg, 0, *budget);
         }
     }
     __syncthreads();
@@ -267,15 +278,15 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
                 if (cost < best) { best = cost; h = q; }
             }
             Split<kResWarps>& sp = tail ? tsplit[VAR ? l : 0] : split[l];
-            sp.h[k] = h;
+            sp.h[k] = (unsigned char)h;
             for (int w = k; w < kResWarps; w += 4) {
                 sp.s[w] = (unsigned char)(w / nch);
                 sp.ch[w] = (unsigned char)(w % nch);
             }
             if (k == 0) {
-                sp.nch = nch;
-                sp.q = kResWarps / nch;
-                sp.m = kResWarps % nch;
+                sp.nch = (unsigned char)nch;
+                sp.q = (unsigned char)(kResWarps / nch);
+                sp.m = (unsigned char)(kResWarps % nch);
             }
         }
         if (!tail && l < lend && k < 3)
@@ -284,8 +295,9 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
     // everything but the bases starts at zero: the zero columns and the rows outside the grid stay zero
     for (int i = a.o_zero / 4 + tid; i < a.floats / 4; i += kResThreads)
         reinterpret_cast<float4*>(sm)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (!VAR && !mbar_wait_bounded(&bimg, 0, max(budget, kTmaWaitCycles))) late = true;  // (it lands before the kernel goes on)
-    int faulted = __syncthreads_or(late);
+    if (!VAR && !mbar_wait_bounded(&bimg, 0, max(*budget, kTmaWaitCycles))) late = 1;  // (it lands before the kernel goes on)
+    __syncthreads();
+    int faulted = late;
     if constexpr (VAR) {
         // the weights (faces negated) of the own rows and three halo rows, the tail's whole levels and its dense inverse in
         // CTA 0; 1 on the diagonal where there is no point
@@ -339,7 +351,8 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         if (tid == 0) mbar_expect_tx(bar, bytes);
     };
     auto await = [&](uint64_t* bar, unsigned& bits, int at) {
-        if (!lost && !wait_bytes(bar, (bits >> at) & 1u, budget, late)) lost = true;
+        if (!lost && !(timed ? wait_timed(bar, (bits >> at) & 1u, *budget, &late) : wait_bytes(bar, (bits >> at) & 1u, kTmaWaitCycles)))
+            lost = true;
         bits ^= 1u << at;
     };
     auto range = [&](int l) {
@@ -354,27 +367,49 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
     // (y, x) of a buffer at base + y * ld + x
     auto at = [&](int ofs, int H, const Slab& s) { return sm + ofs + (H - s.y0) * s.ld + 2; };
     int flip = 0;
-    // the sum over the cluster of every thread's v, the same bits in every thread
-    auto all_sum = [&](Df v) {
-        arm(&bS[flip], 8u * G);
+    auto tree = [](Sum3& v, int most) {  // the sum over the lanes that differ in the bits up to `most`
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v = df_add(v, df_shfl_xor(v, o));
-        Df* const ws = reinterpret_cast<Df*>(wsum);
-        if (cx.lane == 0) ws[cx.warp] = v;
-        gone = __syncthreads_or(lost);
+        for (int o = 16; o > 0; o >>= 1)
+            if (o <= most) v.add(sum3_shfl_xor(v, o));
+    };
+    // the sum over the cluster of every thread's v, formed by warp 0 of each CTA, with the same bits: use(sum) is called there
+    // and its result, and the sum rounded to FP32, are returned in every thread
+    auto all_sum = [&](Sum3 v, auto&& use) {
+        arm(&bS[flip], 16u * G);
+        Limbs l = to_limbs(v, __reduce_max_sync(0xffffffffu, limb_top(v)));
+#pragma unroll
+        for (int i = 0; i < 3; ++i) l.w[i] = __reduce_add_sync(0xffffffffu, l.w[i]);
+        if (cx.lane == 0) wb.sum[cx.warp] = l;
+        __syncthreads();
         if (cx.warp == 0) {
-            Df t = ws[cx.lane & (kResWarps - 1)];
-#pragma unroll
-            for (int o = kResWarps / 2; o > 0; o >>= 1) t = df_add(t, df_shfl_xor(t, o));
-            if (cx.lane < G) put2(&slots[flip][g], cx.lane, &bS[flip], t.h, t.l);
+            Sum3 t = from_limbs(wb.sum[cx.lane & (kResWarps - 1)]);
+            tree(t, kResWarps / 2);
+            if (cx.lane < G) put4(&slots[flip][g], cx.lane, &bS[flip], t.s, t.c, t.e);
+            await(&bS[flip], uS, flip);
+            const float4 w = slots[flip][cx.lane & 15];
+            t = (cx.lane & 15) < G ? Sum3{w.x, w.y, w.z} : Sum3{};
+            tree(t, 8);
+            const float r = use(t);
+            if (cx.lane == 0) sum_r = make_float2(r, t.s);
+        } else {
+            uS ^= 1u << flip;
         }
-        await(&bS[flip], uS, flip);
-        Df t = reinterpret_cast<Df*>(slots[flip])[cx.lane & 15];
-        if ((cx.lane & 15) >= G) t = Df{0.f, 0.f};
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) t = df_add(t, df_shfl_xor(t, o));
+        gone = __syncthreads_or(lost);
         flip ^= 1;
-        return t;
+        return sum_r;
+    };
+    // a reduction of nothing: every CTA has come here
+    auto meet = [&]() {
+        arm(&bS[flip], 16u * G);
+        __syncthreads();
+        if (cx.warp == 0) {
+            if (cx.lane < G) put4(&slots[flip][g], cx.lane, &bS[flip], 0.f, 0.f, 0.f);
+            await(&bS[flip], uS, flip);
+        } else {
+            uS ^= 1u << flip;
+        }
+        gone = __syncthreads_or(lost);
+        flip ^= 1;
     };
     // This thread's share of a . b (level 0) in the groups that the graph's kernels sum in FP32.  A system that ends after
     // one iteration returns alpha p, so another grouping, which may round alpha the other way, would show in the result's
@@ -389,13 +424,13 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         const Slab s = range(0);
         const int nx = s.nx, ny = s.ny, N = nx * ny;
         asm volatile("fence.acq_rel.cluster;" ::: "memory");
-        (void)all_sum(Df{0.f, 0.f});
+        meet();
         asm volatile("fence.acq_rel.cluster;" ::: "memory");
-        Df t{0.f, 0.f};
+        Sum3 t{};
         float v = 0.f;
         int n = 0;
         auto flush = [&]() {
-            t = df_add(t, v);
+            t.add(v);
             v = 0.f;
             n = 0;
         };
@@ -474,7 +509,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         await(&bS[flip], uS, flip);
         double t = 0.0;
         if (cx.warp == 0) {
-            t = cx.lane < G ? slots[flip][cx.lane] : 0.0;
+            t = cx.lane < G ? *reinterpret_cast<const double*>(&slots[flip][cx.lane]) : 0.0;
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
             t = __shfl_sync(0xffffffffu, t, 0);
@@ -616,7 +651,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         const float* R = at(L.oR, kHR, s);
         float *X = at(L.oX, kHX, s), *Y = at(L.oY, kHY, s), *D = at(L.oD, kHD, s);
         const float* E = at(loc ? a.tail[VAR ? l + 1 : 0].oD : a.lev[l + 1].oD, kHD, sc);
-        Df tot{0.f, 0.f};
+        Sum3 tot{};
         if (!loc) arm(&bD[l], s.halo_bytes(kHD));
         if (s.some()) {
             cx.strips(sp, 3, max(0, s.y0 - 2), min(s.ny, s.y1 + 2), nx, [&](int y, int n, int x) {
@@ -680,7 +715,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
                     p2 = __ffma2_rn(b, z, p2);
                     u = c; c = w;
                 }
-                tot = df_add(tot, p2.x + p2.y);
+                tot.add(p2.x + p2.y);
             });
         }
         __syncthreads();
@@ -789,11 +824,11 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
             put(Br + (m - own_r * a.re) * kSP + c0 + c, own_r, &bB, v);
         });
         await(&bB, uB, 0);
-        Df tot{0.f, 0.f};
+        Sum3 tot{};
         product(SX, Br, nx, nx, rows, [&](int r, float v) {
             const int y = s.y0 + r;
             D[y * ld + m] = v;
-            tot = df_add(tot, v * R[y * ld + m]);
+            tot.add(v * R[y * ld + m]);
         });
         __syncthreads();
         if (s.some())  // the edge rows, in pairs
@@ -807,7 +842,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
 
     // z = M r into D of level 0; returns this thread's part of r.z
     auto cycle = [&]() {
-        Df t{0.f, 0.f};
+        Sum3 t{};
         for (int l = 0; l < le; ++l) down(l, false);
         if constexpr (VAR) tail();
         else t = exact();
@@ -870,9 +905,9 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         const double v = __ldg(f + gofs + i);
         part = fma(v, v, part);
     }
-    if (tid < G) put(reinterpret_cast<float*>(&late_in[g]), tid, &bS[0], __int_as_float(faulted));
+    if (tid < G) put(reinterpret_cast<float*>(&wb.late_in[g]), tid, &bS[0], __int_as_float(faulted));
     const double sum_f = all_sum64(part, 4u * G);
-    for (int t = 0; t < G; ++t) faulted |= late_in[t];
+    for (int t = 0; t < G; ++t) faulted |= wb.late_in[t];
     if (tid == 0) {
         bc[0] = sum_f;
         bc[1] = bc[5] * bc[5] * sum_f;
@@ -902,12 +937,11 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
             if (cx.lane == 0) bc[4] = h;
         } else if (cx.warp == 2) {
             const double t = fmax(bc[2], 0.25 * (thr64 / rr64));
-            if (cx.lane == 0) bc[5] = t;
+            if (cx.lane == 0) thr_s = sum3_of(t);
         }
         arm(&bR[0], s0.halo_bytes(kHR));
         __syncthreads();
         const double hs = bc[3], is = bc[4];
-        const Df thr{(float)bc[5], (float)(bc[5] - (double)(float)bc[5])};
         // the inner right-hand side r / ||r|| in FP32, with its halo rows
         if (s0.some())
             cx.strips(split[0], 0, s0.y0, s0.y1, s0.nx, [&](int y, int n, int x) {
@@ -928,17 +962,19 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
             reinterpret_cast<float4*>(sm)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncthreads();
         await(&bR[0], uR, 0);
-        Df rz{1.f, 0.f};
+        Sum3 rz{1.f, 0.f, 0.f};  // (warp 0's)
         int it = 0, breakdown = 0;
         for (;;) {
             // z = M r into D
-            Df t;
-            t = cycle();
+            Sum3 t = cycle();
             if (siters == 0) t = grid_dot(L0.oR, kHR, L0.oD, kHD, true);
-            const Df rzn = all_sum(t);
-            if (!isfinite(rzn.h)) breakdown = 1;
-            const float beta = df_div(rzn, rz);
-            rz = rzn;
+            const float2 zr = all_sum(t, [&](const Sum3& s) {
+                const float q = sum3_div(s, rz);
+                rz = s;
+                return q;
+            });
+            if (!isfinite(zr.y)) breakdown = 1;
+            const float beta = zr.x;
             // p = z + beta p on the own rows and one halo row, q = (A - d I) p into Y
             const float* Z = at(L0.oD, kHD, s0);
             float* Q = at(L0.oY, kHY, s0);
@@ -951,7 +987,7 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
                         st2(o, it == 0 ? ld2(z) : __ffma2_rn(dup(beta), ld2(o), ld2(z)));
                 });
             __syncthreads();
-            t = Df{0.f, 0.f};
+            t = Sum3{};
             if (s0.some()) {
                 const Op A = op_of(L0, s0);
                 cx.strips(split[0], 0, s0.y0, s0.y1, s0.nx, [&](int y, int n, int x) {
@@ -967,17 +1003,17 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
                         p2 = __ffma2_rn(c, v, p2);  // c is zero in the padding column
                         u = c; c = w;
                     }
-                    t = df_add(t, p2.x + p2.y);
+                    t.add(p2.x + p2.y);
                 });
             }
             if (siters == 0) t = grid_dot(a.o_p, kHP, L0.oY, kHY, false);
-            const Df pq = all_sum(t);
+            const float2 pq = all_sum(t, [&](const Sum3& s) { return sum3_div(rz, s); });
             float af = 0.f;
-            if (!(pq.h > 0.f) || !isfinite(pq.h)) breakdown = 1;
-            else af = df_div(rz, pq);
+            if (!(pq.y > 0.f) || !isfinite(pq.y)) breakdown = 1;
+            else af = pq.x;
             // x += alpha p, r -= alpha q with the halo rows of r
             arm(&bR[0], s0.halo_bytes(kHR));
-            t = Df{0.f, 0.f};
+            t = Sum3{};
             if (s0.some())
                 cx.strips(split[0], 0, s0.y0, s0.y1, s0.nx, [&](int y, int n, int x) {
                     const bool last = x + 1 >= s0.nx;
@@ -994,14 +1030,14 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
                         cx.share(0, L0.oR, kHR, s0, &bR[0], y + i, x, rv);
                         p2 = __ffma2_rn(rv, rv, p2);
                     }
-                    t = df_add(t, p2.x + p2.y);
+                    t.add(p2.x + p2.y);
                 });
-            const Df rr = all_sum(t);
+            const float2 rr = all_sum(t, [&](const Sum3& s) { return sum3_le(s, thr_s) ? 1.f : 0.f; });
             await(&bR[0], uR, 0);
             ++it;
             ++siters;
-            if (!isfinite(rr.h)) breakdown = 1;
-            if (rr.h < thr.h || (rr.h == thr.h && rr.l <= thr.l) || breakdown || it >= max_iters || gone) break;
+            if (!isfinite(rr.y)) breakdown = 1;
+            if (rr.x != 0.f || breakdown || it >= max_iters || gone) break;
         }
         if (tid == 0 && g == 0) out.its[outer] = it;
         ++outer;

@@ -2397,7 +2397,9 @@ int setup_device(bura_plan* p, long long N, bura_plan** out) {
     if ((rc = dalloc(p, &p->r64, v64b)) != BURA_OK) return fail(rc);
     const size_t max_blocks = (size_t)nsm * std::max(8, o.blocks_per_sm);
     const size_t max_groups = (max_blocks + kRedGroup - 1) / kRedGroup;
-    if ((rc = dalloc(p, &p->partial, (max_blocks + max_groups) * KMAXP * sizeof(double))) != BURA_OK) return fail(rc);
+    // block partials (FP32 data: half as much again for the third words), or block and group partials
+    const size_t max_partials = max_blocks + std::max(max_groups, (max_blocks + 1) / 2);
+    if ((rc = dalloc(p, &p->partial, max_partials * KMAXP * sizeof(double))) != BURA_OK) return fail(rc);
     if ((rc = dalloc(p, &p->tickets, (max_groups + 2) * sizeof(unsigned int))) != BURA_OK) return fail(rc);
     if (cudaMemset(p->tickets, 0, (max_groups + 2) * sizeof(unsigned int)) != cudaSuccess) return fail(BURA_ECUDA);
     p->red_nblk = p->tickets + max_groups + 1;
