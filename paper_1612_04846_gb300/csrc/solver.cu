@@ -140,10 +140,10 @@ struct Work {
         bool on = false;
         Sweep3Lev geo{};
         std::vector<typename TmaLev::Ent> maps;
-        const CUtensorMap& at(int box, const void* buf) const {
+        const CUtensorMap* at(int box, const void* buf) const {  // null: no such map, and the sweep that asks reports it
             for (const auto& e : maps)
-                if (e.box == box && e.buf == buf) return e.map;
-            return maps[0].map;  // (every pair that a sweep asks for is in the list)
+                if (e.box == box && e.buf == buf) return &e.map;
+            return nullptr;
         }
     };
     std::vector<S3Lev> s3;
@@ -229,6 +229,7 @@ struct bura_plan {
     cudaGraph_t sgraph = nullptr;
     cudaGraphExec_t sexec = nullptr;
     long long s_fixed = 0, s_outer = 0, s_body = 0;  // launches: once, per refinement step, per PCG iteration
+    cudaError_t sweep_err = cudaSuccess;  // a staged 3-D sweep that was not launched
     bool res_on = false;         // the whole solve is one launch (resident.cu)
     ResArgs res{};
     bool pending = false;        // a device-driven solve's outcome has not been read into st yet
@@ -797,13 +798,14 @@ int upload_packed(bura_plan* p, const HostLevel& h, Sweep3Lev& g) {
 }
 
 // Whether level l of an FP32 work set runs the staged 3-D sweeps (kSweep3MinN points along x, half that along the other
-// axes: below, an item's fill of its ring costs more than the sweep saves), and its maps.  The buffers exist.
+// axes: below, an item's fill of its ring costs more than the sweep saves), and its maps.  The buffers exist.  Plans that ask
+// for the grid sweeps keep them.
 template <class T>
 int build_sweep3(bura_plan* p, Work<T>& w, int l) {
     const int nlev = (int)p->hl.size();
     const HostLevel& h = p->hl[l];
     auto& t = w.s3[l];
-    if (sizeof(T) != 4 || p->dim != 3 || (p->var && p->opt.smoother_bf16) || w.Kp > 16 || l + 1 >= nlev || w.deg[l] < 2 ||
+    if (sizeof(T) != 4 || p->dim != 3 || p->opt.sweeps == BURA_SWEEP_GRID || (p->var && p->opt.smoother_bf16) || w.Kp > 16 || l + 1 >= nlev || w.deg[l] < 2 ||
         h.n[0] < kSweep3MinN || std::min(h.n[1], h.n[2]) < kSweep3MinN / 2)
         return BURA_OK;
     const HostLevel& hc = p->hl[l + 1];
@@ -1337,6 +1339,7 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
     const auto& tl = w.tma[l];
     const auto& s3l = w.s3[l];
     const bool s3 = s3l.on;
+    auto note = [&](cudaError_t e) { if (e != cudaSuccess) p->sweep_err = e; };
     // one Chebyshev step, TMA-staged where the level has tensor maps
     auto cheb = [&](const T* xin, const T* din, T* xout, T* dout, ChebStepT<T> cs, const Red& red) {
         const CUtensorMap* mx = tl.on ? tl.find(TB_HALO, xin) : nullptr;
@@ -1346,9 +1349,9 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
             (void)tma_cheb_step(tl.geo, p->nsm, *mx, md, *mb, reinterpret_cast<float*>(xout),
                                 reinterpret_cast<float*>(dout), f32_step(cs), f32_ptr(w.dsh), red, s);
         else if (s3)
-            (void)sweep3_step(s3l.geo, s3l.at(S3B_HALO, xin), din ? &s3l.at(S3B_TILE, din) : nullptr, s3l.at(S3B_TILE, b),
-                              reinterpret_cast<float*>(xout), reinterpret_cast<float*>(dout), f32_step(cs), f32_ptr(w.dsh),
-                              red, s);
+            note(sweep3_step(s3l.geo, s3l.at(S3B_HALO, xin), din != nullptr, din ? s3l.at(S3B_TILE, din) : nullptr,
+                             s3l.at(S3B_TILE, b), reinterpret_cast<float*>(xout), reinterpret_cast<float*>(dout), f32_step(cs),
+                             f32_ptr(w.dsh), red, s));
         else
             Ops<T>::cheb_step(g, L, dim, var, xin, din, b, xout, dout, cs, w.dsh, red, s);
     };
@@ -1450,9 +1453,9 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
                [&] { Ops<T>::cheb_zero(g, L, dim, var, b, A, step_of(w, l, 0), w.dsh, s); });
     } else if (s3) {  // both steps from zero in one staged sweep
         traced(p, K_PRE2, f32, fine, vbytes<T>(p, l, deg > 2 ? 3.0 : 2.0, true), s, [&] {
-            (void)sweep3_pre(s3l.geo, s3l.at(S3B_HALO, b), reinterpret_cast<float*>(A),
-                             reinterpret_cast<float*>(deg > 2 ? D : nullptr), f32_step(step_of(w, l, 0)),
-                             f32_step(step_of(w, l, 1)), f32_ptr(w.dsh), none, s);
+            note(sweep3_pre(s3l.geo, s3l.at(S3B_HALO, b), reinterpret_cast<float*>(A),
+                            reinterpret_cast<float*>(deg > 2 ? D : nullptr), f32_step(step_of(w, l, 0)),
+                            f32_step(step_of(w, l, 1)), f32_ptr(w.dsh), none, s));
         });
         for (int m = 2; m < deg; ++m) {
             T* dout = m < deg - 1 ? D : nullptr;
@@ -1507,8 +1510,8 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
     // second sweep: 27 (3-D) stencil evaluations per coarse point cost more than the extra vector pass.
     if (s3) {
         traced(p, K_RESTRICT, f32, fine, vbytes<T>(p, l, 2.0, true) + vbytes<T>(p, l + 1, 1.0, false), s, [&] {
-            (void)sweep3_residual_restrict(s3l.geo, s3l.at(S3B_RHALO, cur), s3l.at(S3B_RTILE, b),
-                                           reinterpret_cast<float*>(w.b[l + 1]), f32_ptr(w.dsh), none, s);
+            note(sweep3_residual_restrict(s3l.geo, s3l.at(S3B_RHALO, cur), s3l.at(S3B_RTILE, b),
+                                          reinterpret_cast<float*>(w.b[l + 1]), f32_ptr(w.dsh), none, s));
         });
     } else if (dim == 3 || var) {
         traced(p, K_RESID, f32, fine, vbytes<T>(p, l, 3.0, true), s,
@@ -1524,9 +1527,9 @@ T* vcycle(bura_plan* p, Work<T>& w, int l, const T* b, bool rz_fused, cudaStream
     int m0 = 0;
     if (s3) {  // the correction and the first post-smoothing step in one staged sweep
         traced(p, K_PROCHEB, f32, fine, vbytes<T>(p, l, 4.0, true) + vbytes<T>(p, l + 1, 1.0, false), s, [&] {
-            (void)sweep3_prolong_step(s3l.geo, s3l.at(S3B_HALO, cur), s3l.at(S3B_COARSE, ec), s3l.at(S3B_TILE, b),
-                                      reinterpret_cast<float*>(oth), reinterpret_cast<float*>(D),
-                                      f32_step(step_of(w, l, 0, false)), f32_ptr(w.dsh), none, s);
+            note(sweep3_prolong_step(s3l.geo, s3l.at(S3B_HALO, cur), s3l.at(S3B_COARSE, ec), s3l.at(S3B_TILE, b),
+                                     reinterpret_cast<float*>(oth), reinterpret_cast<float*>(D),
+                                     f32_step(step_of(w, l, 0, false)), f32_ptr(w.dsh), none, s));
         });
         std::swap(cur, oth);
         m0 = 1;
@@ -1576,11 +1579,12 @@ int pcg_body(bura_plan* p, Work<T>& w, unsigned long long cond, cudaStream_t s) 
         if (mz && ma && mbb)
             (void)tma_spmv_p(tl.geo, p->nsm, *mz, *ma, *mbb, tl.var ? &tl.w_halo : nullptr, reinterpret_cast<float*>(w.pa),
                              reinterpret_cast<float*>(w.pb), reinterpret_cast<float*>(w.q), ralpha, s);
-        else if (s3)
-            (void)sweep3_spmv(s3l.geo, s3l.at(S3B_HALO, z), s3l.at(S3B_HALO, w.pa), s3l.at(S3B_HALO, w.pb),
-                              reinterpret_cast<float*>(w.pa), reinterpret_cast<float*>(w.pb), reinterpret_cast<float*>(w.q),
-                              ralpha, s);
-        else if (split_sweeps(p))
+        else if (s3) {
+            const cudaError_t e = sweep3_spmv(s3l.geo, s3l.at(S3B_HALO, z), s3l.at(S3B_HALO, w.pa), s3l.at(S3B_HALO, w.pb),
+                                              reinterpret_cast<float*>(w.pa), reinterpret_cast<float*>(w.pb),
+                                              reinterpret_cast<float*>(w.q), ralpha, s);
+            if (e != cudaSuccess) p->sweep_err = e;
+        } else if (split_sweeps(p))
             Ops<T>::spmv_q(g, L, p->dim, p->var, w.pa, w.pb, w.q, ralpha, s);
         else
             Ops<T>::spmv_p(g, L, p->dim, p->var, z, w.pa, w.pb, w.q, ralpha, s);
@@ -1602,6 +1606,9 @@ int pcg_body(bura_plan* p, Work<T>& w, unsigned long long cond, cudaStream_t s) 
     });
     red_finish(p, rconv, w.Kp, f32, s);
     CKL();
+    const cudaError_t missed = p->sweep_err;
+    p->sweep_err = cudaSuccess;
+    CK(missed);
     return BURA_OK;
 }
 

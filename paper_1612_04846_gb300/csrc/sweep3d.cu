@@ -446,37 +446,42 @@ cudaError_t launch3(const Sweep3Lev& g, Sweep3 a, const Red& red, cudaStream_t s
 
 }  // namespace
 
-cudaError_t sweep3_step(const Sweep3Lev& g, const CUtensorMap& x, const CUtensorMap* din, const CUtensorMap& b, float* xout,
-                        float* dout, ChebStepT<float> cs, const float* dsh, const Red& red, cudaStream_t s) {
+cudaError_t sweep3_step(const Sweep3Lev& g, const CUtensorMap* x, bool has_din, const CUtensorMap* din, const CUtensorMap* b,
+                        float* xout, float* dout, ChebStepT<float> cs, const float* dsh, const Red& red, cudaStream_t s) {
     Sweep3 a{};
-    a.v = x; a.b = b; a.out = xout; a.out2 = dout; a.c1 = cs; a.dsh = dsh; a.w = g.w;
-    a.d = din ? *din : b;
-    a.din = din ? dsh : nullptr;  // (a flag)
+    if (!x || !b || (has_din && !din)) return cudaErrorInvalidValue;
+    a.v = *x; a.b = *b; a.out = xout; a.out2 = dout; a.c1 = cs; a.dsh = dsh; a.w = g.w;
+    a.d = has_din ? *din : *b;
+    a.din = has_din ? dsh : nullptr;  // (a flag)
     return launch3<S3_STEP>(g, a, red, s);
 }
-cudaError_t sweep3_pre(const Sweep3Lev& g, const CUtensorMap& b, float* xout, float* dout, ChebStepT<float> c0,
+cudaError_t sweep3_pre(const Sweep3Lev& g, const CUtensorMap* b, float* xout, float* dout, ChebStepT<float> c0,
                        ChebStepT<float> c1, const float* dsh, const Red& none, cudaStream_t s) {
     Sweep3 a{};
-    a.v = b; a.out = xout; a.out2 = dout; a.c0 = c0; a.c1 = c1; a.dsh = dsh; a.w = g.w;
+    if (!b) return cudaErrorInvalidValue;
+    a.v = *b; a.out = xout; a.out2 = dout; a.c0 = c0; a.c1 = c1; a.dsh = dsh; a.w = g.w;
     return launch3<S3_PRE>(g, a, none, s);
 }
-cudaError_t sweep3_residual_restrict(const Sweep3Lev& g, const CUtensorMap& x, const CUtensorMap& b, float* bc, const float* dsh,
+cudaError_t sweep3_residual_restrict(const Sweep3Lev& g, const CUtensorMap* x, const CUtensorMap* b, float* bc, const float* dsh,
                                      const Red& none, cudaStream_t s) {
     Sweep3 a{};
-    a.v = x; a.b = b; a.out = bc; a.dsh = dsh; a.w = g.wr;
+    if (!x || !b) return cudaErrorInvalidValue;
+    a.v = *x; a.b = *b; a.out = bc; a.dsh = dsh; a.w = g.wr;
     return launch3<S3_RESR>(g, a, none, s);
 }
-cudaError_t sweep3_prolong_step(const Sweep3Lev& g, const CUtensorMap& x, const CUtensorMap& ec, const CUtensorMap& b,
+cudaError_t sweep3_prolong_step(const Sweep3Lev& g, const CUtensorMap* x, const CUtensorMap* ec, const CUtensorMap* b,
                                 float* xout, float* dout, ChebStepT<float> cs, const float* dsh, const Red& none,
                                 cudaStream_t s) {
     Sweep3 a{};
-    a.v = x; a.e = ec; a.b = b; a.out = xout; a.out2 = dout; a.c1 = cs; a.dsh = dsh; a.w = g.w;
+    if (!x || !ec || !b) return cudaErrorInvalidValue;
+    a.v = *x; a.e = *ec; a.b = *b; a.out = xout; a.out2 = dout; a.c1 = cs; a.dsh = dsh; a.w = g.w;
     return launch3<S3_PROL>(g, a, none, s);
 }
-cudaError_t sweep3_spmv(const Sweep3Lev& g, const CUtensorMap& z, const CUtensorMap& mpa, const CUtensorMap& mpb, float* pa,
+cudaError_t sweep3_spmv(const Sweep3Lev& g, const CUtensorMap* z, const CUtensorMap* mpa, const CUtensorMap* mpb, float* pa,
                         float* pb, float* q, const Red& red, cudaStream_t s) {
     Sweep3 a{};
-    a.v = z; a.p0 = mpa; a.p1 = mpb; a.pa = pa; a.pb = pb; a.out = q; a.w = g.w;
+    if (!z || !mpa || !mpb) return cudaErrorInvalidValue;
+    a.v = *z; a.p0 = *mpa; a.p1 = *mpb; a.pa = pa; a.pb = pb; a.out = q; a.w = g.w;
     return launch3<S3_SPMV>(g, a, red, s);
 }
 

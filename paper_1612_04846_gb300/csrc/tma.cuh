@@ -248,21 +248,22 @@ struct Sweep3Lev {
     CUtensorMap w, wr;              // variable coefficients: the packed weights, [nz + 1][ny + 1][nx + 1] float4 (the faces
                                     // below a point along x, y, z and its diagonal), with the halo boxes HALO and RHALO
 };
-// x: HALO map; din (may be null) and b: TILE maps
-cudaError_t sweep3_step(const Sweep3Lev& g, const CUtensorMap& x, const CUtensorMap* din, const CUtensorMap& b, float* xout,
-                        float* dout, ChebStepT<float> cs, const float* dsh, const Red& red, cudaStream_t s);
+// Each returns cudaErrorInvalidValue, and launches nothing, when a map that it needs is null.
+// x: HALO map; din (needed with has_din) and b: TILE maps
+cudaError_t sweep3_step(const Sweep3Lev& g, const CUtensorMap* x, bool has_din, const CUtensorMap* din, const CUtensorMap* b,
+                        float* xout, float* dout, ChebStepT<float> cs, const float* dsh, const Red& red, cudaStream_t s);
 // both pre-smoothing steps from a zero guess (d_2 into dout unless null); b: HALO map
-cudaError_t sweep3_pre(const Sweep3Lev& g, const CUtensorMap& b, float* xout, float* dout, ChebStepT<float> c0,
+cudaError_t sweep3_pre(const Sweep3Lev& g, const CUtensorMap* b, float* xout, float* dout, ChebStepT<float> c0,
                        ChebStepT<float> c1, const float* dsh, const Red& none, cudaStream_t s);
 // bc = R (b - (A - d_j I) x), full weighting; x: RHALO map, b: RTILE map
-cudaError_t sweep3_residual_restrict(const Sweep3Lev& g, const CUtensorMap& x, const CUtensorMap& b, float* bc, const float* dsh,
+cudaError_t sweep3_residual_restrict(const Sweep3Lev& g, const CUtensorMap* x, const CUtensorMap* b, float* bc, const float* dsh,
                                      const Red& none, cudaStream_t s);
 // a Chebyshev step without previous direction on x + P ec; x: HALO map, ec: the coarse level's COARSE map, b: TILE map
-cudaError_t sweep3_prolong_step(const Sweep3Lev& g, const CUtensorMap& x, const CUtensorMap& ec, const CUtensorMap& b,
+cudaError_t sweep3_prolong_step(const Sweep3Lev& g, const CUtensorMap* x, const CUtensorMap* ec, const CUtensorMap* b,
                                 float* xout, float* dout, ChebStepT<float> cs, const float* dsh, const Red& none,
                                 cudaStream_t s);
 // p = z + beta p (into the buffer the parity selects) and q = (A - d_j I) p with p . q; z, pa, pb: HALO maps
-cudaError_t sweep3_spmv(const Sweep3Lev& g, const CUtensorMap& z, const CUtensorMap& mpa, const CUtensorMap& mpb, float* pa,
+cudaError_t sweep3_spmv(const Sweep3Lev& g, const CUtensorMap* z, const CUtensorMap* mpa, const CUtensorMap* mpb, float* pa,
                         float* pb, float* q, const Red& red, cudaStream_t s);
 
 }  // namespace bura
