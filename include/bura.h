@@ -331,6 +331,8 @@ int bura_get_stats(const bura_plan* plan, bura_stats* stats);
  * Enable (1) or disable (0) per-kernel timing: every fine-level kernel launch of later solves is
  * bracketed by CUDA events recorded on the solve stream, and its duration and algorithmic bytes are
  * accumulated per kernel type.  Enabling resets the counters.  Costs one event pair per launch.
+ * A profiled solve launches the kernels of the plan's ordinary solve one by one from the host; the solve of a small
+ * 2-D plan, which is one launch and its output stage, is two entries (resident_solve_f32, resident_output).
  */
 int bura_set_profiling(bura_plan* plan, int enable);
 

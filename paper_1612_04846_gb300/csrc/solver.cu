@@ -47,7 +47,7 @@ struct HostLevel {
 // Kernel types for launch counting and per-kernel timing (fine level only).
 enum KId { K_SPMV, K_CGUPD, K_CHEB0, K_CHEB, K_RESTRICT, K_PRE2, K_PROLONG, K_COARSE, K_DOT, K_BCAST, K_NORM,
            K_RES64, K_CAST, K_CORR64, K_WSUM, K_GATHER, K_CLUSTER, K_PRE2R, K_PROCHEB, K_RESDF, K_CASTDF, K_REDFIN,
-                  K_POST2, K_RESID, K_PUPD, K_FDIAG, K_POST2S, K_RESV, K_NK };
+           K_POST2, K_RESID, K_PUPD, K_FDIAG, K_POST2S, K_RESV, K_RES, K_RESOUT, K_NK };
 // [kernel][f32][coarser level]
 const char* const kNames[K_NK][2][2] = {
     {{"spmv_p_f64", "spmv_p_f64@coarse"}, {"spmv_p_f32", "spmv_p_f32@coarse"}},
@@ -77,7 +77,9 @@ const char* const kNames[K_NK][2][2] = {
     {{"p_update_f64", "p_update_f64"}, {"p_update_f32", "p_update_f32"}},
     {{"coarse_fdiag_f64", "coarse_fdiag_f64@coarse"}, {"coarse_fdiag_f32", "coarse_fdiag_f32@coarse"}},
     {{"post2_strip_f64", "post2_strip_f64@coarse"}, {"post2_strip_f32", "post2_strip_f32@coarse"}},
-    {{"coarse_resident_f64", "coarse_resident_f64@coarse"}, {"coarse_resident_f32", "coarse_resident_f32@coarse"}}};
+    {{"coarse_resident_f64", "coarse_resident_f64@coarse"}, {"coarse_resident_f32", "coarse_resident_f32@coarse"}},
+    {{"resident_solve_f64", "resident_solve_f64"}, {"resident_solve_f32", "resident_solve_f32"}},
+    {{"resident_output", "resident_output"}, {"resident_output", "resident_output"}}};
 constexpr int kSlots = K_NK * 4;
 
 struct Tracer {
@@ -2708,8 +2710,14 @@ int enqueue_device_solve(bura_plan* p, const double* f, double* u, double* V, do
     if (!(tol > 0)) return BURA_EINVAL;
     CK(cudaSetDevice(p->dev));
     if (p->res_on) {
-        CK(launch_resident(p->res, p->K, f, tol, s));
-        CK(launch_resident_out(p->res, p->K, p->cdev, u, V, accumulate, p->hstate, s));
+        const double N = (double)p->hl[0].N, vb = N * p->K * 8.0;
+        cudaError_t e = cudaSuccess;
+        p->tr.launches = 0;
+        traced(p, K_RES, true, true, N * 8.0 + vb, s, [&] { e = launch_resident(p->res, p->K, f, tol, s); });
+        CK(e);
+        traced(p, K_RESOUT, false, true, V ? 2.0 * vb : vb + N * 8.0 * (accumulate ? 2.0 : 1.0), s,
+               [&] { e = launch_resident_out(p->res, p->K, p->cdev, u, V, accumulate, p->hstate, s); });
+        CK(e);
         CK(cudaEventRecord(p->done, s));
         p->pending = true;
         return BURA_OK;
@@ -2725,12 +2733,21 @@ int enqueue_device_solve(bura_plan* p, const double* f, double* u, double* V, do
     return BURA_OK;
 }
 
+// The same, to its end.  A one-launch solve is this with profiling on too (its launches timed), so that a profile is of
+// the kernels that the plan's solves run.
+int run_device_solve(bura_plan* p, const double* f, double* u, double* V, double tol, cudaStream_t s, int accumulate) {
+    CA(enqueue_device_solve(p, f, u, V, tol, s, accumulate));
+    const int rc = read_outcome(p);
+    if (p->tr.on) {
+        CK(cudaStreamSynchronize(s));
+        collect_trace(p);
+    }
+    return rc;
+}
+
 // The solve and the output sum u = sum_j c_j v_j (accumulate = 1: u += ...), stream-ordered on s.
 int solve_into(bura_plan* p, const double* f, double* u, double tol, cudaStream_t s, int accumulate) {
-    if (device_driven(p)) {
-        CA(enqueue_device_solve(p, f, u, nullptr, tol, s, accumulate));
-        return read_outcome(p);
-    }
+    if (device_driven(p) || p->res_on) return run_device_solve(p, f, u, nullptr, tol, s, accumulate);
     int rc = solve_core(p, f, tol, s);
     if (rc != BURA_OK && rc != BURA_ENOCONV) return rc;
     const double N = (double)p->hl[0].N;
@@ -2845,10 +2862,7 @@ int bura_solve_host(bura_plan* p, const double* f, double* u, double tol, void* 
 int bura_solve_systems(bura_plan* p, const double* f, double* V, double tol, void* stream) {
     if (!p || !f || !V) return BURA_EINVAL;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    if (device_driven(p)) {
-        CA(enqueue_device_solve(p, f, nullptr, V, tol, s, 0));
-        return read_outcome(p);
-    }
+    if (device_driven(p) || p->res_on) return run_device_solve(p, f, nullptr, V, tol, s, 0);
     int rc = solve_core(p, f, tol, s);
     if (rc != BURA_OK && rc != BURA_ENOCONV) return rc;
     traced(p, K_GATHER, false, true, 2.0 * p->hl[0].N * p->K * 8.0, s, [&] {
