@@ -411,14 +411,20 @@ __global__ void __launch_bounds__(kResThreads, 512 / kResThreads) k_resident(con
         gone = __syncthreads_or(lost);
         flip ^= 1;
     };
-    // This thread's share of a . b (level 0) in the groups that the graph's kernels sum in FP32.  A system that ends after
+    // This thread's share of a . b (level 0) in the groups that other kernels of the same solve sum in FP32, so that a plan's
+    // result does not depend on which of the two solves it.  A system that ends after
     // one iteration returns alpha p, so another grouping, which may round alpha the other way, would show in the result's
     // eighth digit (small powers, whose largest shifts converge at once: one plan of 32 in ten batches).  Taken in the first
     // iteration only, later ones correct such a difference (the cost: 63^2 47 -> 48 us, 383 x 255, k = 8, 282 -> 330, 32
     // mixed problems 2.51 -> 2.81 ms).  A group's values are read from the CTAs
     // that own their rows, behind a reduction used as a barrier: unlike a cluster barrier it is bounded, and a CTA that gave
-    // up keeps its shared memory until all are done.
-    //   one exact solve, or variable coefficients: points P and P + 64, P in the even runs of 64 (the grid sweeps)
+    // up keeps its shared memory until all are done.  A change of the other kernels' tiles, blocks or threads changes their
+    // groups: tests/test_gpu_resident_groups.py compares the two.
+    //   one exact solve: points P and P + 64, P in the even runs of 64 (the grid kernels of the graph, whose whole cycle is
+    //     that solve)
+    //   variable coefficients: the same, the groups of the grid sweeps (BURA_SWEEP_GRID).  Larger variable-coefficient plans
+    //     run the TMA-staged sweeps, whose groups are other ones: with a ring depth set (which keeps the graph) a small plan
+    //     takes those, and such a system may differ by 4e-8
     //   else: the points of a thread of k_spmv_tma, or, with rz, of k_post2_tma, up to eight at a time
     auto grid_dot = [&](int oa, int Ha, int ob, int Hb, bool rz) {
         const Slab s = range(0);
