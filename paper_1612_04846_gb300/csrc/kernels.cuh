@@ -258,8 +258,8 @@ cudaError_t fdiag_prepare(int nx, int ny, int nsys, int* G, size_t* smem);
 template <class T>
 cudaError_t fdiag_launch(const FdiagArgs& a, int G, size_t smem, int nsys, cudaStream_t s);
 
-// A whole mixed-precision solve of a small 2-D constant-coefficient plan in one launch (resident.cu): a
-// thread-block cluster per system runs the refinement and CG loops on vectors kept in shared memory.
+// A whole mixed-precision solve of a small 2-D plan in one launch (resident.cu): a thread-block cluster per system runs the
+// refinement and CG loops on vectors kept in shared memory.
 constexpr int kResMaxLevels = 10;
 constexpr int kResMaxOuter = 64;                 // refinement steps whose iteration counts a record holds
 constexpr size_t kResSmemMax = 230400;           // dynamic shared memory of a CTA (227 KB less the static arrays)

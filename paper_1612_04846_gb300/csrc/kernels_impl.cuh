@@ -556,7 +556,8 @@ __device__ void reduce_finish(Accum<T>& acc, const Red& red, int Kp) {
         // The three words of the sums in a plane each, [thread row][system]; a thread adds a pair of systems (packed) of up to
         // four rows at a time into the first of them, until one row is left.  Eight CTAs an SM do this at the same time at the
         // end of a light sweep, so its instructions count: where no thread has folded (at most seven products each), the first
-        // step adds plain FP32 values.
+        // step adds plain FP32 values.  1023^2, 8 systems, pairs of FP32 words -> three (ncu): cg_update 27.8 -> 29.2 us, post2
+        // 39.0 -> 39.7, spmv 23.1 -> 23.5 (with every step through shared memory 28.8 to 30.4, 40.0 and 23.7).
         const int plane = (int)blockDim.y * Kp, Q = Kp / 2;
         float* sw = reinterpret_cast<float*>(sm);
         float2* pw = reinterpret_cast<float2*>(sm);
@@ -1097,7 +1098,7 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_min_blocks<DIM, VAR>()) k
 // gathered vectors), so they take as many rows at once as fit: one row per thread and chunk, every row of the matrix in
 // flight or waiting for an SM (the general sweep ran 6 of its 8 CTAs per SM first and 2 after them), 64 registers, the
 // columns and values of eight entries loaded before the first gather.  The sums keep the order of the entries.  P1 elements
-// on 63^3, 8 systems, 35 iterations of degree 8: 4.70 -> 3.86 ms; 512 threads a CTA: 4.05; 128, two gathers at a time: 4.38;
+// on 63^3, 8 systems, 35 iterations of degree 8: 4.70 -> 3.82 ms; 512 threads a CTA: 4.05; 128, two gathers at a time: 4.38;
 // the general sweep (two rows a thread) with a batch of four or eight: 4.99, 5.51.
 constexpr int kCsrThreads = 256, kCsrBatch = 8;
 constexpr int kCsrCtas = 4, kCsrCtasDot = 3;  // per SM; the accumulators of a reduction do not fit 64 registers

@@ -17,7 +17,7 @@
 // more load per tile brings the weights, packed as a float4 per point (the faces below it along x and y, its diagonal) that
 // all systems of the tile share.  k_pre2_restrict_tma then keeps the first iterate c2 Dinv b of the tile in shared memory
 // (a division per point instead of one per use) and runs two CTAs per SM.  The grid kernels' nine passes a level were
-// launch-bound at 511^2 and read the weights through L1 per thread: 511^2, k = 7: 3.79 -> 2.90 ms; 1023^2: 11.4 -> 6.8;
+// launch-bound at 511^2 and read the weights through L1 per thread: 511^2, k = 7: 3.79 -> 2.80 ms; 1023^2: 11.4 -> 6.8;
 // 447 x 255, k = 9: 5.17 -> 3.05.
 #include <cudaTypedefs.h>
 

@@ -31,15 +31,15 @@
 //
 // The exact solve of level le is fdiag.cu's fast diagonalization, every sum in the same order.
 //
-// Measured (GB300, one solve, tol 1e-6, graph of kernels -> here): 63^2, k = 5: 168 -> 45 us; 127^2, k = 6: 372 -> 100;
-// 255^2, k = 7: 550 -> 201; 383 x 255, k = 8: 812 -> 330.  What is left is latency: a 127^2 iteration is 9.5 us, of
-// which the exact solve's four products and three exchanges take 3.6.
+// Measured (GB300, one call of bura_solve, alpha = 0.5, tol 1e-6, graph of kernels -> here): 63^2, k = 5: 168 -> 49 us; 127^2,
+// k = 6: 418 -> 120; 255^2, k = 7: 539 -> 233; 383 x 255, k = 8: 883 -> 405.  What is left is latency: a 127^2 iteration is
+// some 10 us, of which the exact solve's four products and three exchanges take 3.6; the warps issue in 18 % of the cycles.
 //
 // Variable coefficients: every level's face and diagonal weights stay in the owner's shared memory too (three floats a
 // point, so the largest grid is about 2 / 3 as wide), copied in while the first residual is taken.  The exact level is one
 // dense product per system; grids above 31 put their last levels on the cluster's first CTA, which then runs them without
-// an exchange (a boundary at 15 instead: 127^2 376 -> 403 us, and 191^2 no longer fits).  63^2, k = 5: 1477 -> 279 us;
-// 127^2, k = 6: 2198 -> 376; 191^2: 2819 -> 503.
+// an exchange (a boundary at 15 instead: 127^2 7 % slower, and 191^2 no longer fits).  63^2, k = 5: 945 -> 211 us; 127^2,
+// k = 6: 1240 -> 276; 191^2: 1919 -> 387.
 //
 // V-cycle only: an iteration of a larger plan launches its levels from the first one of at most kResCycleMaxN points a
 // side here.  About 10 of the launch's 25 us are its start (loading weights and tables), so it takes the place of five or

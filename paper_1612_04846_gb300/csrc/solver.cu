@@ -121,8 +121,8 @@ struct Work {
     size_t fd_smem = 0;
     T* dsh = nullptr;  // the shifts d_j (KMAXP entries) in the kernels' precision
     Scal* scal = nullptr;
-    // TMA-staged sweeps (FP32, 2-D, constant coefficients) of the levels with at least one tile per SM:
-    // tensor maps of the level's vectors, with a halo box (stencil inputs) and a plain box
+    // TMA-staged sweeps (FP32, 2-D) of the levels above the coarse kernel's: tensor maps of the level's vectors, with a
+    // halo box (stencil inputs) and a plain box
     struct TmaLev {
         bool on = false;
         TmaGeo geo{};
@@ -558,8 +558,7 @@ int pack_weights2(bura_plan* p, const Lev& L, CUtensorMap& rsrc, CUtensorMap& ha
     return BURA_OK;
 }
 
-// Tensor maps for the TMA-staged sweeps: FP32, 2-D, levels that the grid
-// kernels would run (not the coarse kernel's) with at least one tile per SM.
+// Tensor maps for the TMA-staged sweeps: FP32, 2-D, every level that the grid kernels would run (not the coarse kernel's).
 template <class T>
 int build_tma(bura_plan* p, Work<T>& w) {
     const int nlev = (int)p->hl.size();
