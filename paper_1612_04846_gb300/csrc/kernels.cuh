@@ -128,7 +128,7 @@ struct Red {
 // partials in block order and applies op; launched right after the producer on the same stream.
 constexpr int kRedFinishThreads = 256;
 constexpr int kRedFinishThreads32 = 512;  // FP32 data, whose partials are three words: all of 8 systems x 1280 blocks in flight
-constexpr int kRedFinBatch32 = 10, kRedFinBatchFew = 4;  // blocks loaded at once per thread; ... of a small grid
+constexpr int kRedFinBatch32 = 10, kRedFinBatchFew = 5;  // blocks loaded at once per thread; ... of a small grid
 void launch_red_finish(const Red& red, int Kp, bool f32, cudaStream_t s);
 
 // One level of the single-CTA coarse V-cycle: its vectors live in the CTA's shared memory at the

@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kSweepThreads, 2)
         c0[q] = VAR ? dfv{0.f, 0.f} : dfv{op.ch[off + q], op.cl[off + q]};
         dd[q] = VAR ? dfv{op.dh[off + q], op.dl[off + q]} : dfv{0.f, 0.f};
     }
-    Accum<float> acc;
+    AccumG<float> acc;
     const int b0 = blockIdx.x, nb = gridDim.x;
     BURA_SWEEP(L.N) {
         const Coord c = coord<DIM>(L, P);

@@ -222,17 +222,17 @@ __global__ void __launch_bounds__(F32 ? kRedFinishThreads32 : kRedFinishThreads)
             sd[2 * tid + 1] = part.hi();
         }
         __syncthreads();
-        __shared__ double total[KMAXP];
+        __shared__ Sum3 total[KMAXP];  // (converted by one warp below: an FP64 step takes 16 clocks a warp)
         const int lane = tid & 31;
         for (int q = tid >> 5; q < Kp; q += kThreads / 32) {  // (sd[group * Kp + system])
             Sum3 t{};
             for (int h = lane; h < G; h += 32) t.add(sd[h * Kp + q]);
 #pragma unroll
             for (int o = 16; o; o >>= 1) t.add(sum3_shfl_xor(t, o));
-            if (lane == 0) total[q] = t.value();
+            if (lane == 0) total[q] = t;
         }
         __syncthreads();
-        if (tid < 32) red_ops(red, &sc, tid, tid < Kp ? total[tid] : 0.0, Kp);
+        if (tid < 32) red_ops(red, &sc, tid, tid < Kp ? total[tid].value() : 0.0, Kp);
     } else {
         red_apply(red, &sc, red_thread_sum(red.partial, nblk, Kp), Kp, sm);  // its first barrier publishes the copy
     }

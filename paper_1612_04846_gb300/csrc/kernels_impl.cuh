@@ -99,12 +99,58 @@ struct Accum<float> {
         n = 0;
         folded = true;
     }
-    // the last fold; a thread that never folded holds one FP32 value
-    __device__ __forceinline__ void close() {
+    // The thread's sums into its slots of the three planes of words at `own` (plane / 4 float4 each), after the last fold.  A
+    // thread that never folded holds one FP32 value: the first words; then, if any thread of the block folded, the others.
+    __device__ __forceinline__ void store_first(float4* own) {
         if (folded) flush();
         else for (int v = 0; v < W; ++v) tot[v].s = part[v];
+        own[0] = make_float4(tot[0].s, tot[1].s, tot[2].s, tot[3].s);
+    }
+    __device__ __forceinline__ void store_rest(float4* own, int plane) {
+        own[plane / 4] = make_float4(tot[0].c, tot[1].c, tot[2].c, tot[3].c);
+        own[plane / 2] = make_float4(tot[0].e, tot[1].e, tot[2].e, tot[3].e);
     }
 };
+// The same with the sums in shared memory, in the slots that the block's reduction takes them from (the dynamic shared memory
+// of a grid sweep is the reduction's alone): they are touched at every eighth product only, and cost a sweep's loads no
+// registers (511^2, 8 systems: cg_update 12.3 -> 11.2 us; the sparse step with r.z no longer spills them).
+struct AccumShared {
+    static constexpr int W = 4;
+    float part[W];
+    int n;
+    bool folded;
+    __device__ AccumShared() : n(0), folded(false) {
+        for (int v = 0; v < W; ++v) part[v] = 0.f;
+    }
+    __device__ __forceinline__ void add(const float (&a)[W], const float (&b)[W]) {
+        for (int v = 0; v < W; ++v) part[v] = fmaf(a[v], b[v], part[v]);
+        if (++n == 8) flush();
+    }
+    __device__ __forceinline__ void flush() {
+        extern __shared__ __align__(16) double sm[];
+        const int plane = (int)(blockDim.x * blockDim.y);  // in float4
+        float4* own = reinterpret_cast<float4*>(sm) + threadIdx.y * blockDim.x + threadIdx.x;
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 s = folded ? own[0] : z, c = folded ? own[plane] : z, e = folded ? own[2 * plane] : z;
+        Sum3 t[W] = {{s.x, c.x, e.x}, {s.y, c.y, e.y}, {s.z, c.z, e.z}, {s.w, c.w, e.w}};
+        for (int v = 0; v < W; ++v) { t[v].add(part[v]); part[v] = 0.f; }
+        own[0] = make_float4(t[0].s, t[1].s, t[2].s, t[3].s);
+        own[plane] = make_float4(t[0].c, t[1].c, t[2].c, t[3].c);
+        own[2 * plane] = make_float4(t[0].e, t[1].e, t[2].e, t[3].e);
+        n = 0;
+        folded = true;
+    }
+    __device__ __forceinline__ void store_first(float4* own) {
+        if (folded) flush();
+        else own[0] = make_float4(part[0], part[1], part[2], part[3]);
+    }
+    __device__ __forceinline__ void store_rest(float4* own, int plane) {
+        if (!folded) own[plane / 4] = own[plane / 2] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+};
+template <class T> struct GridAccum { using type = Accum<T>; };
+template <> struct GridAccum<float> { using type = AccumShared; };
+template <class T> using AccumG = typename GridAccum<T>::type;
 
 struct Coord { int i, j, l; };
 
@@ -541,8 +587,8 @@ __device__ __forceinline__ void red_apply(const Red& red, Scal* S, double part, 
 // Block reduction of per-thread partials (W systems per thread, chunk = threadIdx.x) followed by
 // the grid reduction in the last block, or, for a deferred reduction, by k_red_finish.  Every thread
 // of the block must call this.
-template <class T>
-__device__ void reduce_finish(Accum<T>& acc, const Red& red, int Kp) {
+template <class T, class A>
+__device__ void reduce_finish(A& acc, const Red& red, int Kp) {
     constexpr int W = VecT<T>::W;
     extern __shared__ __align__(16) double sm[];
     __shared__ int am_last;
@@ -556,22 +602,21 @@ __device__ void reduce_finish(Accum<T>& acc, const Red& red, int Kp) {
         // The three words of the sums in a plane each, [thread row][system]; a thread adds a pair of systems (packed) of up to
         // four rows at a time into the first of them, until one row is left.  Eight CTAs an SM do this at the same time at the
         // end of a light sweep, so its instructions count: where no thread has folded (at most seven products each), the first
-        // step adds plain FP32 values.  1023^2, 8 systems, pairs of FP32 words -> three (ncu): cg_update 27.8 -> 29.2 us, post2
-        // 39.0 -> 39.7, spmv 23.1 -> 23.5 (with every step through shared memory 28.8 to 30.4, 40.0 and 23.7).
+        // step adds plain FP32 values.  Pairs of FP32 words -> three, ncu at 511^2: 8 systems cg_update 11.1 -> 11.2 us, spmv 11.6
+        // -> 11.5, post2 15.4 -> 15.5; 13 systems 17.2 -> 17.7, 15.2 -> 16.0, 18.7 -> 18.8 (with every step through shared
+        // memory, 8 systems at 1023^2: cg_update 27.8 -> 29.6, post2 39.0 -> 40.0).
         const int plane = (int)blockDim.y * Kp, Q = Kp / 2;
         float* sw = reinterpret_cast<float*>(sm);
         float2* pw = reinterpret_cast<float2*>(sm);
         float4* own = reinterpret_cast<float4*>(sw + tid * W);
+        acc.store_first(own);
         const bool wide = __syncthreads_or(acc.folded);
-        acc.close();
-        own[0] = make_float4(acc.tot[0].s, acc.tot[1].s, acc.tot[2].s, acc.tot[3].s);
         if (wide) {
-            own[plane / 4] = make_float4(acc.tot[0].c, acc.tot[1].c, acc.tot[2].c, acc.tot[3].c);
-            own[plane / 2] = make_float4(acc.tot[0].e, acc.tot[1].e, acc.tot[2].e, acc.tot[3].e);
+            acc.store_rest(own, plane);
+            __syncthreads();
         }
         auto step = [&](int rows, auto&& at, auto&& plus) {
             const int m = (rows + 3) / 4;
-            __syncthreads();
             for (int i = tid; i < m * Q; i += nthr) {
                 Sum3x2 t = at(i);
 #pragma unroll
@@ -581,6 +626,7 @@ __device__ void reduce_finish(Accum<T>& acc, const Red& red, int Kp) {
                 pw[i + plane / 2] = t.c;
                 pw[i + plane] = t.e;
             }
+            __syncthreads();
             return m;
         };
         int rows = (int)blockDim.y;
@@ -591,7 +637,6 @@ __device__ void reduce_finish(Accum<T>& acc, const Red& red, int Kp) {
         // down to one row, or to 32, which the first warp adds: a lane every m-th row, then a tree over m rows
         auto plus3 = [&](Sum3x2& t, int k) { t.add(all3(k)); };
         while (rows > (nthr < 32 ? 1 : 32)) rows = step(rows, all3, plus3);
-        __syncthreads();
         if (tid < 32 && rows > 1) {
             const int m = Q <= 2 ? 16 : Q <= 4 ? 8 : 4;
             Sum3x2 t{};
@@ -753,7 +798,7 @@ __device__ __forceinline__ void sw_cheb_zero(const Lev& L, int Kp, const T* b, T
 template <class T, int DIM, bool VAR, class LD>
 __device__ __forceinline__ void sw_cheb_step(const Lev& L, int Kp, const LD& ld, const T* din, bool din_is_x,
                                              const T* b, T* xout, T* dout, ChebStepT<T> cs, const T* dsh,
-                                             Accum<T>* acc, int b0, int nb) {
+                                             AccumG<T>* acc, int b0, int nb) {
     constexpr int W = VecT<T>::W;
     const int off = threadIdx.x * W;
     T c1[W], c2[W], d[W];
@@ -930,7 +975,7 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_min_blocks<DIM, VAR>()) k
         ld.beta[v] = scal_val<T>(red.scal->beta, red.scal->betaf, off + v);
         dsh[v] = scal_val<T>(red.scal->dsh, red.scal->dshf, off + v);
     }
-    Accum<T> acc;
+    AccumG<T> acc;
     sweep_u<StencilState<T>>(
         L.N, b0, nb, [&](int P, StencilState<T>& st) { stencil<T, DIM, VAR>(L, Kp, P, off, ld, st.xc, st.Ax, st.diag); },
         [&](int P, StencilState<T>& st) {
@@ -986,7 +1031,7 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_min_blocks<DIM, VAR>()) k
     LoadPlain<T> ld{p};
     T dsh[W];
     for (int v = 0; v < W; ++v) dsh[v] = scal_val<T>(red.scal->dsh, red.scal->dshf, off + v);
-    Accum<T> acc;
+    AccumG<T> acc;
     if constexpr (DIM == 3) {
         zmarch<T, VAR>(L, Kp, p, blockIdx.x, gridDim.x, [&](int, size_t base, const T(&xc)[W], const T(&Ax)[W], T) {
             T qv[W];
@@ -1019,7 +1064,7 @@ __global__ void __launch_bounds__(kSweepThreads, kSweepMinBlocks) k_cg_update(in
     const T* __restrict__ p = red.scal->parity ? pa : pb;  // the direction k_spmv_p just wrote
     T a[W];
     for (int v = 0; v < W; ++v) a[v] = scal_val<T>(red.scal->alpha, red.scal->alphaf, off + v);
-    Accum<T> acc;
+    AccumG<T> acc;
     struct St { T xv[VecT<T>::W], rv[VecT<T>::W], pv[VecT<T>::W], qv[VecT<T>::W]; };
     sweep_u<St>(
         N, b0, nb,
@@ -1058,7 +1103,7 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_min_blocks<DIM, VAR>()) k
                             const T* __restrict__ dsh, Red red) {
     pdl_wait();
     LoadPlain<T> ld{xin};
-    Accum<T> acc;
+    AccumG<T> acc;
     const bool dot = red.op != RED_NONE;
     if constexpr (DIM == 3) {
         constexpr int W = VecT<T>::W;
@@ -1140,7 +1185,7 @@ __global__ void __launch_bounds__(kCsrThreads, DOT ? kCsrCtasDot : kCsrCtas) k_c
     pdl_wait();
     constexpr int W = VecT<T>::W;
     const int off = threadIdx.x * W;
-    Accum<T> acc;
+    AccumG<T> acc;
     for (long long t = (long long)blockIdx.x * blockDim.y + threadIdx.y; t < L.N; t += (long long)gridDim.x * blockDim.y) {
         const int P = (int)t;
         const size_t base = (size_t)P * Kp + off;
@@ -1171,7 +1216,7 @@ __global__ void __launch_bounds__(kCsrThreads, kCsrCtasDot) k_csr_spmv(Lev L, in
     constexpr int W = VecT<T>::W;
     const int off = threadIdx.x * W;
     const T* __restrict__ p = red.scal->parity ? pa : pb;
-    Accum<T> acc;
+    AccumG<T> acc;
     for (long long t = (long long)blockIdx.x * blockDim.y + threadIdx.y; t < L.N; t += (long long)gridDim.x * blockDim.y) {
         const int P = (int)t;
         const size_t base = (size_t)P * Kp + off;
@@ -1209,7 +1254,7 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_min_blocks<DIM, VAR>()) k
     pdl_wait();
     constexpr int W = VecT<T>::W;
     LoadProlong<T, DIM> ld{Lf, Lc, Kp, (int)threadIdx.x * W, x, ec};
-    Accum<T> acc;
+    AccumG<T> acc;
     const bool dot = red.op != RED_NONE;
     sw_cheb_step<T, DIM, VAR>(Lf, Kp, ld, nullptr, false, b, xout, dout, cs, dsh, dot ? &acc : nullptr, blockIdx.x,
                               gridDim.x);
@@ -1373,7 +1418,7 @@ __global__ void __launch_bounds__(kSweepThreads, kSweepMinBlocks) k_dot(int N, i
     constexpr int W = VecT<T>::W;
     const int off = threadIdx.x * W;
     const int b0 = blockIdx.x, nb = gridDim.x;
-    Accum<T> acc;
+    AccumG<T> acc;
     struct St { T av[VecT<T>::W], bv[VecT<T>::W]; };
     sweep_u<St>(
         N, b0, nb,

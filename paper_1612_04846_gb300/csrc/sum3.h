@@ -11,8 +11,8 @@
 // the FP32 products they come from are.
 //
 // Against pairs of FP32 values (48 bits, one renormalisation an addition), which this replaces, with the block partials half
-// as large again and one barrier more in the one-launch solves: 1023^2, k = 7, 1858 -> 1886 us; sums over 511^2 plans 2609 ->
-// 2724; variable 511^2 2.85 -> 2.91 ms; sparse 63^3 3.70 -> 3.81; 63^2 48.5 -> 49.0; 383 x 255 335 -> 337; the results are the
+// as large again and one barrier more in the one-launch solves: 1023^2, k = 7, 1857 -> 1873 us; sums over 511^2 plans 2609 ->
+// 2677; variable 511^2 2302 -> 2325; sparse 63^3 3773 -> 3800; 63^2 48.5 -> 49.8; 383 x 255 334 -> 339; the results are the
 // same bit for bit.  FP64 throughout: 1023^2 1958, sums 2958.
 #pragma once
 #include <math.h>
