@@ -151,7 +151,7 @@ class ClockSampler:
 # Per workload of profiles/ncu_traffic.json: the sources of the kernels whose DRAM traffic it records
 # (device code and the headers it includes).  Host-only files and the sources of other kernels do not
 # change the recorded traffic, so they are not hashed.
-TRAFFIC_SOURCES = {"2d_1023_k7": ("kernels_f32.cu", "kernels_tma.cu", "kernels.cuh", "kernels_impl.cuh", "tma.cuh")}
+TRAFFIC_SOURCES = {"2d_1023_k7": ("kernels_f32.cu", "kernels_tma.cu", "kernels.cuh", "kernels_impl.cuh", "sum3.h", "tma.cuh")}
 
 
 def sources_sha(workload="2d_1023_k7"):

@@ -22,9 +22,10 @@
 // Measured on the fine level of a 255^3, k = 9 solve with variable coefficients (one vector is 796 MB with its padding),
 // one launch, against the passes each replaces (per-thread cp.async staging or grid sweeps): PRE 0.48 ms (0.27 + 0.60),
 // RESR 0.44 (0.52 + 0.21), PROL 0.63 (0.37 + 0.60), STEP 0.53 (0.65), SPMV 0.57 (0.37 + 0.59); the solve 148.5 -> 107.3 ms.
-// STEP, PROL and SPMV run at 5.9 to 6.4 TB/s of DRAM traffic, the copy peak; PRE and RESR, with half the vectors per
-// point, are bound by instruction issue.  With the copies and their addresses done by the threads the same five passes
-// issued 3 to 4 times the instructions (PRE 460 per warp and chunk) and were no faster than the passes they replace.
+// STEP, PROL and SPMV run at 5.7 to 6.7 TB/s of DRAM traffic (ncu; a plain copy 6.8); PRE and RESR, with half the vectors
+// per point, move 3.3 to 4.6 and wait for shared memory and the plane's barrier (half to 58 % of the issue slots taken).
+// With the copies and their addresses done by the threads the same five passes issued 3 to 4 times the instructions (PRE
+// 460 per warp and chunk) and were no faster than the passes they replace.
 #include "kernels_impl.cuh"
 #include "tma.cuh"
 
