@@ -104,7 +104,8 @@ typedef struct {
     double inner_rtol;    /* largest relative residual reduction asked of one FP32 inner solve; the FP64
                              refinement plans ceil(log need / log inner_rtol) steps; default 1e-5 */
     int coarse_degree;    /* Chebyshev degree on the coarsest level when it has > 1 point; 0 = auto */
-    int block_points;     /* grid points per CTA of the level sweeps (CTA = points x 16-byte chunks); 0 = auto */
+    int block_points;     /* grid points per CTA of the level sweeps (CTA = points x 16-byte chunks; at least 4, in
+                             FP64 2); 0 = auto */
     int blocks_per_sm;    /* CTAs per SM of the grid-stride sweeps; 0 = auto */
     int coarse_kernel;    /* bura_coarse_kernel; default BURA_COARSE_AUTO */
     int cluster_size;     /* largest cluster tried for BURA_COARSE_CLUSTER: 2, 4, 8 or 16; 0 = 16.  The

@@ -330,7 +330,7 @@ Launch make_launch(int Kp, int W, long long N, int nsm, int block_points, int bl
     Launch g;
     g.Kp = Kp;
     g.C = Kp / W;
-    g.PPB = block_points > 0 ? block_points : (g.C <= 4 ? 64 : 32);
+    g.PPB = block_points > 0 ? std::max(block_points, W) : (g.C <= 4 ? 64 : 32);  // (a reduction takes a thread per system)
     if (g.PPB * g.C > kSweepThreads) g.PPB = kSweepThreads / g.C;
     long long tiles = (N + g.PPB - 1) / g.PPB;
     long long cap = (long long)nsm * (blocks_per_sm > 0 ? blocks_per_sm : 8);

@@ -41,3 +41,24 @@ def test_block_shapes(lib, k, points, per_sm):
         lib.bura_destroy(plan)
     ur = exact.bura_value(nps, f, e["c"], e["d"])
     assert np.linalg.norm(u.cpu().numpy() - ur) <= tol * np.linalg.norm(ur)
+
+
+@pytest.mark.parametrize("points", [1, 3])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_the_smallest_blocks(lib, points, precision):
+    """Blocks of fewer threads than systems, in which no thread would hold some system's total: they take a thread each."""
+    shape, k, tol = (31, 15), 7, 1e-6
+    nps = tuple(reversed(shape))
+    f = W.rhs_uniform(nps, 97)
+    e = tables.entry(0.5, k)
+    o = lib.bura_default_options()
+    o.precision, o.sweeps, o.block_points = precision, lib.BURA_SWEEP_GRID, points
+    plan = lib.bura_setup(shape, 0.5, k, options=o)
+    try:
+        u = torch.zeros(f.size, dtype=torch.float64, device="cuda")
+        assert lib.bura_solve(plan, torch.from_numpy(f).cuda(), u, tol) == lib.BURA_OK
+        torch.cuda.synchronize()
+    finally:
+        lib.bura_destroy(plan)
+    ur = exact.bura_value(nps, f, e["c"], e["d"])
+    assert np.linalg.norm(u.cpu().numpy() - ur) <= tol * np.linalg.norm(ur)
