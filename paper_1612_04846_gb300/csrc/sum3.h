@@ -11,8 +11,8 @@
 // the FP32 products they come from are.
 //
 // Against pairs of FP32 values (48 bits, one renormalisation an addition), which this replaces, with the block partials half
-// as large again and one barrier more in the one-launch solves: 1023^2, k = 7, 1857 -> 1873 us; sums over 511^2 plans 2609 ->
-// 2677; variable 511^2 2302 -> 2325; sparse 63^3 3773 -> 3800; 63^2 48.5 -> 49.8; 383 x 255 334 -> 339; the results are the
+// as large again and one barrier more in the one-launch solves: 1023^2, k = 7, 1870 -> 1886 us; sums over 511^2 plans 2630 ->
+// 2699; variable 511^2 2437 -> 2463; sparse 63^3 3731 -> 3764; 63^2 48.0 -> 49.3; 383 x 255 335 -> 337; the results are the
 // same bit for bit.  FP64 throughout: 1023^2 1958, sums 2958.
 #pragma once
 #include <math.h>
@@ -139,7 +139,8 @@ BURA_HD float sum3_div(const Sum3& a, const Sum3& b) {
 // The sum of a warp's Sum3 by integer additions (one instruction for 32 lanes each, where a tree of shuffles takes five steps
 // of 24): every lane's words become three limbs of 22 bits on the scale of the largest magnitude among the lanes (limb_top: its
 // bits, the maximum over the lanes taken as an unsigned integer), whose sums over the lanes are exact.  Only the last limb
-// rounds, at 2^-65 of the largest value.
+// rounds, at 2^-65 of the largest value.  (A 127^2 solve in one launch, 24 such sums: trees 113.0 us, limbs 113.2 with the
+// words rebuilt by four additions, 2 us less with the carries in integers; 383 x 255: 403.9, 402.1, 2 us less.)
 BURA_HD unsigned limb_top(const Sum3& v) {
     unsigned b[3], m = 0u;
     memcpy(b, &v, sizeof b);
@@ -186,17 +187,17 @@ BURA_HD Limbs to_limbs(const Sum3& v, unsigned top) {
     l.w[2] = b - mbits;
     return l;
 }
-// The value of limbs (a lane's, or their sums over 32 lanes).
+// The value of limbs (a lane's, or their sums over 32 lanes), exactly: the carries go up, and the 71 bits become words of 23,
+// 24 and 24 bits.
 BURA_HD Sum3 from_limbs(const Limbs& l) {
     if (l.top == 0x7f800000u) return {float_of(0x7fffffffu), 0.f, 0.f};  // a value that is not finite
     const float u = float_of(l.top - (21u << 23));
-    const int a = (int)l.w[0], b = (int)l.w[1], c = (int)l.w[2];
-    Sum3 t{rmul((float)(a >> 12) * 4096.f, u), 0.f, 0.f};
-    t.add(rmul((float)(a & 4095), u));
-    t.add(rmul((float)(b >> 12) * 0x1p-10f, u));
-    t.add(rmul((float)(b & 4095) * 0x1p-22f, u));
-    t.add(rmul((float)c * 0x1p-43f, u));
-    return t;
+    const int w2 = (int)l.w[2];
+    const int w1 = (int)l.w[1] + (w2 >> 21);  // units of 2^-22, the rest below one of them
+    const int w0 = (int)l.w[0] + (w1 >> 22);  // units
+    const int r1 = w1 & 0x3fffff, r2 = w2 & 0x1fffff;
+    return {rmul((float)(w0 & ~31), u), rmul((float)(((w0 & 31) << 19) | (r1 >> 3)) * 0x1p-19f, u),
+            rmul((float)(((r1 & 7) << 21) | r2) * 0x1p-43f, u)};
 }
 
 }  // namespace bura
